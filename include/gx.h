@@ -290,13 +290,16 @@ typedef struct {
 gx_status gx_network_set_schedule(gx_network* net, const gx_schedule* sched);
 gx_status gx_network_get_schedule(const gx_network* net, gx_schedule* sched);
 
-/* Cluster-resident solver (default off).  A scenario whose state fits the shared memory
- * of a thread-block cluster (1 to 16 CTAs; each CTA holds every device for a range of
- * hours, batteries exchange their hours over distributed shared memory) runs its whole
- * forward or adjoint loop in one persistent launch that tests its own convergence.
- * Other scenarios, and all of them while this is off, run on the per-iteration kernels.
- * The two paths take the same iterates up to the summation order of the residual
- * partials (so possibly a different stopping chunk). */
+/* Cluster-resident solver.  A scenario whose state fits the shared memory of a thread-block
+ * cluster (1 to 16 CTAs; each CTA holds every device for a range of hours, batteries exchange
+ * their hours over distributed shared memory) can run its forward or adjoint loop in a
+ * persistent launch that tests its own convergence.  on != 0: every such scenario does; 0: none,
+ * all run on the per-iteration kernels.  Until this is called the library decides, per loop and
+ * again as scenarios stop, by estimated time: scenarios go to clusters while all that are still
+ * iterating fit the device side by side; never after a call of gx_network_set_schedule or another
+ * launch mode than 2, nor while gx_profile_enable is on.  The two paths take bitwise the same
+ * iterates for horizons up to 192 hours (longer ones always run on the per-iteration kernels
+ * where they have batteries); only the residual partials are summed in another order. */
 gx_status gx_network_use_persistent(gx_network* net, int on);
 /* *cluster_ctas: CTAs of the cluster scenario `scen` runs on, 0 if it runs on the
  * per-iteration kernels (not resident, not launchable on this device, or switched off). */

@@ -15,6 +15,9 @@ using namespace gx;
 
 namespace {
 
+constexpr int kNoCluster = 1 << 16;  // weight in the active count of a scenario that fits no cluster
+constexpr int kCrsStreams = 8;  // launch groups of the resident path run side by side
+
 thread_local std::string g_err;
 
 gx_status fail(gx_status s, const std::string& msg) {
@@ -44,6 +47,7 @@ struct NetH {
     int gen0 = 0, line0 = 0, bat0 = 0, bus0 = 0, ptr0 = 0, eta0 = 0;
     std::vector<double> line_bref;  // reference capacity of a scaling susceptance (0: fixed beta)
     std::vector<int> l_scale;       // per line: its scaling index, -1 if beta is fixed
+    bool crs_ok = true;             // device counts of every bus fit the resident path's records
     std::vector<int> bus_sdres;     // per bus: its dual-residual record among the scaling ones, -1 if none
 };
 
@@ -95,17 +99,24 @@ struct gx_network {
     std::vector<double> sc_b, sc_bmin;
     std::vector<int2> sc_pool, sc_dres_l;
     std::vector<ScaleDres> sc_dres, sc_dres_pool;  // bus_dres_w targets; pool-word targets
-    // cluster-resident solver: scenarios grouped by (cluster size, hours per battery lane)
-    struct CrsGroup {
-        int C = 0, hpl = 0, first = 0, n = 0;
-        size_t smem = 0;
-        bool ok = false;  // launchable on this device (checked at bind)
+    // cluster-resident solver: the launch shapes a scenario can take, by (network, horizon)
+    struct CrsChoice {
+        CrsShape shape;
+        double us = 0;    // estimated time per iteration
+        double room = 0;  // share of the device one such cluster takes
     };
-    std::vector<CrsGroup> crs_groups;
-    std::vector<int> crs_list;         // scenario indices, group by group
-    std::vector<int> crs_group;        // per scenario: its group, -1 = per-iteration kernels only
+    std::map<std::pair<int, int>, std::vector<CrsChoice>> crs_choices;
+    int crs_clusters[kCrsMaxC + 1] = {};  // clusters of C whole-SM CTAs the device holds (set at bind)
+    std::vector<int4> crs_bus, crs_line;
+    CrsTables crs_tables{};            // their places in the workspace
+    std::vector<int2> crs_bat;
+    std::vector<int> crs_gen, crs_end, crs_cls, crs_rep;
     std::vector<int> done_loop;        // done flags of the per-iteration loop (cluster-resident ones set)
-    bool use_crs = false;
+    bool actw_set = false;             // the scenarios' weights in the active count are in the workspace
+    int thr_dev = -1;                  // what the loop graphs' pause threshold in the workspace holds
+    int use_crs = -1;                  // 1 on, 0 off, -1 not chosen: by rule (crs_active)
+    cudaStream_t crs_streams[kCrsStreams] = {};
+    cudaEvent_t crs_fork = nullptr, crs_join[kCrsStreams] = {};
     long long bus_el = 0, gen_el = 0, line_el = 0, bat_el = 0;
     int n_bus_blk = 0, n_line_blk = 0, n_bat_warps = 0, n_cost_blk = 0, n_gwarps = 0, gs_total = 0;
     int tot_gen = 0, tot_line = 0, tot_bat = 0, tot_bus = 0, tot_ptr = 0, tot_ramp = 0;
@@ -115,6 +126,8 @@ struct gx_network {
     int max_ramp_T = 1;
     // workspace offsets
     size_t o_scen, o_bbs, o_lbs, o_bws, o_cbs, o_gwarp, o_knet, o_busblk, o_pool, o_prep, o_crs;
+    size_t crs_begin, crs_end_off;
+    size_t o_crbus, o_crgen, o_crend, o_crline, o_crbat, o_crcls, o_crrep;
     size_t o_bus4blk, o_l4bs, o_l4blk, o_batw, o_buscpl, o_busdone;
     size_t o_scl, o_sce, o_scb, o_scbm, o_scp, o_scd, o_scdl, o_scgw;
     size_t o_rgen, o_rrate, o_gramp, o_rws, o_rdd, o_ardd, o_rf[4], o_ra[4], o_rpart;
@@ -125,7 +138,7 @@ struct gx_network {
     size_t o_f[16], o_a[16];  // forward / adjoint state arrays, order of StatePtrs
     size_t o_fend, o_aend;    // end of the forward / adjoint state range (ramp arrays included)
     size_t o_mgen, o_mload, o_mline, o_mbat, o_ag, o_al;
-    size_t o_done, o_iters, o_status, o_adjit, o_nact, o_ctr, o_inb, o_err, o_wsel, o_resid, o_rbest, o_cost, o_h, o_grads, o_wprime, o_obj, o_stlo, o_sthi, o_pact;
+    size_t o_done, o_iters, o_status, o_adjit, o_nact, o_thr, o_ctr, o_inb, o_err, o_wsel, o_resid, o_rbest, o_cost, o_h, o_grads, o_wprime, o_obj, o_stlo, o_sthi, o_pact;
     size_t o_flow, o_price, o_shed, o_bpart, o_lpart, o_btpart, o_cpart;
     Layout lay;
     // binding
@@ -145,7 +158,7 @@ struct gx_network {
     int graph_next = 0;
     cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    int* h_nact = nullptr;  // pinned host copies: [0] active-scenario count, [1] iteration counter
+    int* h_nact = nullptr;  // pinned: [0] active-scenario count, [1] iteration counter, [2] pause threshold
     int use_graphs = 2;     // 0 eager launches, 1 one graph per chunk, 2 the whole loop as one graph
     gx_schedule sched{1, 2};  // kernel schedule (gx_network_set_schedule)
     bool sched_set = false;   // the caller chose the schedule (else bind picks it by workspace size)
@@ -169,6 +182,11 @@ struct gx_network {
         if (cap_stream2) cudaStreamDestroy(cap_stream2);
         if (ev_fork) cudaEventDestroy(ev_fork);
         if (ev_join) cudaEventDestroy(ev_join);
+        if (crs_fork) cudaEventDestroy(crs_fork);
+        for (auto& e : crs_join)
+            if (e) cudaEventDestroy(e);
+        for (auto& q : crs_streams)
+            if (q) cudaStreamDestroy(q);
         if (h_nact) cudaFreeHost(h_nact);
     }
 };
@@ -335,6 +353,14 @@ static void make_ctx(gx_network* net) {
     c.bus_staged = net->sched.bus_staged;
     c.bus4_smem = (int)net->bus4_smem;
     c.bat_warps = net->sched.bat_warps;
+    CrsTables& t = net->crs_tables;
+    t.bus = reinterpret_cast<const int4*>(d + net->o_crbus);
+    t.gen = I(net->o_crgen);
+    t.end = I(net->o_crend);
+    t.line = reinterpret_cast<const int4*>(d + net->o_crline);
+    t.bat = reinterpret_cast<const int2*>(d + net->o_crbat);
+    t.bat_cls = I(net->o_crcls);
+    t.cls_rep = I(net->o_crrep);
     c.err = I(net->o_err);
     // the adjoint iteration: same arrays, its own penalties and battery pivots
     Ctx& a = net->actx;
@@ -355,15 +381,17 @@ static void make_ctx(gx_network* net) {
 
 namespace gx {
 // Condition of the device-side loop (a conditional WHILE node around one residual-check
-// chunk): run another chunk while a scenario is still iterating and the cap is not reached.
+// chunk): run another chunk while more than *pause scenarios are still iterating and the cap is
+// not reached (0: until all have stopped).
 // The reduction marks every scenario done once the counter reaches the cap, so the loop
 // ends after at most cap / chunk bodies.
-__global__ void k_loop_cond(const int* n_active, const int* iter_ctr, int max_it, cudaGraphConditionalHandle h) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) cudaGraphSetConditional(h, (*n_active > 0 && *iter_ctr < max_it) ? 1u : 0u);
+__global__ void k_loop_cond(const int* n_active, const int* iter_ctr, const int* pause, int max_it,
+                            cudaGraphConditionalHandle h) {
+    if (threadIdx.x == 0 && blockIdx.x == 0) cudaGraphSetConditional(h, (*n_active > *pause && *iter_ctr < max_it) ? 1u : 0u);
 }
 
-int launch_loop_cond(const Ctx& c, int max_it, cudaGraphConditionalHandle h, cudaStream_t st) {
-    k_loop_cond<<<1, 32, 0, st>>>(c.n_active, c.iter_ctr, max_it, h);
+int launch_loop_cond(const Ctx& c, const int* pause, int max_it, cudaGraphConditionalHandle h, cudaStream_t st) {
+    k_loop_cond<<<1, 32, 0, st>>>(c.n_active, c.iter_ctr, pause, max_it, h);
     return 1;
 }
 
@@ -486,50 +514,158 @@ static void derive_network(NetH& h, const gx_opts& o) {
     }
 }
 
-// Cluster-resident groups.  A scenario takes the smallest cluster (1, 2, 4, 8 or 16 CTAs)
-// whose per-CTA shared-memory image fits kCrsSmemBudget; scenarios that fit none run on
-// the per-iteration kernels.  Scenarios with the same cluster size and battery lane
-// width form one launch, sized for the largest image among them.
-constexpr size_t kCrsSmemBudget = 200 * 1024;
-
-static int crs_hpl_bucket(int T) {
-    const int h = (T + 31) / 32;
-    return h <= 1 ? 1 : h <= 2 ? 2 : h <= 3 ? 3 : h <= 6 ? 6 : 8;
+// Static tables of the cluster-resident path: buses sorted by device count (generators and line
+// ends, descending: the lanes of a warp then walk lists of equal length), and the devices
+// renumbered in that order, each bus's in the order of its incidence lists (the summation order
+// of the bus kernels).
+static void build_crs_tables(gx_network* net) {
+    for (NetH& h : net->nets) {
+        std::vector<int> ord(h.N), pos(h.N), gslot(h.G), eslot(2 * (size_t)h.L), bslot(h.B);
+        for (int n = 0; n < h.N; ++n) ord[n] = n;
+        auto weight = [&](int n) { return 2 * (h.gptr[n + 1] - h.gptr[n]) + (h.eptr[n + 1] - h.eptr[n]); };
+        std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return weight(a) > weight(b); });
+        int g = 0, e = 0, b = 0;
+        for (int k = 0; k < h.N; ++k) {
+            const int n = ord[k];
+            pos[n] = k;
+            if (h.gptr[n + 1] - h.gptr[n] > kCrsMaxEnds || h.eptr[n + 1] - h.eptr[n] > kCrsMaxEnds ||
+                h.bptr[n + 1] - h.bptr[n] > kCrsMaxBats)
+                h.crs_ok = false;
+            net->crs_bus.push_back(make_int4(g, e, b, n));
+            for (int q = h.gptr[n]; q < h.gptr[n + 1]; ++q, ++g) net->crs_gen.push_back(h.gidx[q]);
+            for (int q = h.eptr[n]; q < h.eptr[n + 1]; ++q, ++e) {
+                net->crs_end.push_back(h.eidx[q]);
+                eslot[h.eidx[q]] = e;
+            }
+            for (int q = h.bptr[n]; q < h.bptr[n + 1]; ++q, ++b) bslot[h.bidx[q]] = b;
+        }
+        for (int l = 0; l < h.L; ++l)
+            net->crs_line.push_back(make_int4(pos[h.line_from[l]], pos[h.line_to[l]], eslot[2 * l], eslot[2 * l + 1]));
+        std::map<std::pair<double, double>, int> cls;  // batteries of equal efficiencies share their pivots
+        const size_t rep0 = net->crs_rep.size();
+        net->crs_rep.resize(rep0 + h.B, 0);
+        for (int k = 0; k < h.B; ++k) {
+            net->crs_bat.push_back(make_int2(pos[h.bat_bus[k]], bslot[k]));
+            const auto it = cls.emplace(std::make_pair(h.bat_effc[k], h.bat_effd[k]), (int)cls.size());
+            if (it.second) net->crs_rep[rep0 + it.first->second] = k;
+            net->crs_cls.push_back(it.first->second);
+        }
+        for (ScenDev& sd : net->sdev)
+            if (&net->nets[sd.net] == &h) sd.n_dd = (int)cls.size();
+    }
 }
 
-static void build_crs_groups(gx_network* net) {
-    net->crs_groups.clear();
-    net->crs_list.clear();
-    net->crs_group.assign(net->S, -1);
-    std::map<std::pair<int, int>, std::vector<int>> by;
-    std::map<std::pair<int, int>, size_t> smem;
-    for (int s = 0; s < net->S; ++s) {
-        const ScenDev& sd = net->sdev[s];
-        if (sd.R > 0) continue;  // ramping generators: per-iteration kernels only
-        for (int C = 1; C <= kCrsMaxC; C *= 2) {
-            const int H = (sd.T + C - 1) / C, nbo = (sd.B + C - 1) / C;
-            const size_t bytes = crs_offsets(sd.N, sd.G, sd.L, sd.B, H, nbo, sd.T).total;
-            if (bytes <= kCrsSmemBudget) {
-                const auto key = std::make_pair(C, crs_hpl_bucket(sd.T));
-                by[key].push_back(s);
-                smem[key] = std::max(smem[key], bytes);
-                break;
+// Estimated microseconds of one resident iteration: a non-negative least-squares fit over 845
+// timed shapes of 17 networks (5 to 500 buses, 1 to 168 hours; 6 % rms): a fixed part, the
+// cluster exchange, the bus step's rounds and work, the device items per warp, the batteries'
+// rounds and work, and the barriers' cost per warp.
+static double crs_cost(const ScenDev& sd, const CrsShape& p) {
+    const int HQ = crs_hours(sd.T, p.C, p.V) / p.V, W = p.threads / 32;
+    const int nbo = (sd.B + p.C - 1) / p.C, groups = W / p.kw;
+    auto rounds = [](int items, int per) { return (double)((items + per - 1) / per); };
+    const double bus = 2.0 + (double)sd.G / sd.N + 3.0 * sd.L / sd.N;
+    const double dev = (2.5 * sd.L + sd.G + sd.N) * HQ / 32.0 / W;
+    const double sweep = 0.45 * p.hpl;
+    static const double k4[8] = {0.33, 0.44, 0.0793, 0.0061, 0.1234, 0.1744, 0.0525, 0.0122};
+    static const double k1[8] = {0.22, 0.44, 0.0684, 0.0023, 0.0996, 0.0929, 0.0448, 0.0127};
+    const double* k = p.V == 4 ? k4 : k1;
+    return k[0] + (p.C > 1 ? k[1] : 0.0) + k[2] * rounds(sd.N * HQ, p.threads) * bus + k[3] * sd.N * HQ / 32.0 * bus +
+           k[4] * dev + k[5] * rounds(nbo, groups) * (1.0 + sweep * (p.kw == 2 ? 1.4 : 1.0)) +
+           k[6] * nbo * p.kw * (1.0 + sweep) + k[7] * W;
+}
+
+// The launch shapes of a scenario on the resident path: per cluster size whose image fits the
+// SM's shared memory, the item width and block size of the least estimated time; cluster sizes
+// ascending, those that gain nothing over a smaller one left out.  Empty: the scenario runs on
+// the per-iteration kernels only.  Battery lanes are split as in the battery kernel (two warps
+// where the batch's longest horizon exceeds 96 hours).
+static const std::vector<gx_network::CrsChoice>& crs_choices(gx_network* net, int s) {
+    const ScenDev& sd = net->sdev[s];
+    const auto key = std::make_pair(sd.net, sd.T);
+    const auto it = net->crs_choices.find(key);
+    if (it != net->crs_choices.end()) return it->second;
+    std::vector<gx_network::CrsChoice>& out = net->crs_choices[key];
+    // ramping generators run on the per-iteration kernels; a bus's counts are 12 and 8 bits
+    if (sd.R > 0 || !net->nets[sd.net].crs_ok) return out;
+    for (int C = 1; C <= kCrsMaxC; ++C) {
+        gx_network::CrsChoice best;
+        if (net->crs_clusters[C] < 1) continue;
+        for (int V : {4, 1}) {
+            if (crs_hours(sd.T, C, V) * (C - 1) >= sd.T) continue;  // an empty rank
+            for (int threads : {128, 256, 384, 512, 640}) {
+                CrsShape p;
+                p.C = C; p.V = V; p.threads = threads;
+                p.kw = net->ctx.max_bat_T > 96 && sd.T > 32 ? 2 : 1;
+                p.hpl = (sd.T + 32 * p.kw - 1) / (32 * p.kw);
+                if (p.hpl > 3) continue;
+                const int HS = crs_hours(sd.T, C, V), nbo = (sd.B + C - 1) / C;
+                p.reg = p.kw == 2 && nbo * 64 <= threads;
+                for (int adj = 0; adj < 2; ++adj)
+                    for (int sm = p.reg ? 0 : 1; sm >= 0; --sm) {
+                        p.bat_smem[adj] = sm;
+                        p.smem[adj] = crs_offsets(sd.N, sd.G, sd.L, sd.B, HS, C, sd.T, std::min(sd.n_dd, nbo), adj, sm, threads, V, p.kw).total;
+                        if (p.smem[adj] <= kCrsSmemMax) break;
+                    }
+                const size_t image = std::max(p.smem[0], p.smem[1]);
+                if (image > kCrsSmemMax) continue;
+                gx_network::CrsChoice ch;
+                ch.shape = p;
+                ch.us = crs_cost(sd, p);
+                // CTAs that share an SM: its registers (96 per thread) and shared memory
+                const int per_sm = std::max(1, std::min<int>(kCrsMaxThreads / threads, (int)(kCrsSmemMax / (image + 1024))));
+                ch.room = 1.0 / ((double)net->crs_clusters[C] * per_sm);
+                if (!best.shape.C || ch.us < best.us) best = ch;
             }
         }
+        if (!best.shape.C || (!out.empty() && best.us > 0.97 * out.back().us)) continue;
+        bool ok = true;
+        for (int adj = 0; adj < 2 && ok; ++adj) ok = crs_prepare(adj, best.shape) == cudaSuccess;
+        cudaGetLastError();
+        if (ok) out.push_back(best);
     }
-    for (auto& kv : by) {
-        gx_network::CrsGroup g;
-        g.C = kv.first.first;
-        g.hpl = kv.first.second;
-        g.first = (int)net->crs_list.size();
-        g.n = (int)kv.second.size();
-        g.smem = smem[kv.first];
-        for (int s : kv.second) {
-            net->crs_group[s] = (int)net->crs_groups.size();
-            net->crs_list.push_back(s);
+    return out;
+}
+
+// Launch shapes for the scenarios `act`, all of which have choices: each starts from its
+// smallest cluster, then the slowest is enlarged while the device still holds all of them side by
+// side (scenarios of one size take one cluster size).  Returns the estimated time per iteration, that
+// of the slowest; *fits: whether the smallest clusters already fit side by side.
+static double crs_assign(gx_network* net, const std::vector<int>& act, std::vector<CrsShape>* shapes, bool* fits) {
+    const size_t n = act.size();
+    std::vector<const std::vector<gx_network::CrsChoice>*> ch(n);
+    std::vector<size_t> at(n, 0);
+    double room = 0;
+    bool one = true;
+    for (size_t i = 0; i < n; ++i) {
+        ch[i] = &crs_choices(net, act[i]);
+        one = one && ch[i] == ch[0];
+        room += (*ch[i])[0].room;
+    }
+    // clusters of mixed sizes leave gaps in the processing clusters that hold them
+    const double limit = one ? 1.0 + 1e-9 : 0.9;
+    *fits = room <= limit;
+    if (one) {
+        for (size_t k = 1; k < ch[0]->size(); ++k)
+            if ((double)n * (*ch[0])[k].room <= limit) std::fill(at.begin(), at.end(), k);
+    } else if (*fits) {
+        for (;;) {
+            size_t w = 0;
+            for (size_t i = 1; i < n; ++i)
+                if ((*ch[i])[at[i]].us > (*ch[w])[at[w]].us) w = i;
+            if (at[w] + 1 >= ch[w]->size()) break;
+            const double more = (*ch[w])[at[w] + 1].room - (*ch[w])[at[w]].room;
+            if (room + more > limit) break;
+            room += more;
+            ++at[w];
         }
-        net->crs_groups.push_back(g);
     }
+    double us = 0;
+    if (shapes) shapes->resize(n);
+    for (size_t i = 0; i < n; ++i) {
+        us = std::max(us, (*ch[i])[at[i]].us);
+        if (shapes) (*shapes)[i] = (*ch[i])[at[i]].shape;
+    }
+    return us;
 }
 
 // Bus-kernel block records and the pool records of the bus ranges they cover.  Blocks of
@@ -1006,7 +1142,7 @@ gx_status gx_network_create(const gx_network_desc* nets, int n_nets, const gx_sc
         }
     }
     net->sc_dres.insert(net->sc_dres.end(), net->sc_dres_pool.begin(), net->sc_dres_pool.end());
-    build_crs_groups(net);
+    build_crs_tables(net);
     net->k_net.resize(K);
     for (int k = 0; k < n_nets; ++k)
         for (int q = 0; q < net->nets[k].G + net->nets[k].L + net->nets[k].B; ++q) net->k_net[net->nets[k].eta0 + q] = k;
@@ -1027,7 +1163,7 @@ gx_status gx_network_create(const gx_network_desc* nets, int n_nets, const gx_sc
     net->o_busblk = L.add(sizeof(BusBlk) * std::max<size_t>(net->bus_blk.size(), 1));
     net->o_pool = L.add(I4((long long)net->pool.size()));
     net->o_prep = L.add(8 * std::max<size_t>(net->prep.size(), 1));
-    net->o_crs = L.add(I4((long long)net->crs_list.size()));
+    net->o_crs = L.add(I4(S));
     net->o_bus4blk = L.add(sizeof(BusBlk) * std::max<size_t>(net->bus4_blk.size(), 1));
     net->o_buscpl = L.add(I4(std::max<long long>((long long)net->bus_cpl.size(), 1)));
     net->o_busdone = L.add(I4(std::max<long long>((long long)net->bus4_blk.size(), 1)));
@@ -1073,7 +1209,7 @@ gx_status gx_network_create(const gx_network_desc* nets, int n_nets, const gx_sc
     net->o_ag = L.add(F4(eg));
     net->o_al = L.add(F4(eb));
     net->o_done = L.add(I4(S)); net->o_iters = L.add(I4(S)); net->o_status = L.add(I4(S)); net->o_adjit = L.add(I4(S));
-    net->o_nact = L.add(I4(1)); net->o_ctr = L.add(I4(1)); net->o_inb = L.add(I4(S)); net->o_err = L.add(I4(1));
+    net->o_thr = L.add(I4(1)); net->o_ctr = L.add(I4(1)); net->o_inb = L.add(I4(S)); net->o_err = L.add(I4(1));
     net->o_wsel = L.add(I4(S));
     net->o_resid = L.add(D8(2LL * S)); net->o_rbest = L.add(D8(S)); net->o_cost = L.add(D8(S)); net->o_h = L.add(D8(S));
     net->o_grads = L.add(D8(gs)); net->o_wprime = L.add(D8(S)); net->o_obj = L.add(D8(1));
@@ -1084,6 +1220,17 @@ gx_status gx_network_create(const gx_network_desc* nets, int n_nets, const gx_sc
     net->o_btpart = L.add(F4((long long)net->n_bat_warps * kDevPart));
     net->o_rpart = L.add(F4((long long)net->n_ramp_warps * kDevPart));
     net->o_cpart = L.add(D8(2LL * net->n_cost_blk));
+    net->o_nact = L.add(I4(1 + S));
+    // the resident path's tables, uploaded by a copy of their own
+    net->crs_begin = L.total;
+    net->o_crbus = L.add(16 * std::max<size_t>(net->crs_bus.size(), 1));
+    net->o_crgen = L.add(I4((long long)net->crs_gen.size()));
+    net->o_crend = L.add(I4((long long)net->crs_end.size()));
+    net->o_crline = L.add(16 * std::max<size_t>(net->crs_line.size(), 1));
+    net->o_crbat = L.add(8 * std::max<size_t>(net->crs_bat.size(), 1));
+    net->o_crcls = L.add(I4((long long)net->crs_cls.size()));
+    net->o_crrep = L.add(I4((long long)net->crs_rep.size()));
+    net->crs_end_off = L.total;
     net->in_batch.assign(S, 0);
     net->done_init.assign(S, 1);
     net->wprime.assign(S, 0.0);
@@ -1121,7 +1268,6 @@ gx_status gx_network_bind(gx_network* net, void* dev_mem, size_t bytes, void* st
     put(net->o_busblk, net->bus_blk.data(), sizeof(BusBlk) * net->bus_blk.size());
     put(net->o_pool, net->pool.data(), 4 * net->pool.size());
     put(net->o_prep, net->prep.data(), 8 * net->prep.size());
-    put(net->o_crs, net->crs_list.data(), 4 * net->crs_list.size());
     put(net->o_bus4blk, net->bus4_blk.data(), sizeof(BusBlk) * net->bus4_blk.size());
     put(net->o_buscpl, net->bus_cpl.data(), 4 * net->bus_cpl.size());
     put(net->o_l4bs, net->line4_blk_scen.data(), 4 * net->line4_blk_scen.size());
@@ -1183,9 +1329,19 @@ gx_status gx_network_bind(gx_network* net, void* dev_mem, size_t bytes, void* st
     }
     GX_CUDA(cudaMemcpyAsync(net->dev, h.data(), net->static_end, cudaMemcpyHostToDevice, st));
     GX_CUDA(cudaMemsetAsync(net->dev + net->static_end, 0, net->lay.total - net->static_end, st));
+    std::vector<uint8_t> t(net->crs_end_off - net->crs_begin, 0);
+    auto put_t = [&](size_t off, const void* src, size_t n) { if (n) std::memcpy(t.data() + (off - net->crs_begin), src, n); };
+    put_t(net->o_crbus, net->crs_bus.data(), 16 * net->crs_bus.size());
+    put_t(net->o_crgen, net->crs_gen.data(), 4 * net->crs_gen.size());
+    put_t(net->o_crend, net->crs_end.data(), 4 * net->crs_end.size());
+    put_t(net->o_crline, net->crs_line.data(), 16 * net->crs_line.size());
+    put_t(net->o_crbat, net->crs_bat.data(), 8 * net->crs_bat.size());
+    put_t(net->o_crcls, net->crs_cls.data(), 4 * net->crs_cls.size());
+    put_t(net->o_crrep, net->crs_rep.data(), 4 * net->crs_rep.size());
+    GX_CUDA(cudaMemcpyAsync(net->dev + net->crs_begin, t.data(), t.size(), cudaMemcpyHostToDevice, st));
     GX_CUDA(cudaStreamSynchronize(st));
     net->dd_dirty = false;
-    if (!net->h_nact) GX_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&net->h_nact), 2 * sizeof(int), cudaHostAllocDefault));
+    if (!net->h_nact) GX_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&net->h_nact), 4 * sizeof(int), cudaHostAllocDefault));
     if (!net->cap_stream) GX_CUDA(cudaStreamCreateWithFlags(&net->cap_stream, cudaStreamNonBlocking));
     if (!net->cap_stream2) GX_CUDA(cudaStreamCreateWithFlags(&net->cap_stream2, cudaStreamNonBlocking));
     if (!net->ev_fork) GX_CUDA(cudaEventCreateWithFlags(&net->ev_fork, cudaEventDisableTiming));
@@ -1204,13 +1360,17 @@ gx_status gx_network_bind(gx_network* net, void* dev_mem, size_t bytes, void* st
         if (!net->sched_set) net->sched.bus_staged = net->l2_resident ? 0 : 1;
     }
     make_ctx(net);
-    for (auto& g : net->crs_groups) {
-        g.ok = true;
-        for (int adj = 0; adj < 2 && g.ok; ++adj)
-            g.ok = crs_prepare(adj, g.hpl, kCrsSmemBudget) == cudaSuccess &&
-                   crs_max_clusters(adj, g.hpl, g.C, g.smem) >= 1;
-        cudaGetLastError();
+    // clusters of C CTAs, one per SM, that the device holds at once
+    net->crs_choices.clear();
+    net->thr_dev = 0;  // (the workspace starts zeroed)
+    net->actw_set = false;
+    CrsShape probe;
+    probe.threads = kCrsMaxThreads;
+    for (int C = 1; C <= kCrsMaxC; ++C) {
+        probe.C = C;
+        net->crs_clusters[C] = crs_prepare(0, probe) == cudaSuccess ? crs_max_clusters(0, probe, 200 * 1024) : 0;
     }
+    cudaGetLastError();
     net->solved = false;
     net->adj_ready = false;
     return GX_OK;
@@ -1397,7 +1557,7 @@ static gx_status loop_graph(gx_network* net, const Ctx& c, int adj, int every, i
     if (ce != cudaSuccess) return bail(ce, "cudaStreamBeginCaptureToGraph");
     int dummy = 0;
     gx_status e = enqueue_iters(net, c, adj, every, 0, every, true, true, net->cap_stream, &dummy, false);
-    if (!e) launch_loop_cond(c, max_it, h, net->cap_stream);
+    if (!e) launch_loop_cond(c, reinterpret_cast<const int*>(net->dev + net->o_thr), max_it, h, net->cap_stream);
     cudaGraph_t captured = nullptr;
     ce = cudaStreamEndCapture(net->cap_stream, &captured);
     if (e) { cudaGraphDestroy(graph); return e; }
@@ -1412,38 +1572,72 @@ static gx_status loop_graph(gx_network* net, const Ctx& c, int adj, int every, i
     return GX_OK;
 }
 
-static bool crs_on(const gx_network* net, int s) {
-    const int g = net->crs_group[s];
-    return net->use_crs && g >= 0 && net->crs_groups[g].ok;
+// Whether resident launches are in force.  Until gx_network_use_persistent chooses, they are
+// unless the caller asked for something of the per-iteration kernels (a launch mode, a kernel
+// schedule, their sampled timing) or a battery's horizon exceeds 192 hours, where the two paths
+// do not round alike.
+static bool crs_active(const gx_network* net) {
+    if (net->use_crs >= 0) return net->use_crs != 0;
+    return net->use_graphs == 2 && !net->sched_set && !net->prof && net->ctx.max_bat_T <= 192;
 }
 
-// Run the batch's cluster-resident scenarios (one persistent launch per group) and set
-// up the done flags of the per-iteration loop so that it skips them.  *n_stream: the
-// batch's scenarios left for that loop.
-static gx_status run_crs(gx_network* net, int adj, cudaStream_t st, int* launches, int* n_stream) {
+// Launch the resident loops of the scenarios `act` (one launch per group of equal shape, the
+// groups on streams of their own unless there is one).  it0 >= 0: iterations already run by all
+// of them, -1: by each what its iteration count says; pause_at: stop at the next residual check
+// once at most that many are still iterating (0: run all to their end).  What follows on `st`
+// waits for them (crs_wait).
+static gx_status crs_launch(gx_network* net, int adj, const std::vector<int>& act, const std::vector<CrsShape>& shapes, int it0,
+                            int pause_at, bool alone, cudaStream_t st, int* launches, int* used) {
     const Ctx& c = adj ? net->actx : net->ctx;
     const double tol = adj ? net->opts.adj_tol : net->opts.tol;
-    std::vector<int> want(net->crs_groups.size(), 0);
-    int ns = 0, nc = 0;
-    for (int s = 0; s < net->S; ++s) {
-        if (!net->in_batch[s]) continue;
-        if (crs_on(net, s)) { want[net->crs_group[s]] = 1; ++nc; }
-        else ++ns;
+    *used = 0;
+    struct Group { CrsShape shape; int first, n; };
+    std::vector<Group> groups;
+    std::vector<int> list;
+    // (largest clusters first: they need the most contiguous room)
+    typedef std::tuple<int, int, int, int, int, int, int, int> Key;
+    std::map<Key, std::vector<size_t>> by;
+    for (size_t i = 0; i < act.size(); ++i) {
+        const CrsShape& p = shapes[i];
+        by[Key(-p.C, p.V, p.threads, p.kw, p.hpl, p.reg, p.bat_smem[0], p.bat_smem[1])].push_back(i);
     }
-    *n_stream = ns;
-    if (nc == 0) return GX_OK;
-    const int* inb = reinterpret_cast<const int*>(net->dev + net->o_inb);
-    const int* list = reinterpret_cast<const int*>(net->dev + net->o_crs);
+    for (const auto& kv : by) {
+        Group g{shapes[kv.second[0]], (int)list.size(), (int)kv.second.size()};
+        for (size_t i : kv.second) {
+            for (int k = 0; k < 2; ++k) g.shape.smem[k] = std::max(g.shape.smem[k], shapes[i].smem[k]);
+            list.push_back(act[i]);
+        }
+        groups.push_back(g);
+    }
+    int* dlist = reinterpret_cast<int*>(net->dev + net->o_crs);
+    GX_CUDA(cudaMemcpyAsync(dlist, list.data(), 4 * list.size(), cudaMemcpyHostToDevice, st));
+    if (pause_at > 0) {
+        const int n = (int)act.size();
+        GX_CUDA(cudaMemcpyAsync(c.n_active, &n, sizeof(int), cudaMemcpyHostToDevice, st));
+    }
     if (net->prof) GX_CUDA(cudaEventRecord(net->ev[0], st));
     int nl = 0;
-    for (size_t k = 0; k < net->crs_groups.size(); ++k) {
-        const auto& g = net->crs_groups[k];
-        if (!want[k]) continue;
-        nl += launch_crs(c, adj, list + g.first, g.n, inb, g.C, g.hpl, g.smem, tol, st);
+    if (groups.size() == 1 && alone) {
+        nl += launch_crs(c, net->crs_tables, adj, dlist, groups[0].n, groups[0].shape, tol, it0, pause_at, st);
+    } else {
+        if (!net->crs_fork) GX_CUDA(cudaEventCreateWithFlags(&net->crs_fork, cudaEventDisableTiming));
+        GX_CUDA(cudaEventRecord(net->crs_fork, st));
+        const int ns = (int)std::min<size_t>(groups.size(), kCrsStreams);
+        for (int k = 0; k < ns; ++k) {
+            if (!net->crs_streams[k]) GX_CUDA(cudaStreamCreateWithFlags(&net->crs_streams[k], cudaStreamNonBlocking));
+            if (!net->crs_join[k]) GX_CUDA(cudaEventCreateWithFlags(&net->crs_join[k], cudaEventDisableTiming));
+            GX_CUDA(cudaStreamWaitEvent(net->crs_streams[k], net->crs_fork, 0));
+        }
+        for (size_t k = 0; k < groups.size(); ++k)
+            nl += launch_crs(c, net->crs_tables, adj, dlist + groups[k].first, groups[k].n, groups[k].shape, tol, it0, pause_at,
+                             net->crs_streams[k % ns]);
+        for (int k = 0; k < ns; ++k) GX_CUDA(cudaEventRecord(net->crs_join[k], net->crs_streams[k]));
+        *used = ns;
     }
     GX_CUDA(cudaGetLastError());
     *launches += nl;
     if (net->prof) {
+        for (int k = 0; k < *used; ++k) GX_CUDA(cudaStreamWaitEvent(st, net->crs_join[k], 0));
         GX_CUDA(cudaEventRecord(net->ev[1], st));
         GX_CUDA(cudaEventSynchronize(net->ev[1]));
         float ms = 0;
@@ -1452,11 +1646,11 @@ static gx_status run_crs(gx_network* net, int adj, cudaStream_t st, int* launche
         net->prof_samples[3] += nl;
         net->prof_launches[3] += nl;
     }
-    if (ns > 0) {
-        net->done_loop.assign(net->S, 1);
-        for (int s = 0; s < net->S; ++s) net->done_loop[s] = (net->in_batch[s] && !crs_on(net, s)) ? 0 : 1;
-        GX_CUDA(cudaMemcpyAsync(net->dev + net->o_done, net->done_loop.data(), 4 * net->S, cudaMemcpyHostToDevice, st));
-    }
+    return GX_OK;
+}
+
+static gx_status crs_wait(gx_network* net, int used, cudaStream_t st) {
+    for (int k = 0; k < used; ++k) GX_CUDA(cudaStreamWaitEvent(st, net->crs_join[k], 0));
     return GX_OK;
 }
 
@@ -1471,7 +1665,8 @@ static gx_status run_crs(gx_network* net, int adj, cudaStream_t st, int* launche
 // from graph-recorded events).
 static gx_status read_stamps(gx_network* net, int nchunks, cudaStream_t st);
 
-static gx_status run_loop(gx_network* net, int adj, cudaStream_t st, int* launches, int* iters_out, int it0 = 0) {
+static gx_status run_loop(gx_network* net, int adj, cudaStream_t st, int* launches, int* iters_out, int it0 = 0,
+                          int pause_at = 0) {
     const Ctx& c = adj ? net->actx : net->ctx;
     const int max_it = adj ? net->opts.adj_max_iter : net->opts.max_iter;
     const int every = net->opts.check_every;
@@ -1480,6 +1675,11 @@ static gx_status run_loop(gx_network* net, int adj, cudaStream_t st, int* launch
     GX_CUDA(cudaMemsetAsync(c.iter_ctr, 0, sizeof(int), st));
     if (it0 > 0) *launches += launch_tick(c, it0, st);
     if (net->use_graphs == 2 && max_it % every == 0) {
+        if (net->thr_dev != pause_at) {
+            net->h_nact[2] = pause_at;
+            GX_CUDA(cudaMemcpyAsync(net->dev + net->o_thr, net->h_nact + 2, sizeof(int), cudaMemcpyHostToDevice, st));
+            net->thr_dev = pause_at;
+        }
         cudaGraphExec_t exec = nullptr;
         if (gx_status e = loop_graph(net, c, adj, every, max_it, &exec)) return e;
         GX_CUDA(cudaGraphLaunch(exec, st));
@@ -1515,7 +1715,7 @@ static gx_status run_loop(gx_network* net, int adj, cudaStream_t st, int* launch
         ++nch;
         GX_CUDA(cudaGetLastError());
         GX_CUDA(cudaStreamSynchronize(st));
-        if (*net->h_nact == 0) break;
+        if (*net->h_nact <= pause_at) break;
     }
     *iters_out = it;
     if (net->prof) {
@@ -1525,6 +1725,120 @@ static gx_status run_loop(gx_network* net, int adj, cudaStream_t st, int* launch
         return read_stamps(net, nch, st);
     }
     return GX_OK;
+}
+
+// The scenarios of `act` whose done flag is still clear (synchronises).
+static gx_status still_active(gx_network* net, cudaStream_t st, std::vector<int>& act) {
+    std::vector<int> done(net->S);
+    GX_CUDA(cudaMemcpyAsync(done.data(), net->dev + net->o_done, 4 * (size_t)net->S, cudaMemcpyDeviceToHost, st));
+    GX_CUDA(cudaStreamSynchronize(st));
+    std::vector<int> left;
+    for (int s : act)
+        if (!done[s]) left.push_back(s);
+    act.swap(left);
+    return GX_OK;
+}
+
+// Estimated microseconds of one iteration of the per-iteration kernels with `act` iterating: three
+// dependent launches (10 to 11 us for one scenario of any size here), then 3.3 to 3.6 us per million
+// device-hours (100 buses, 168 h: 10.9 us for 2 scenarios, 15.4 for 16).
+static double stream_cost(const gx_network* net, const std::vector<int>& act) {
+    double dh = 0;
+    for (int s : act) dh += (double)net->sdev[s].T * (net->sdev[s].N + net->sdev[s].G + net->sdev[s].L + net->sdev[s].B);
+    return 10.0 + 3.5e-6 * dh;
+}
+
+// Iterate the batch's scenarios to their stops on whichever path is estimated faster for those
+// still iterating.  Both take bitwise the same iterates and test the same residuals at the same
+// iterations, so a change of path or of cluster size at a residual check changes no result:
+//  * while the scenarios do not fit the device's shared memory side by side, or one of them fits
+//    no cluster, the per-iteration kernels run them all, and pause once the rest fit;
+//  * once they fit and a resident iteration is estimated shorter, each runs in its cluster; as
+//    scenarios stop, the rest pause and take larger clusters where that is worth a tenth.
+static gx_status iterate(gx_network* net, int adj, cudaStream_t st, int* launches, int it0 = 0) {
+    int it = it0, used = 0;
+    if (!crs_active(net)) return run_loop(net, adj, st, launches, &it, it0);
+    const int max_it = adj ? net->opts.adj_max_iter : net->opts.max_iter;
+    std::vector<int> act;
+    for (int s = 0; s < net->S; ++s)
+        if (net->in_batch[s]) act.push_back(s);
+    if (it0 > 0) {
+        if (gx_status e = still_active(net, st, act)) return e;
+        if (act.empty() || it0 >= max_it) return GX_OK;
+    }
+    if (!net->actw_set) {
+        std::vector<int> w(net->S, 1);
+        for (int s = 0; s < net->S; ++s)
+            if (crs_choices(net, s).empty()) w[s] = kNoCluster;
+        GX_CUDA(cudaMemcpyAsync(net->dev + net->o_nact + sizeof(int), w.data(), 4 * (size_t)net->S, cudaMemcpyHostToDevice, st));
+        GX_CUDA(cudaStreamSynchronize(st));  // `w` is local
+        net->actw_set = true;
+    }
+    std::vector<CrsShape> shapes;
+    const bool asked = net->use_crs == 1;  // every scenario that fits a cluster runs in it
+    if (asked) {
+        std::vector<int> res;
+        for (int s : act)
+            if (!crs_choices(net, s).empty()) res.push_back(s);
+        const bool mixed = res.size() < act.size();
+        if (res.empty() || (mixed && it0 > 0)) return run_loop(net, adj, st, launches, &it, it0);
+        if (mixed) {  // the others on the per-iteration kernels beside them
+            net->done_loop.assign(net->S, 1);
+            for (int s : act)
+                if (crs_choices(net, s).empty()) net->done_loop[s] = 0;
+            GX_CUDA(cudaMemcpyAsync(net->dev + net->o_done, net->done_loop.data(), 4 * net->S, cudaMemcpyHostToDevice, st));
+            bool fits;
+            crs_assign(net, res, &shapes, &fits);
+            if (gx_status e = crs_launch(net, adj, res, shapes, it0, 0, false, st, launches, &used)) return e;
+            const gx_status le = run_loop(net, adj, st, launches, &it, it0);
+            if (gx_status e = crs_wait(net, used, st)) return e;
+            return le;
+        }
+    }
+    bool resident = false;
+    for (;;) {
+        const int n = (int)act.size();
+        int n_fit = 0;
+        for (int s : act) n_fit += !crs_choices(net, s).empty();
+        bool fits = false;
+        double us = 0;
+        if (n_fit == n) us = crs_assign(net, act, &shapes, &fits);
+        if (!resident && !asked && !(fits && us < 0.95 * stream_cost(net, act))) {
+            // Pause once no scenario without a cluster is left (they count kNoCluster each) and as
+            // many others as fit for certain: the most for which the largest ones fit.
+            std::vector<int> big;
+            for (int s : act)
+                if (!crs_choices(net, s).empty()) big.push_back(s);
+            std::sort(big.begin(), big.end(), [&](int a, int b) { return crs_choices(net, a)[0].room > crs_choices(net, b)[0].room; });
+            int pause_at = 0;
+            for (size_t k = std::min<size_t>(big.size(), (size_t)n - 1); k >= 1 && pause_at == 0; --k) {
+                big.resize(k);
+                bool f;
+                if (crs_assign(net, big, nullptr, &f) < 0.95 * stream_cost(net, big) && f) pause_at = (int)k;
+            }
+            if (gx_status e = run_loop(net, adj, st, launches, &it, it, pause_at)) return e;
+            if (pause_at == 0 || it >= max_it) return GX_OK;
+            if (gx_status e = still_active(net, st, act)) return e;
+            if (act.empty()) return GX_OK;
+            continue;
+        }
+        // the largest count of remaining scenarios at which larger clusters pay for the pause
+        // (estimated on the slowest of them, for whichever remain)
+        int pause_at = 0;
+        std::vector<int> big = act;
+        std::sort(big.begin(), big.end(), [&](int a, int b) { return crs_choices(net, a)[0].us > crs_choices(net, b)[0].us; });
+        for (int k = net->prof ? 0 : n - 1; k >= 1 && pause_at == 0; k = k > 8 ? k * 7 / 8 : k - 1) {
+            big.resize(k);
+            bool f;
+            if (crs_assign(net, big, nullptr, &f) < 0.9 * us && f) pause_at = k;
+        }
+        if (gx_status e = crs_launch(net, adj, act, shapes, resident ? -1 : it, pause_at, true, st, launches, &used)) return e;
+        if (gx_status e = crs_wait(net, used, st)) return e;
+        if (pause_at == 0) return GX_OK;
+        if (gx_status e = still_active(net, st, act)) return e;
+        if (act.empty()) return GX_OK;
+        resident = true;
+    }
 }
 
 // Sampled kernel timing: every residual-check chunk's last iteration writes, per kernel
@@ -1720,10 +2034,7 @@ gx_status gx_dispatch_solve_batch(gx_network* net, const float* eta_dev, const i
         launches += launch_bus(c, M_INIT, 0, 0, st);
     }
     c.warm = nullptr;
-    int it = 0, ns = 0;
-    if (gx_status e = run_crs(net, 0, st, &launches, &ns)) return e;
-    if (ns > 0)
-        if (gx_status e = run_loop(net, 0, st, &launches, &it, it0)) return e;
+    if (gx_status e = iterate(net, 0, st, &launches, it0)) return e;
     launches += launch_extract(c, reinterpret_cast<const int*>(net->dev + net->o_inb), st);
     launches += launch_objective(c, reinterpret_cast<const double*>(net->dev + net->o_wprime),
                                  reinterpret_cast<double*>(net->dev + net->o_obj), st);
@@ -1764,10 +2075,7 @@ gx_status gx_dispatch_grad_batch(gx_network* net, const float* eta_dev, int warm
             launches += launch_bus(ac, M_RESET, 1, 0, st);
         }
         launches += launch_bus(ac, M_INIT, 1, 0, st);
-        int it = 0, ns = 0;
-        if (gx_status e = run_crs(net, 1, st, &launches, &ns)) return e;
-        if (ns > 0)
-            if (gx_status e = run_loop(net, 1, st, &launches, &it)) return e;
+        if (gx_status e = iterate(net, 1, st, &launches)) return e;
         net->adj_ready = true;
     }
     const int* inb = reinterpret_cast<const int*>(net->dev + net->o_inb);
@@ -1832,14 +2140,24 @@ gx_status gx_network_attach_gnn(gx_network* net, gx_gnn* gnn) {
 
 gx_status gx_network_use_persistent(gx_network* net, int on) {
     if (!net) return fail(GX_ERR_INVALID_ARG, "net is NULL");
-    net->use_crs = on != 0;
+    net->use_crs = on != 0 ? 1 : 0;
     return GX_OK;
 }
 
 gx_status gx_network_persistent_info(const gx_network* net, int scen, int* cluster_ctas) {
     if (!net || !cluster_ctas) return fail(GX_ERR_INVALID_ARG, "NULL argument");
     if (scen < 0 || scen >= net->S) return fail(GX_ERR_INVALID_ARG, "scenario out of range");
-    *cluster_ctas = crs_on(net, scen) ? net->crs_groups[net->crs_group[scen]].C : 0;
+    *cluster_ctas = 0;
+    if (!net->dev || !crs_active(net)) return GX_OK;
+    gx_network* nn = const_cast<gx_network*>(net);  // (the shapes are worked out on first use)
+    std::vector<int> fit;
+    for (int s = 0; s < net->S; ++s)
+        if (!crs_choices(nn, s).empty()) fit.push_back(s);
+    std::vector<CrsShape> shapes;
+    bool fits;
+    if (!fit.empty()) crs_assign(nn, fit, &shapes, &fits);
+    for (size_t i = 0; i < fit.size(); ++i)
+        if (fit[i] == scen) *cluster_ctas = shapes[i].C;
     return GX_OK;
 }
 

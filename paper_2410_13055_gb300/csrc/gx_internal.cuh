@@ -77,23 +77,55 @@ constexpr int kStageMax = GX_STAGE_MAX_KB * 1024;
 #endif
 
 // Cluster-resident solver: one thread-block cluster of C CTAs per scenario, CTA r owning
-// hours [r*H, (r+1)*H) of every device (H = ceil(T / C)), its state in shared memory.
-constexpr int kCrsThreads = 256;
+// hours [r*H, (r+1)*H) of every device, its state in shared memory.
+constexpr int kCrsMaxThreads = 640;  // 20 warps of at most 96 registers
 constexpr int kCrsMaxC = 16;
-constexpr int kCrsRed = 10;  // residual partial sums per rank (9 used)
-constexpr int kCrsBatState = 7;  // per owned battery-hour: zc zd zs yc yd ys xb
+constexpr int kCrsRed = 10;          // residual partial sums per rank (9 used)
+constexpr size_t kCrsSmemMax = 227 * 1024;
+constexpr int kCrsMaxEnds = 4095;    // generators or line ends of one bus (12-bit counts)
+constexpr int kCrsMaxBats = 255;     // batteries of one bus (8-bit count)
+
+// How a scenario runs on the resident path.
+struct CrsShape {
+    int C = 0;        // CTAs of its cluster (0: it does not fit)
+    int V = 4;        // hours per thread item: 4 or 1
+    int threads = 0;
+    int kw = 1;       // warps per battery
+    int hpl = 1;      // hours per lane of a battery's warps
+    int reg = 0;      // battery state in its lanes' registers (two warps, one battery per group)
+    int bat_smem[2] = {0, 0};   // forward, adjoint: battery state in shared memory (else in its workspace rows)
+    size_t smem[2] = {0, 0};
+};
+
+// Static tables of the resident path, per network (concatenated over networks): buses sorted
+// by device count, and the devices renumbered so that a bus's are consecutive.
+struct CrsTables {
+    const int4* bus;     // by sorted position: first generator, line-end, battery slot; bus
+    const int* gen;      // generator of each slot
+    const int* end;      // line end (2 l + side) of each slot
+    const int4* line;    // sorted position of the from and to bus, slots of the from and to end
+    const int2* bat;     // sorted position of the battery's bus, its injection slot
+    const int* bat_cls;  // efficiency class (one row of pivots each) ...
+    const int* cls_rep;  // ... and a battery of each class
+};
+
+// Hours per CTA.
+__host__ __device__ inline int crs_hours(int T, int C, int V) { return ((T + C - 1) / C + V - 1) / V * V; }
+
+// Floats of a prox-target row: the horizon rounded up to a quad.
+__host__ __device__ inline int crs_row(int T) { return (T + 3) / 4 * 4; }
 
 // Byte offsets in a CTA's dynamic shared memory, identical on every rank of a cluster
 // (remote ranks are addressed at the same offsets).
 struct CrsOff {
-    size_t red, wred, flag;
-    size_t pbar, u, thb, xl, ld, aux;  // [N*H] bus-hours (aux: adjoint load gradient, NaN if fixed)
-    size_t xg, cap;                    // [G*H] (cap: forward capacity, adjoint cost gradient or NaN)
-    size_t dl, sg, vf, vt;             // [L*H]
-    size_t xb;                         // [B*H]
-    size_t lcap;                       // [L] flow limit as an angle, eta_l / beta_l
-    size_t bst;                        // [nbo][kCrsBatState][T] batteries owned by this rank
-    size_t lmask;                      // [L*H] bytes (adjoint)
+    size_t red, wred, xch, bar, flag, busr, busf, genr, endr, liner, linef, linec, bslot, batr, batg, idd, scan;
+    size_t pbar, u, thb, xl, ld;  // [N][HS] bus-hours (ld: load, or the adjoint coefficient, NaN if fixed)
+    size_t xg, cap;               // [G][HS] (cap: forward capacity, adjoint coefficient or NaN)
+    size_t dl, q;                 // [L][HS], [2L][HS] phase copies by end slot
+    size_t xb;                    // [B][HS]
+    size_t vrow;                  // [nbo][TR] owned batteries' prox targets (then their new injections)
+    size_t bst;                   // [nbo][6][T] owned batteries' state
+    size_t lmask;                 // [L][HS / V] bytes, one bit per hour (adjoint)
     size_t total;
 };
 
@@ -103,21 +135,33 @@ __host__ __device__ inline size_t crs_take(size_t& p, size_t bytes) {
     return r;
 }
 
-__host__ __device__ inline CrsOff crs_offsets(int N, int G, int L, int B, int H, int nbo, int T) {
+__host__ __device__ inline CrsOff crs_offsets(int N, int G, int L, int B, int HS, int C, int T, int dd_rows, int adj,
+                                              int bat_smem, int threads, int V, int kw) {
     CrsOff o{};
     size_t p = 0;
-    o.red = crs_take(p, sizeof(double) * kCrsMaxC * kCrsRed);
-    o.wred = crs_take(p, sizeof(float) * (kCrsThreads / 32) * kCrsRed);
+    const int nbo = (B + C - 1) / C;
+    o.red = crs_take(p, sizeof(double) * 2 * C * kCrsRed);
+    o.wred = crs_take(p, 4 * (size_t)(threads / 32) * kCrsRed);
+    o.xch = crs_take(p, 4 * 8 * (size_t)(threads / 32));
+    o.bar = crs_take(p, 16);
     o.flag = crs_take(p, 16);
-    const size_t nb = (size_t)N * H * 4, ng = (size_t)G * H * 4, nl = (size_t)L * H * 4;
+    o.busr = crs_take(p, 16 * (size_t)N); o.busf = crs_take(p, 16 * (size_t)N);
+    o.genr = crs_take(p, 8 * (size_t)G);
+    o.endr = crs_take(p, 32 * (size_t)L + 16);  // (and one entry read past an empty last list)
+    o.liner = crs_take(p, 16 * (size_t)L); o.linef = crs_take(p, 16 * (size_t)L); o.linec = crs_take(p, 16 * (size_t)L);
+    o.bslot = crs_take(p, 8 * (size_t)B);
+    o.batr = crs_take(p, 32 * (size_t)nbo); o.batg = crs_take(p, 8 * (size_t)nbo);
+    o.idd = crs_take(p, 4 * (size_t)dd_rows * T);
+    o.scan = crs_take(p, 4 * (size_t)dd_rows * 12 * 32 * kw);
+    const size_t nb = (size_t)N * HS * 4, ng = (size_t)G * HS * 4, nl = (size_t)L * HS * 4;
     o.pbar = crs_take(p, nb); o.u = crs_take(p, nb); o.thb = crs_take(p, nb);
-    o.xl = crs_take(p, nb); o.ld = crs_take(p, nb); o.aux = crs_take(p, nb);
+    o.xl = crs_take(p, nb); o.ld = crs_take(p, nb);
     o.xg = crs_take(p, ng); o.cap = crs_take(p, ng);
-    o.dl = crs_take(p, nl); o.sg = crs_take(p, nl); o.vf = crs_take(p, nl); o.vt = crs_take(p, nl);
-    o.xb = crs_take(p, (size_t)B * H * 4);
-    o.lcap = crs_take(p, (size_t)L * 4);
-    o.bst = crs_take(p, (size_t)nbo * kCrsBatState * T * 4);
-    o.lmask = crs_take(p, (size_t)L * H);
+    o.dl = crs_take(p, nl); o.q = crs_take(p, 2 * nl);
+    o.xb = crs_take(p, (size_t)B * HS * 4);
+    o.vrow = crs_take(p, 4 * (size_t)nbo * crs_row(T));
+    o.bst = crs_take(p, bat_smem ? (size_t)nbo * 6 * T * 4 : 0);
+    o.lmask = crs_take(p, adj ? (size_t)L * (HS / V) : 0);
     o.total = p;
     return o;
 }
@@ -174,6 +218,7 @@ struct ScenDev {
                                        // arrays, first warp of the ramp kernel
     long long e_ramp;                  // element offset of the scenario's ramp state rows
     int cost_blk0;                     // first block of the cost reduction
+    int n_dd;                          // distinct battery efficiency pairs of the network (pivot rows)
     float weight;
     double load_norm;                  // sqrt(sum load^2), >= 1e-30
 };
@@ -276,7 +321,8 @@ struct Ctx {
     int* iters;         // [S]
     int* status;        // [S]
     int* adj_iters;     // [S]
-    int* n_active;      // [1]
+    // [0] the scenarios still iterating, each with its weight, [1 + s] the weight of scenario s (0: 1)
+    int* n_active;
     double* resid;      // [S*2]
     double* rbest;      // [S] smallest max(primal, dual) residual of the current solve
     double* cost;       // [S]
@@ -404,13 +450,15 @@ int launch_prep(const Ctx& c, cudaStream_t st);
 // Allow the staged bus kernel `smem` bytes of dynamic shared memory (once per process is
 // enough; called at bind).
 cudaError_t bus_staged_prepare(int smem);
-int launch_loop_cond(const Ctx& c, int max_it, cudaGraphConditionalHandle h, cudaStream_t st);
-// Cluster-resident solver (gx_crs.cu): iterate the scenarios in `scen` (in_batch ones
-// only) to convergence, C CTAs per scenario, hpl hours per lane of a battery warp.
-cudaError_t crs_prepare(int adj, int hpl, size_t smem_max);
-int crs_max_clusters(int adj, int hpl, int C, size_t smem);
-int launch_crs(const Ctx& c, int adj, const int* scen, int n, const int* in_batch, int C, int hpl, size_t smem,
-               double tol, cudaStream_t st);
+int launch_loop_cond(const Ctx& c, const int* pause, int max_it, cudaGraphConditionalHandle h, cudaStream_t st);
+typedef void (*CrsFn)(Ctx, CrsTables, const int*, int, int, double, int, int);
+// Cluster-resident solver (gx_crs.cu): iterate the scenarios in `scen` to convergence, one cluster
+// each; it0 >= 0: iterations already run, -1: each scenario's own count; pause_at > 0: stop at the
+// next residual check once at most that many scenarios (counted down in n_active) are iterating.
+cudaError_t crs_prepare(int adj, const CrsShape& p);
+int crs_max_clusters(int adj, const CrsShape& p, size_t smem);
+int launch_crs(const Ctx& c, const CrsTables& tab, int adj, const int* scen, int n, const CrsShape& p, double tol, int it0, int pause_at,
+               cudaStream_t st);
 int launch_reduce(const Ctx& c, int adj, double tol, cudaStream_t st);
 int launch_tick(const Ctx& c, int chunk, cudaStream_t st);
 int launch_extract(const Ctx& c, const int* in_batch, cudaStream_t st);

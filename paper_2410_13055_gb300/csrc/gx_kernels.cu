@@ -1475,6 +1475,7 @@ __global__ void __launch_bounds__(kBlock) k_reduce(const Ctx c, int adj, double 
     if (c.prof_act != nullptr && threadIdx.x == 0) c.prof_act[s] += 1;
     const int it = *c.iter_ctr;
     const int final_ = it >= c.max_it;
+    const int weight = max(c.n_active[1 + s], 1);
     const ScenDev sc = c.scen[s];
     double a[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     for (int b = threadIdx.x; b < sc.bus4_nblk; b += kBlock) {
@@ -1542,7 +1543,7 @@ __global__ void __launch_bounds__(kBlock) k_reduce(const Ctx c, int adj, double 
             c.done[s] = 1;
             itp[s] = it;
         } else {
-            atomicAdd(c.n_active, 1);
+            atomicAdd(c.n_active, weight);
         }
     }
 }

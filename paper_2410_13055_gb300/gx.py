@@ -344,8 +344,9 @@ class Network:
         return {"bus_staged": sc.bus_staged, "bat_warps": sc.bat_warps}
 
     def use_persistent(self, on=True):
-        """Cluster-resident persistent launches for the scenarios that fit (default) or the
-        per-iteration kernels for every scenario."""
+        """Cluster-resident persistent launches for every scenario that fits, or the
+        per-iteration kernels for all of them; until this is called the library decides by
+        estimated time (gx_network_use_persistent)."""
         _check(_lib.gx_network_use_persistent(self._h, int(bool(on))), "gx_network_use_persistent", False)
 
     def persistent_info(self):
