@@ -56,53 +56,66 @@ __device__ __forceinline__ int scen_of_row(const ScenDev* sc, int S, long long r
 }
 
 // ---------------------------------------------------------------- features
-__global__ void k_features(const Ctx c, const float* __restrict__ eta, float* __restrict__ X,
-                           __nv_bfloat16* __restrict__ Xb, long long M) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= M) return;
-    const int s = scen_of_row(c.scen, c.S, i);
-    const ScenDev sc = c.scen[s];
-    const long long loc = i - sc.e_bus;
-    const int n = (int)(loc / sc.Tp), t = (int)(loc - (long long)n * sc.Tp);
-    float f[kFin];
+// One thread per hour quad of a bus (the bus kernels' blocks), so that the bus's device lists are
+// walked once for four rows and the capacity factors come 16 bytes at a time.
+__global__ void __launch_bounds__(kBusQBlock) k_features(const Ctx c, const float* __restrict__ eta,
+                                                         __nv_bfloat16* __restrict__ Xb) {
+    const BusBlk bb = c.bus4_blk[blockIdx.x];
+    const int local = bb.item0 + threadIdx.x;
+    if (local >= bb.nitems) return;
+    const ScenDev& sc = c.scen[bb.s];
+    const int Tq = bb.Tp >> 2;
+    const int n = local / Tq, t0 = (local - n * Tq) * 4;
+    const int nb = sc.ptr0 + n, gen0 = sc.gen0, eta0 = sc.eta0, eta_l = eta0 + sc.G, eta_b = eta_l + sc.L;
+    const long long row = bb.e_bus + (long long)n * bb.Tp + t0;
+    float avail[4] = {0.f, 0.f, 0.f, 0.f}, costw[4] = {0.f, 0.f, 0.f, 0.f}, freec[4] = {0.f, 0.f, 0.f, 0.f},
+          dear[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int q = c.bus_gptr[nb]; q < c.bus_gptr[nb + 1]; ++q) {
+        const int g = c.bus_gidx[gen0 + q];
+        const float4 cf = *reinterpret_cast<const float4*>(c.cf + bb.e_gen + (long long)g * bb.Tp + t0);
+        const float cv[4] = {cf.x, cf.y, cf.z, cf.w};
+        const float eg = fmaxf(eta[eta0 + g], 0.f), cost = c.g_cost[gen0 + g];
 #pragma unroll
-    for (int k = 0; k < kFin; ++k) f[k] = 0.f;
-    if (t < sc.T) {
-        const int nb = sc.ptr0 + n;
-        float avail = 0.f, costw = 0.f, freec = 0.f, dear = 0.f;
-        for (int q = c.bus_gptr[nb]; q < c.bus_gptr[nb + 1]; ++q) {
-            const int g = c.bus_gidx[sc.gen0 + q];
-            const float cap = c.cf[sc.e_gen + (long long)g * sc.Tp + t] * fmaxf(eta[sc.eta0 + g], 0.f);
-            const float cost = c.g_cost[sc.gen0 + g];
-            avail += cap;
-            if (cost == 0.f) freec += cap;
-            else { dear += cap; costw += cap * cost; }
+        for (int h = 0; h < 4; ++h) {
+            const float cap = cv[h] * eg;
+            avail[h] += cap;
+            if (cost == 0.f) freec[h] += cap;
+            else { dear[h] += cap; costw[h] += cap * cost; }
         }
-        float bat = 0.f;
-        for (int q = c.bus_bptr[nb]; q < c.bus_bptr[nb + 1]; ++q)
-            bat += fmaxf(eta[sc.eta0 + sc.G + sc.L + c.bus_bidx[sc.bat0 + q]], 0.f);
-        float lin = 0.f;
-        for (int q = c.bus_eptr[nb]; q < c.bus_eptr[nb + 1]; ++q)
-            lin += fmaxf(eta[sc.eta0 + sc.G + (c.bus_eidx[2 * sc.line0 + q] >> 1)], 0.f);
-        const float L = c.load[i];
-        const float h = (float)(t % 24);
-        f[0] = L * 0.01f;
-        f[1] = avail * 0.01f;
-        f[2] = dear > 0.f ? costw / dear * 0.01f : 0.f;
-        f[3] = freec * 0.01f;
-        f[4] = bat * 0.01f;
-        f[5] = lin * 0.01f;
-        f[6] = sinf(6.283185307179586f * h / 24.f);
-        f[7] = cosf(6.283185307179586f * h / 24.f);
-        f[8] = (L - freec) * 0.01f;
-        f[9] = 1.f;
     }
-    float4* o = reinterpret_cast<float4*>(X + i * kFin);
+    float bat = 0.f;
+    for (int q = c.bus_bptr[nb]; q < c.bus_bptr[nb + 1]; ++q) bat += fmaxf(eta[eta_b + c.bus_bidx[sc.bat0 + q]], 0.f);
+    float lin = 0.f;
+    for (int q = c.bus_eptr[nb]; q < c.bus_eptr[nb + 1]; ++q)
+        lin += fmaxf(eta[eta_l + (c.bus_eidx[2 * sc.line0 + q] >> 1)], 0.f);
+    const float4 L4 = *reinterpret_cast<const float4*>(c.load + row);
+    const float Lv[4] = {L4.x, L4.y, L4.z, L4.w};
 #pragma unroll
-    for (int k = 0; k < kFin / 4; ++k) o[k] = make_float4(f[4 * k], f[4 * k + 1], f[4 * k + 2], f[4 * k + 3]);
-    __nv_bfloat162* ob = reinterpret_cast<__nv_bfloat162*>(Xb + i * kFin);
+    for (int h = 0; h < 4; ++h) {
+        float f[kFin];
 #pragma unroll
-    for (int k = 0; k < kFin / 2; ++k) ob[k] = __floats2bfloat162_rn(f[2 * k], f[2 * k + 1]);
+        for (int k = 0; k < kFin; ++k) f[k] = 0.f;
+        if (t0 + h < bb.T) {
+            const float hr = (float)((t0 + h) % 24);
+            f[0] = Lv[h] * 0.01f;
+            f[1] = avail[h] * 0.01f;
+            f[2] = dear[h] > 0.f ? costw[h] / dear[h] * 0.01f : 0.f;
+            f[3] = freec[h] * 0.01f;
+            f[4] = bat * 0.01f;
+            f[5] = lin * 0.01f;
+            f[6] = sinf(6.283185307179586f * hr / 24.f);
+            f[7] = cosf(6.283185307179586f * hr / 24.f);
+            f[8] = (Lv[h] - freec[h]) * 0.01f;
+            f[9] = 1.f;
+        }
+        uint4 o[2];
+        __nv_bfloat162* ob = reinterpret_cast<__nv_bfloat162*>(o);
+#pragma unroll
+        for (int k = 0; k < kFin / 2; ++k) ob[k] = __floats2bfloat162_rn(f[2 * k], f[2 * k + 1]);
+        uint4* dst = reinterpret_cast<uint4*>(Xb + (row + h) * kFin);
+        dst[0] = o[0];
+        dst[1] = o[1];
+    }
 }
 
 // ---------------------------------------------------------------- dense layers
@@ -117,8 +130,11 @@ __global__ void k_features(const Ctx c, const float* __restrict__ eta, float* __
 //    thread t of the CTA owns row row0 + t in the epilogue.
 // Epilogues: kEpiFwd  Z = D + b;  H = relu(Z) (+ resid);  and a BF16 copy of H for the next
 //                     layer's operand;
-//            kEpiBwd  dH[:, 0:64] += D[:, 0:64];  dAgg = D[:, 64:128]   (D = dZ W^T).
-enum : int { kEpiFwd = 0, kEpiBwd = 1 };
+//            kEpiBwd  dH[:, 0:64] += D[:, 0:64];  dAgg = D[:, 64:128]   (D = dZ W^T);
+//            kEpiHead the last layer of a prediction: H as in kEpiFwd, of which only the output
+//                     layer y = H W_out + b_out leaves the CTA, as prices ($/MWh) and angles.
+// A prediction needs no Z (kept for the backward pass alone): o.Z is null there.
+enum : int { kEpiFwd = 0, kEpiBwd = 1, kEpiHead = 2 };
 
 struct DenseOut {
     const float* bias;
@@ -129,6 +145,8 @@ struct DenseOut {
     float* dH;
     float* dAgg;
     int* err;
+    const float* head;  // kEpiHead: W_out [64][2], b_out [2]; predictions, prices then angles
+    float* pred;
 };
 
 template <int NKB, int KW, int N>
@@ -215,6 +233,9 @@ __global__ void __launch_bounds__(128) k_dense(const __grid_constant__ CUtensorM
             // columns 4 (l % 8) .. +3 of rows 4 i + l / 8, i = 0..7.
             const uint32_t tq = tmem + ((uint32_t)(warp * 32) << 16);
             const int cq = lane & 7, rq = lane >> 3;
+            float y0[8], y1[8];  // kEpiHead: the lane's share of its rows' outputs
+#pragma unroll
+            for (int i = 0; i < 8; ++i) y0[i] = y1[i] = 0.f;
 #pragma unroll 1
             for (int c = 0; c < N / 32; ++c) {
                 float v[32];
@@ -225,20 +246,30 @@ __global__ void __launch_bounds__(128) k_dense(const __grid_constant__ CUtensorM
                 __syncwarp();
                 const int col = 32 * c + 4 * cq;
                 float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (EPI == kEpiFwd) b = *reinterpret_cast<const float4*>(o.bias + col);
+                if (EPI != kEpiBwd) b = *reinterpret_cast<const float4*>(o.bias + col);
+                float4 w0, w1;  // W_out of the lane's four columns
+                if (EPI == kEpiHead) {
+                    w0 = *reinterpret_cast<const float4*>(o.head + 2 * col);
+                    w1 = *reinterpret_cast<const float4*>(o.head + 2 * col + 4);
+                }
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const int lr = 4 * i + rq;
                     const long long r = row0 + warp * 32 + lr;
                     if (r >= M) continue;
                     const float4 d = *reinterpret_cast<const float4*>(sE + lr * Sh::EPITCH + 4 * cq);
-                    if (EPI == kEpiFwd) {
+                    if (EPI != kEpiBwd) {
                         const float4 z = make_float4(d.x + b.x, d.y + b.y, d.z + b.z, d.w + b.w);
-                        if (o.Z) *reinterpret_cast<float4*>(o.Z + r * N + col) = z;
+                        if (EPI == kEpiFwd && o.Z) *reinterpret_cast<float4*>(o.Z + r * N + col) = z;
                         float4 h = make_float4(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f), fmaxf(z.z, 0.f), fmaxf(z.w, 0.f));
                         if (o.resid) {
                             const float4 a = *reinterpret_cast<const float4*>(o.resid + r * N + col);
                             h.x += a.x; h.y += a.y; h.z += a.z; h.w += a.w;
+                        }
+                        if (EPI == kEpiHead) {
+                            y0[i] += h.x * w0.x + h.y * w0.z + h.z * w1.x + h.w * w1.z;
+                            y1[i] += h.x * w0.y + h.y * w0.w + h.z * w1.y + h.w * w1.w;
+                            continue;
                         }
                         *reinterpret_cast<float4*>(o.H + r * N + col) = h;
                         if (o.Hb) {
@@ -257,6 +288,21 @@ __global__ void __launch_bounds__(128) k_dense(const __grid_constant__ CUtensorM
                     }
                 }
                 __syncwarp();
+            }
+            if (EPI == kEpiHead) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+#pragma unroll
+                    for (int x = 1; x < 8; x <<= 1) {
+                        y0[i] += __shfl_xor_sync(0xffffffffu, y0[i], x);
+                        y1[i] += __shfl_xor_sync(0xffffffffu, y1[i], x);
+                    }
+                    const long long r = row0 + warp * 32 + 4 * i + rq;
+                    if (cq == 0 && r < M) {
+                        o.pred[r] = 100.f * (y0[i] + o.head[2 * kH]);
+                        o.pred[M + r] = y1[i] + o.head[2 * kH + 1];
+                    }
+                }
             }
         }
     }
@@ -375,61 +421,120 @@ __global__ void __launch_bounds__(128, 1) k_wgrad(const __grid_constant__ CUtens
     }
 }
 
-constexpr int kChunk = 256;  // rows per block of the bias-gradient column sums
+// ---------------------------------------------------------------- elementwise helpers
+__device__ __forceinline__ void store_bf16x4(__nv_bfloat16* p, const float4& v) {
+    __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+    *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+}
+__device__ __forceinline__ void relu_mask(float4& d, const float4& z) {
+    d.x = z.x > 0.f ? d.x : 0.f;
+    d.y = z.y > 0.f ? d.y : 0.f;
+    d.z = z.z > 0.f ? d.z : 0.f;
+    d.w = z.w > 0.f ? d.w : 0.f;
+}
+// A block's column sums (each thread's four columns from f on) into db: shared memory, then one
+// atomic per column.
+__device__ __forceinline__ void add_colsum(float* sh, const float4& v, int f, float* db) {
+    for (int i = threadIdx.x; i < kH; i += blockDim.x) sh[i] = 0.f;
+    __syncthreads();
+    float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        x[j] += __shfl_xor_sync(0xffffffffu, x[j], 16);
+        if ((threadIdx.x & 16) == 0) atomicAdd(&sh[f + j], x[j]);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kH; i += blockDim.x) atomicAdd(&db[i], sh[i]);
+}
 
-// column sums of dZ [M][N] into db[N] (FP32 atomics per block)
-template <int N>
-__global__ void k_colsum(const float* __restrict__ dZ, long long M, float* __restrict__ db) {
-    __shared__ float sh[N];
-    for (int i = threadIdx.x; i < N; i += blockDim.x) sh[i] = 0.f;
-    __syncthreads();
-    const long long r0 = (long long)blockIdx.x * kChunk;
-    for (long long r = r0 + threadIdx.x / N; r < r0 + kChunk && r < M; r += blockDim.x / N)
-        atomicAdd(&sh[threadIdx.x % N], dZ[r * N + threadIdx.x % N]);
-    __syncthreads();
-    for (int i = threadIdx.x; i < N; i += blockDim.x) atomicAdd(&db[i], sh[i]);
+// The top layer's dZ = dH * (Z > 0): its BF16 copy (the operand of dZ W^T and of the weight
+// gradient) and its column sums (the bias gradient, from the FP32 values); the layers below get
+// theirs from the transposed aggregation.  Streams dH and Z once, 16 bytes a load; dZ itself is
+// not stored.
+constexpr int kReluBlocks = 1216;
+__global__ void __launch_bounds__(256) k_relu_back(const float* __restrict__ dH, const float* __restrict__ Z,
+                                                   __nv_bfloat16* __restrict__ dZb, float* __restrict__ db, long long M) {
+    __shared__ float sh[kH];
+    const int f = 4 * (threadIdx.x & 15);
+    float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (long long r = (long long)blockIdx.x * 16 + (threadIdx.x >> 4); r < M; r += (long long)gridDim.x * 16) {
+        float4 d = *reinterpret_cast<const float4*>(dH + r * kH + f);
+        relu_mask(d, *reinterpret_cast<const float4*>(Z + r * kH + f));
+        store_bf16x4(dZb + r * kH + f, d);
+        cs.x += d.x; cs.y += d.y; cs.z += d.z; cs.w += d.w;
+    }
+    add_colsum(sh, cs, f, db);
 }
 
 // ---------------------------------------------------------------- aggregation
-// outb[i] = BF16 of the mean over neighbour buses m of in[(m, t)] (the next layer's operand;
-// also out[i] in FP32 when out is given), or (transpose) out[i] += sum over neighbours m of
-// in[(m, t)] / deg(m).  One warp per node, two features per lane.
+// outb[i] = BF16 of the mean over neighbour buses m of in[(m, t)] (the next layer's operand), or
+// (transpose) out[i] += sum over neighbours m of in[(m, t)] / deg(m).  A block takes the hour quads
+// of one bus-kernel block, a warp one quad (four consecutive rows of one bus) at a time, 16 lanes a
+// row: the bus's neighbour list is read once per quad, one neighbour per lane, and each neighbour
+// then costs a lane two independent 16-byte loads.  Bound by the gathers from L2 (three times the
+// array on a network with 1.5 lines per bus).  With one row per warp the scenario search, the list
+// walk and the gather were ten dependent loads per 256 bytes.
+// Transposed, the same pass finishes the layer below: with Z given, dZb = BF16 of
+// out * (Z > 0) and its column sums are added into db.
+constexpr int kAggWarps = 8;
 template <int TRANSPOSE>
-__global__ void k_agg(const Ctx c, const float* __restrict__ in, float* __restrict__ out,
-                      __nv_bfloat16* __restrict__ outb, long long M) {
-    const long long i = (long long)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-    if (i >= M) return;
-    const int lane = threadIdx.x & 31;
-    const int s = scen_of_row(c.scen, c.S, i);
-    const ScenDev sc = c.scen[s];
-    const long long loc = i - sc.e_bus;
-    const int n = (int)(loc / sc.Tp), t = (int)(loc - (long long)n * sc.Tp);
-    const int nb = sc.ptr0 + n;
-    const int e0 = c.bus_eptr[nb], e1 = c.bus_eptr[nb + 1];
-    float a0 = 0.f, a1 = 0.f;
-    for (int qq = e0; qq < e1; ++qq) {
-        const int e = c.bus_eidx[2 * sc.line0 + qq];
-        const int l = e >> 1;
-        const int m = (e & 1) ? c.l_from[sc.line0 + l] : c.l_to[sc.line0 + l];
-        const long long j = sc.e_bus + (long long)m * sc.Tp + t;
-        float w = 1.f;
-        if (TRANSPOSE) {
-            const int mb = sc.ptr0 + m;
-            w = 1.f / (float)(c.bus_eptr[mb + 1] - c.bus_eptr[mb]);
+__global__ void __launch_bounds__(32 * kAggWarps) k_agg(const Ctx c, const float* __restrict__ in, float* __restrict__ out,
+                                                        __nv_bfloat16* __restrict__ outb, const float* __restrict__ Z,
+                                                        float* __restrict__ db) {
+    __shared__ float sh[TRANSPOSE ? kH : 1];
+    const BusBlk bb = c.bus4_blk[blockIdx.x];
+    const int ptr0 = c.scen[bb.s].ptr0, line0 = c.scen[bb.s].line0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int sub = lane >> 4, f = 4 * (lane & 15);  // row of the pair, first of the lane's 4 features
+    const int Tq = bb.Tp >> 2;
+    float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = warp; k < kBusQBlock; k += kAggWarps) {
+        const int local = bb.item0 + k;
+        if (local >= bb.nitems) break;
+        const int n = local / Tq, t = (local - n * Tq) * 4;
+        const int e0 = c.bus_eptr[ptr0 + n], deg = c.bus_eptr[ptr0 + n + 1] - e0;
+        float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
+        for (int q0 = 0; q0 < deg; q0 += 32) {
+            const int cnt = min(32, deg - q0);
+            int m = 0;
+            float w = 1.f;
+            if (lane < cnt) {
+                const int e = c.bus_eidx[2 * line0 + e0 + q0 + lane], l = line0 + (e >> 1);
+                m = (e & 1) ? c.l_from[l] : c.l_to[l];
+                if (TRANSPOSE) w = 1.f / (float)(c.bus_eptr[ptr0 + m + 1] - c.bus_eptr[ptr0 + m]);
+            }
+#pragma unroll 4
+            for (int q = 0; q < cnt; ++q) {
+                const int mq = __shfl_sync(0xffffffffu, m, q);
+                const float wq = TRANSPOSE ? __shfl_sync(0xffffffffu, w, q) : 1.f;
+                const float* r = in + (bb.e_bus + (long long)mq * bb.Tp + t + sub) * kH + f;
+                const float4 x = *reinterpret_cast<const float4*>(r), y = *reinterpret_cast<const float4*>(r + 2 * kH);
+                a0.x += wq * x.x; a0.y += wq * x.y; a0.z += wq * x.z; a0.w += wq * x.w;
+                a1.x += wq * y.x; a1.y += wq * y.y; a1.z += wq * y.z; a1.w += wq * y.w;
+            }
         }
-        const float2 v = reinterpret_cast<const float2*>(in + j * kH)[lane];
-        a0 += w * v.x;
-        a1 += w * v.y;
+        const long long o0 = (bb.e_bus + (long long)n * bb.Tp + t + sub) * kH + f, o1 = o0 + 2 * kH;
+        if (!TRANSPOSE) {
+            const float w = deg > 0 ? 1.f / (float)deg : 0.f;
+            store_bf16x4(outb + o0, make_float4(a0.x * w, a0.y * w, a0.z * w, a0.w * w));
+            store_bf16x4(outb + o1, make_float4(a1.x * w, a1.y * w, a1.z * w, a1.w * w));
+        } else {
+            float4* p0 = reinterpret_cast<float4*>(out + o0);
+            float4* p1 = reinterpret_cast<float4*>(out + o1);
+            const float4 b0 = *p0, b1 = *p1;
+            const float4 z0 = *reinterpret_cast<const float4*>(Z + o0), z1 = *reinterpret_cast<const float4*>(Z + o1);
+            a0 = make_float4(b0.x + a0.x, b0.y + a0.y, b0.z + a0.z, b0.w + a0.w);
+            a1 = make_float4(b1.x + a1.x, b1.y + a1.y, b1.z + a1.z, b1.w + a1.w);
+            *p0 = a0;
+            *p1 = a1;
+            relu_mask(a0, z0);
+            relu_mask(a1, z1);
+            store_bf16x4(outb + o0, a0);
+            store_bf16x4(outb + o1, a1);
+            cs.x += a0.x + a1.x; cs.y += a0.y + a1.y; cs.z += a0.z + a1.z; cs.w += a0.w + a1.w;
+        }
     }
-    if (!TRANSPOSE) {
-        const float w = e1 > e0 ? 1.f / (float)(e1 - e0) : 0.f;
-        if (out) reinterpret_cast<float2*>(out + i * kH)[lane] = make_float2(a0 * w, a1 * w);
-        reinterpret_cast<__nv_bfloat162*>(outb + i * kH)[lane] = __floats2bfloat162_rn(a0 * w, a1 * w);
-    } else {
-        float2* o = reinterpret_cast<float2*>(out + i * kH) + lane;
-        const float2 prev = *o;
-        *o = make_float2(prev.x + a0, prev.y + a1);
-    }
+    if (TRANSPOSE) add_colsum(sh, cs, f, db);
 }
 
 // ---------------------------------------------------------------- head, loss, backward head
@@ -516,16 +621,6 @@ __global__ void __launch_bounds__(256) k_head_back(const float* __restrict__ H, 
     }
 }
 
-// dZ = dH * (Z > 0), and its BF16 copy (the operand of dZ W^T)
-__global__ void k_relu_back(const float* __restrict__ dH, const float* __restrict__ Z, float* __restrict__ dZ,
-                            __nv_bfloat16* __restrict__ dZb, long long n) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float d = Z[i] > 0.f ? dH[i] : 0.f;
-    dZ[i] = d;
-    dZb[i] = __float2bfloat16(d);
-}
-
 __global__ void k_adam(float* __restrict__ P, const float* __restrict__ G, float* __restrict__ m1,
                        float* __restrict__ m2, int n, float lr, float b1, float b2, float eps, float c1, float c2) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -562,14 +657,6 @@ __global__ void k_weight_images(const float* __restrict__ P, uint8_t* __restrict
     }
 }
 
-// predictions in the warm-start layout: prices ($/MWh) then angles (rad)
-__global__ void k_unpack(const float* __restrict__ Y, float* __restrict__ out, long long M) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= M) return;
-    out[i] = 100.f * Y[2 * i];
-    out[M + i] = Y[2 * i + 1];
-}
-
 }  // namespace
 }  // namespace gx
 
@@ -582,8 +669,8 @@ struct gx_gnn {
     size_t bytes = 0;
     uint8_t* dev = nullptr;
     // offsets
-    size_t o_P, o_G, o_m1, o_m2, o_img_in, o_img_fwd, o_img_bwd, o_X, o_Z0, o_Hs, o_Zs, o_Y, o_dY, o_dH,
-        o_dZ, o_dAgg, o_loss, o_err;
+    size_t o_P, o_G, o_m1, o_m2, o_img_in, o_img_fwd, o_img_bwd, o_Z0, o_Hs, o_Zs, o_Y, o_dY, o_dH,
+        o_dAgg, o_loss, o_err;
     // BF16 operands of the tensor-core layers: features, the inputs h_l and neighbour means
     // of each layer (kept for the weight gradients), dZ; and their TMA descriptors (128-row
     // boxes; the features also as a 64-column box for the weight gradient of W_in)
@@ -684,14 +771,12 @@ gx_status gx_gnn_create(const gx_network* net, int hidden, int layers, gx_gnn** 
     g->o_img_in = lay_add(t, kImgIn);
     g->o_img_fwd = lay_add(t, (size_t)kLayers * kImgLayer);
     g->o_img_bwd = lay_add(t, (size_t)kLayers * kImgLayer);
-    g->o_X = lay_add(t, 4 * (size_t)M * kFin);
     g->o_Z0 = lay_add(t, 4 * (size_t)M * kH);
     g->o_Hs = lay_add(t, 4 * (size_t)M * kH * (kLayers + 1));
     g->o_Zs = lay_add(t, 4 * (size_t)M * kH * kLayers);
     g->o_Y = lay_add(t, 4 * (size_t)M * 2);
     g->o_dY = lay_add(t, 4 * (size_t)M * 2);
     g->o_dH = lay_add(t, 4 * (size_t)M * kH);
-    g->o_dZ = lay_add(t, 4 * (size_t)M * kH);
     g->o_Xb = lay_add(t, 2 * (size_t)M * kFin);
     g->o_Hb = lay_add(t, 2 * (size_t)M * kH * kLayers);
     g->o_Agb = lay_add(t, 2 * (size_t)M * kH * kLayers);
@@ -774,6 +859,7 @@ gx_status gx_gnn_bind(gx_gnn* g, void* dev, size_t bytes, uint64_t seed, void* s
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, dev_id);
     if (e == cudaSuccess) e = dense_prepare<1, kFin, kH, kEpiFwd>();
     if (e == cudaSuccess) e = dense_prepare<2, kH, kH, kEpiFwd>();
+    if (e == cudaSuccess) e = dense_prepare<2, kH, kH, kEpiHead>();
     if (e == cudaSuccess) e = dense_prepare<1, kH, 2 * kH, kEpiBwd>();
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_wgrad<2 * kH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWSmem);
@@ -797,7 +883,10 @@ gx_status gx_gnn_bind(gx_gnn* g, void* dev, size_t bytes, uint64_t seed, void* s
 }
 
 // The network's forward pass; a tensor-core wait that runs out records GX_ERR_TIMEOUT in *err.
-static void gnn_forward(gx_gnn* g, const float* eta, cudaStream_t st, int* err) {
+// pred (nullable): a prediction alone, [prices | angles] over the bus rows: nothing is kept for a
+// backward pass, and the output layer runs in the last layer's epilogue.  Without it the outputs
+// go to the training step's Y.
+static void gnn_forward(gx_gnn* g, const float* eta, cudaStream_t st, int* err, float* pred) {
     const Ctx& c = *gx_internal_ctx(g->net);
     const long long M = g->M;
     auto F = [&](size_t o) { return reinterpret_cast<float*>(g->dev + o); };
@@ -805,29 +894,31 @@ static void gnn_forward(gx_gnn* g, const float* eta, cudaStream_t st, int* err) 
     float* P = F(g->o_P);
     auto Hb = [&](int l) { return Bf(g->o_Hb) + (size_t)l * M * kH; };
     auto Agb = [&](int l) { return Bf(g->o_Agb) + (size_t)l * M * kH; };
-    k_features<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(c, eta, F(g->o_X), Bf(g->o_Xb), M);
+    k_features<<<c.n_bus4_blk, kBusQBlock, 0, st>>>(c, eta, Bf(g->o_Xb));
     float* H0 = F(g->o_Hs);
-    DenseOut o{P + kOffBin, nullptr, F(g->o_Z0), H0, Hb(0), nullptr, nullptr, err};
+    DenseOut o{P + kOffBin, nullptr, pred ? nullptr : F(g->o_Z0), H0, Hb(0), nullptr, nullptr, err, nullptr, nullptr};
     dense_launch<1, kFin, kH, kEpiFwd>(g->maps[gx_gnn::kMapX], g->maps[gx_gnn::kMapX], g->dev + g->o_img_in, o, M,
                                         st);
     for (int l = 0; l < kLayers; ++l) {
         float* Hl = F(g->o_Hs) + (size_t)l * M * kH;
         float* Hn = F(g->o_Hs) + (size_t)(l + 1) * M * kH;
-        k_agg<0><<<(unsigned)((M + 7) / 8), 256, 0, st>>>(c, Hl, nullptr, Agb(l), M);
+        k_agg<0><<<c.n_bus4_blk, 32 * kAggWarps, 0, st>>>(c, Hl, nullptr, Agb(l), nullptr, nullptr);
         // H_{l+1} = H_l + relu([H_l, mean] W_l + b_l); its BF16 copy feeds the next layer
-        DenseOut ol{P + kOffL0 + l * kLayerSz + 2 * kH * kH, Hl, F(g->o_Zs) + (size_t)l * M * kH, Hn,
-                    l + 1 < kLayers ? Hb(l + 1) : nullptr, nullptr, nullptr, err};
-        dense_launch<2, kH, kH, kEpiFwd>(g->maps[gx_gnn::kMapH + l], g->maps[gx_gnn::kMapAg + l],
-                                          g->dev + g->o_img_fwd + (size_t)l * kImgLayer, ol, M, st);
+        const bool last = l + 1 == kLayers;
+        DenseOut ol{P + kOffL0 + l * kLayerSz + 2 * kH * kH, Hl, pred ? nullptr : F(g->o_Zs) + (size_t)l * M * kH, Hn,
+                    last ? nullptr : Hb(l + 1), nullptr, nullptr, err, P + kOffWout, pred};
+        const CUtensorMap &mh = g->maps[gx_gnn::kMapH + l], &ma = g->maps[gx_gnn::kMapAg + l];
+        const uint8_t* img = g->dev + g->o_img_fwd + (size_t)l * kImgLayer;
+        if (pred && last) dense_launch<2, kH, kH, kEpiHead>(mh, ma, img, ol, M, st);
+        else dense_launch<2, kH, kH, kEpiFwd>(mh, ma, img, ol, M, st);
     }
-    k_head<<<(unsigned)((M + 7) / 8), 256, 0, st>>>(F(g->o_Hs) + (size_t)kLayers * M * kH, P, F(g->o_Y), M);
+    if (!pred) k_head<<<(unsigned)((M + 7) / 8), 256, 0, st>>>(F(g->o_Hs) + (size_t)kLayers * M * kH, P, F(g->o_Y), M);
 }
 
 gx_status gx_gnn_predict(gx_gnn* g, const float* eta_dev, float* out_dev, void* stream) {
     if (!g || !g->dev || !eta_dev || !out_dev) return gx_internal_fail(GX_ERR_INVALID_ARG, "NULL argument or unbound");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    gnn_forward(g, eta_dev, st, reinterpret_cast<int*>(g->dev + g->o_err));
-    k_unpack<<<(unsigned)((g->M + 255) / 256), 256, 0, st>>>(reinterpret_cast<float*>(g->dev + g->o_Y), out_dev, g->M);
+    gnn_forward(g, eta_dev, st, reinterpret_cast<int*>(g->dev + g->o_err), out_dev);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return gx_internal_fail(GX_ERR_CUDA, std::string("gnn predict: ") + cudaGetErrorString(e));
     return GX_OK;
@@ -839,9 +930,8 @@ namespace gx {
 const gx_network* gx_gnn_internal_net(const gx_gnn* g) { return g ? g->net : nullptr; }
 gx_status gx_gnn_internal_predict(gx_gnn* g, const float* eta, cudaStream_t st, const float** pred) {
     if (!g || !g->dev) return gx_internal_fail(GX_ERR_STATE, "the attached warm-start network is not bound");
-    gnn_forward(g, eta, st, gx_internal_ctx(g->net)->err);  // reported with the solve's status
     float* out = reinterpret_cast<float*>(g->dev + g->o_pred);
-    k_unpack<<<(unsigned)((g->M + 255) / 256), 256, 0, st>>>(reinterpret_cast<float*>(g->dev + g->o_Y), out, g->M);
+    gnn_forward(g, eta, st, gx_internal_ctx(g->net)->err, out);  // reported with the solve's status
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return gx_internal_fail(GX_ERR_CUDA, std::string("gnn predict: ") + cudaGetErrorString(e));
     *pred = out;
@@ -866,7 +956,7 @@ gx_status gx_gnn_train_step(gx_gnn* g, const float* eta_dev, const float* target
     auto F = [&](size_t o) { return reinterpret_cast<float*>(g->dev + o); };
     int* err = reinterpret_cast<int*>(g->dev + g->o_err);
     __nv_bfloat16* dZb = reinterpret_cast<__nv_bfloat16*>(g->dev + g->o_dZb);
-    gnn_forward(g, eta_dev, st, err);
+    gnn_forward(g, eta_dev, st, err, nullptr);
     float* P = F(g->o_P);
     float* G = F(g->o_G);
     cudaMemsetAsync(G, 0, 4 * (size_t)kNParam, st);
@@ -876,31 +966,26 @@ gx_status gx_gnn_train_step(gx_gnn* g, const float* eta_dev, const float* target
     float* dH = F(g->o_dH);
     k_head_back<<<(unsigned)std::min<long long>((M + 7) / 8, kHeadBlocks), 256, 0, st>>>(
         F(g->o_Hs) + (size_t)kLayers * M * kH, F(g->o_dY), P, G, dH, M);
-    const unsigned ew = (unsigned)((M * kH + 255) / 256);
-    const unsigned nchunk = (unsigned)((M + kChunk - 1) / kChunk);
     // persistent weight-gradient CTAs: one per SM, none without a row tile
     const long long ntiles = (M + 127) / 128;
     const unsigned wg = (unsigned)std::min<long long>(ntiles, std::max(g->sms, 1));
     const CUtensorMap& mapdZ = g->maps[gx_gnn::kMapdZ];
+    auto bias = [&](int l) { return l < 0 ? G + kOffBin : G + kOffL0 + l * kLayerSz + 2 * kH * kH; };
+    auto Z = [&](int l) { return l < 0 ? F(g->o_Z0) : F(g->o_Zs) + (size_t)l * M * kH; };
+    k_relu_back<<<(unsigned)std::min<long long>((M + 15) / 16, kReluBlocks), 256, 0, st>>>(
+        dH, Z(kLayers - 1), dZb, bias(kLayers - 1), M);
     for (int l = kLayers - 1; l >= 0; --l) {
-        float* Zl = F(g->o_Zs) + (size_t)l * M * kH;
-        float* dZ = F(g->o_dZ);
-        k_relu_back<<<ew, 256, 0, st>>>(dH, Zl, dZ, dZb, M * kH);
-        float* GW = G + kOffL0 + l * kLayerSz;
-        k_wgrad<2 * kH><<<wg, 128, kWSmem, st>>>(g->maps[gx_gnn::kMapH + l], g->maps[gx_gnn::kMapAg + l], mapdZ, GW,
-                                                   M, err);
-        k_colsum<kH><<<nchunk, 256, 0, st>>>(dZ, M, GW + 2 * kH * kH);
+        k_wgrad<2 * kH><<<wg, 128, kWSmem, st>>>(g->maps[gx_gnn::kMapH + l], g->maps[gx_gnn::kMapAg + l], mapdZ,
+                                                   G + kOffL0 + l * kLayerSz, M, err);
         // [dH_direct, dAgg] = dZ W_l^T on the tensor cores; the residual keeps dH, the direct
-        // half is added into it, the neighbour half goes through the transposed aggregation
-        DenseOut ob{nullptr, nullptr, nullptr, nullptr, nullptr, dH, F(g->o_dAgg), err};
+        // half is added into it, the neighbour half goes through the transposed aggregation,
+        // which also leaves the layer below its dZ and bias gradient
+        DenseOut ob{nullptr, nullptr, nullptr, nullptr, nullptr, dH, F(g->o_dAgg), err, nullptr, nullptr};
         dense_launch<1, kH, 2 * kH, kEpiBwd>(mapdZ, mapdZ, g->dev + g->o_img_bwd + (size_t)l * kImgLayer, ob, M, st);
-        k_agg<1><<<(unsigned)((M + 7) / 8), 256, 0, st>>>(c, F(g->o_dAgg), dH, nullptr, M);
+        k_agg<1><<<c.n_bus4_blk, 32 * kAggWarps, 0, st>>>(c, F(g->o_dAgg), dH, dZb, Z(l - 1), bias(l - 1));
     }
-    float* dZ0 = F(g->o_dZ);
-    k_relu_back<<<ew, 256, 0, st>>>(dH, F(g->o_Z0), dZ0, dZb, M * kH);
     k_wgrad<kFin><<<wg, 128, kWSmem, st>>>(g->maps[gx_gnn::kMapXw], g->maps[gx_gnn::kMapXw], mapdZ, G + kOffWin, M,
                                              err);
-    k_colsum<kH><<<nchunk, 256, 0, st>>>(dZ0, M, G + kOffBin);
     if (lr > 0.f) {
         g->step += 1;
         const float b1 = 0.9f, b2 = 0.999f;
