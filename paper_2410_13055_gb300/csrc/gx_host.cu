@@ -156,8 +156,8 @@ struct gx_network {
         cudaGraphExec_t exec = nullptr;
     } graphs[4];
     int graph_next = 0;
-    cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr, cap_stream3 = nullptr;
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
     int* h_nact = nullptr;  // pinned: [0] active-scenario count, [1] iteration counter, [2] pause threshold
     int use_graphs = 2;     // 0 eager launches, 1 one graph per chunk, 2 the whole loop as one graph
     gx_schedule sched{1, 2};  // kernel schedule (gx_network_set_schedule)
@@ -180,8 +180,10 @@ struct gx_network {
         drop_graphs();
         if (cap_stream) cudaStreamDestroy(cap_stream);
         if (cap_stream2) cudaStreamDestroy(cap_stream2);
+        if (cap_stream3) cudaStreamDestroy(cap_stream3);
         if (ev_fork) cudaEventDestroy(ev_fork);
         if (ev_join) cudaEventDestroy(ev_join);
+        if (ev_join2) cudaEventDestroy(ev_join2);
         if (crs_fork) cudaEventDestroy(crs_fork);
         for (auto& e : crs_join)
             if (e) cudaEventDestroy(e);
@@ -1344,8 +1346,10 @@ gx_status gx_network_bind(gx_network* net, void* dev_mem, size_t bytes, void* st
     if (!net->h_nact) GX_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&net->h_nact), 4 * sizeof(int), cudaHostAllocDefault));
     if (!net->cap_stream) GX_CUDA(cudaStreamCreateWithFlags(&net->cap_stream, cudaStreamNonBlocking));
     if (!net->cap_stream2) GX_CUDA(cudaStreamCreateWithFlags(&net->cap_stream2, cudaStreamNonBlocking));
+    if (!net->cap_stream3) GX_CUDA(cudaStreamCreateWithFlags(&net->cap_stream3, cudaStreamNonBlocking));
     if (!net->ev_fork) GX_CUDA(cudaEventCreateWithFlags(&net->ev_fork, cudaEventDisableTiming));
     if (!net->ev_join) GX_CUDA(cudaEventCreateWithFlags(&net->ev_join, cudaEventDisableTiming));
+    if (!net->ev_join2) GX_CUDA(cudaEventCreateWithFlags(&net->ev_join2, cudaEventDisableTiming));
     if (net->bus4_smem > 0) GX_CUDA(bus_staged_prepare((int)net->bus4_smem));
     {
         int dev = 0, l2 = 0;
@@ -1462,8 +1466,9 @@ static gx_status enqueue_iters(gx_network* net, const Ctx& c, int adj, int chunk
     const int mode = adj ? M_ADJ : M_FWD;
     const double tol = adj ? net->opts.adj_tol : net->opts.tol;
     if (tick) *launches += launch_tick(c, chunk, st);
-    // While capturing, the line and battery proxes are two branches of the graph: they
-    // are independent and both feed the bus kernel.
+    // While capturing, the line, battery and ramp proxes are branches of the graph: they are
+    // independent and all feed the bus kernel.  (A ramp kernel behind the battery kernel on one
+    // branch made the iteration four dependent launches instead of three.)
     const bool fork = (st == net->cap_stream) && (c.n_bat_warps > 0 || c.n_ramp_warps > 0) && c.n_line_blk > 0;
     for (int j = j0; j < j1; ++j) {
         const int want = j == chunk - 1;
@@ -1471,11 +1476,19 @@ static gx_status enqueue_iters(gx_network* net, const Ctx& c, int adj, int chunk
         if (fork) {
             GX_CUDA(cudaEventRecord(net->ev_fork, st));
             GX_CUDA(cudaStreamWaitEvent(net->cap_stream2, net->ev_fork, 0));
+            const bool ramp_branch = c.n_ramp_warps > 0 && c.n_bat_warps > 0;
             nb = launch_bat(c, mode, adj, want, net->cap_stream2);
-            nb += launch_ramp(c, mode, adj, want, net->cap_stream2);
+            if (ramp_branch) {
+                GX_CUDA(cudaStreamWaitEvent(net->cap_stream3, net->ev_fork, 0));
+                nb += launch_ramp(c, mode, adj, want, net->cap_stream3);
+                GX_CUDA(cudaEventRecord(net->ev_join2, net->cap_stream3));
+            } else {
+                nb += launch_ramp(c, mode, adj, want, net->cap_stream2);
+            }
             GX_CUDA(cudaEventRecord(net->ev_join, net->cap_stream2));
             nl = launch_line(c, mode, adj, want, st);
             GX_CUDA(cudaStreamWaitEvent(st, net->ev_join, 0));
+            if (ramp_branch) GX_CUDA(cudaStreamWaitEvent(st, net->ev_join2, 0));
         } else {
             nl = launch_line(c, mode, adj, want, st);
             nb = launch_bat(c, mode, adj, want, st);
