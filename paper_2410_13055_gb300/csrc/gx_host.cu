@@ -1471,7 +1471,7 @@ static gx_status enqueue_iters(gx_network* net, const Ctx& c, int adj, int chunk
     // branch made the iteration four dependent launches instead of three.)
     const bool fork = (st == net->cap_stream) && (c.n_bat_warps > 0 || c.n_ramp_warps > 0) && c.n_line_blk > 0;
     for (int j = j0; j < j1; ++j) {
-        const int want = j == chunk - 1;
+        const int want = j == chunk - 1 ? kWantRes : j == chunk - 2 ? kWantSg : 0;
         int nl = 0, nb = 0;
         if (fork) {
             GX_CUDA(cudaEventRecord(net->ev_fork, st));

@@ -440,6 +440,8 @@ __device__ __forceinline__ void cost_share(const Ctx& c, const ScenDev& sc, long
     }
 }
 
+// want_res of an iteration's launches: the chunk's residual iteration, the one before it
+enum : int { kWantRes = 1, kWantSg = 2 };
 // Launch wrappers (gx_kernels.cu).  Each returns the number of kernels launched.
 int launch_dev(const Ctx& c, int mode, int adj, int want_res, cudaStream_t st);
 int launch_line(const Ctx& c, int mode, int adj, int want_res, cudaStream_t st);

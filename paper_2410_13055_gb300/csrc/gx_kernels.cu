@@ -782,6 +782,10 @@ __device__ __forceinline__ void ld4(const float* p, float (&v)[4]) {
 __device__ __forceinline__ void st4(float* p, const float (&v)[4]) {
     *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
 }
+// Operand orders of the fused multiply-adds are written out in the iteration kernels, so that every
+// instance, with or without the residual terms, takes the same iterates bit for bit.
+// (a x + b y with a x rounded, b y fused:)
+__device__ __forceinline__ float fma_second(float a, float x, float b, float y) { return __fmaf_rn(b, y, __fmul_rn(a, x)); }
 __device__ __forceinline__ void ldm4(const uint8_t* p, int (&v)[4]) {
     const uchar4 q = *reinterpret_cast<const uchar4*>(p);
     v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
@@ -791,10 +795,13 @@ __device__ __forceinline__ void ldm4(const uint8_t* p, int (&v)[4]) {
 #ifndef GX_LINE4_MINB
 #define GX_LINE4_MINB 1
 #endif
-template <int ADJ>
-__global__ void __launch_bounds__(kQBlock, GX_LINE4_MINB) k_line4(const Ctx c, int want_res) {
+// WANT: the residual iteration of a chunk.  sigma enters the residual alone, so the other
+// iterations neither read it nor write it, except the one before a residual (store_sg): 24
+// instead of 32 bytes per line-hour, and none of the residual's arithmetic.
+template <int ADJ, int WANT>
+__global__ void __launch_bounds__(kQBlock, GX_LINE4_MINB) k_line4(const Ctx c, int store_sg) {
     const int blk = blockIdx.x;
-    const bool stamp = want_res && c.stamp_lo != nullptr;
+    const bool stamp = WANT && c.stamp_lo != nullptr;
     if (stamp && threadIdx.x == 0) stamp_start(c, 1);
     // The block's offsets and its lines' end buses in one record (the ends staged in shared
     // memory); then the done flag, the line's state and its end buses' rows are read together,
@@ -814,7 +821,8 @@ __global__ void __launch_bounds__(kQBlock, GX_LINE4_MINB) k_line4(const Ctx c, i
         const long long row = lb.e_line + (long long)l * lb.Tp + t;
         const int lg = lb.line0 + l;
         float d[4], g[4], qf[4], qt[4], pbf[4], uf[4], zf[4], pbt[4], ut[4], zt[4];
-        ld4(X.dl + row, d); ld4(X.sg + row, g); ld4(X.vf + row, qf); ld4(X.vt + row, qt);
+        ld4(X.dl + row, d); ld4(X.vf + row, qf); ld4(X.vt + row, qt);
+        if (WANT) ld4(X.sg + row, g);
         const int end_f = lb.nends ? s_end[2 * (l - lb.l0)] : c.l_from[lg];
         const int end_t = lb.nends ? s_end[2 * (l - lb.l0) + 1] : c.l_to[lg];
         const long long bf = lb.e_bus + (long long)end_f * lb.Tp + t;
@@ -832,7 +840,8 @@ __global__ void __launch_bounds__(kQBlock, GX_LINE4_MINB) k_line4(const Ctx c, i
         const float rth = c.rth_c * w;
         const float capf = fmaxf(etal, 0.f) / beta;
         const float cap = fminf(capf, dthl);
-        const float den = 2.f * c.rho * beta * beta + 0.5f * rth + (dc ? c.eps : 0.f);
+        const float rb = __fmul_rn(c.rho, beta), hr = __fmul_rn(0.5f, rth);
+        const float den = __fadd_rn(__fmaf_rn(__fmul_rn(__fmul_rn(2.f, c.rho), beta), beta, hr), dc ? c.eps : 0.f);
         float fs[4] = {0.f, 0.f, 0.f, 0.f};  // adjoint of a transport line: eps f* of grad h
         if (ADJ && dc) ld4(c.dl + row, fs);
         float dn[4], gn[4], nf[4], nt[4];
@@ -841,25 +850,32 @@ __global__ void __launch_bounds__(kQBlock, GX_LINE4_MINB) k_line4(const Ctx c, i
             dn[h] = gn[h] = nf[h] = nt[h] = 0.f;
             if (t + h >= lb.T) continue;
             const float vf = qf[h] - zf[h], vt = qt[h] - zt[h];
-            const float ef = 0.5f * (g[h] + d[h]) - zf[h], et = 0.5f * (g[h] - d[h]) - zt[h];
-            if (!dc) th2 += beta * beta * (ef * ef + et * et);
+            if (WANT && !dc) {
+                const float ef = 0.5f * (g[h] + d[h]) - zf[h], et = 0.5f * (g[h] - d[h]) - zt[h];
+                th2 += beta * beta * (ef * ef + et * et);
+            }
             const float wf = zf[h] - vf, wt = zt[h] - vt;
-            const float tf = -beta * d[h] - pbf[h] - uf[h];
-            const float tt = beta * d[h] - pbt[h] - ut[h];
-            const float dun = (c.rho * beta * (tt - tf) + 0.5f * rth * (wf - wt) + c.eps * fs[h]) / den;
+            const float tf = __fsub_rn(__fmaf_rn(-beta, d[h], -pbf[h]), uf[h]);
+            const float tt = __fsub_rn(__fmaf_rn(beta, d[h], -pbt[h]), ut[h]);
+            float num = fma_second(rb, __fsub_rn(tt, tf), hr, __fsub_rn(wf, wt));
+            if (ADJ) num = __fmaf_rn(c.eps, fs[h], num);
+            const float dun = num / den;
             if (ADJ) dn[h] = mk[h] ? 0.f : dun;
             else dn[h] = clampf(dun, -cap, cap);
             gn[h] = wf + wt;
-            nf[h] = 0.5f * (gn[h] + dn[h]) + vf;
-            nt[h] = 0.5f * (gn[h] - dn[h]) + vt;
-            const float dd = dn[h] - d[h];
-            dx2 += 2.f * beta * beta * dd * dd;
-            x2 += 2.f * beta * beta * dn[h] * dn[h];
+            nf[h] = __fmaf_rn(0.5f, __fadd_rn(gn[h], dn[h]), vf);
+            nt[h] = __fmaf_rn(0.5f, __fsub_rn(gn[h], dn[h]), vt);
+            if (WANT) {
+                const float dd = dn[h] - d[h];
+                dx2 += 2.f * beta * beta * dd * dd;
+                x2 += 2.f * beta * beta * dn[h] * dn[h];
+            }
         }
-        st4(X.dl + row, dn); st4(X.sg + row, gn); st4(X.vf + row, nf); st4(X.vt + row, nt);
+        st4(X.dl + row, dn); st4(X.vf + row, nf); st4(X.vt + row, nt);
+        if (WANT || store_sg) st4(X.sg + row, gn);
     }
     if (done) return;  // the threads past the network's lines
-    if (want_res) {
+    if (WANT) {
         __shared__ float sh[3][kQBlock / 32];
         float v[3] = {dx2, x2, th2};
         block_sum<3, kQBlock>(v, sh);
@@ -894,10 +910,12 @@ __device__ __forceinline__ void gen_load4(const Ctx& c, const StatePtrs& X, cons
 // without them the flag test is compiled out.  At most 128 registers, so four blocks fit
 // an SM: uncapped, the adjoint instance took 136, three blocks per SM, and a 16-scenario
 // medium grid (3.45 blocks per SM) ran part of its blocks as a second wave.
-template <int ADJ, int RAMP>
-__global__ void __launch_bounds__(kBusQBlock, kBus4MinBlocks) k_bus4(const Ctx c, int want_res) {
+// WANT: the residual iteration of a chunk; the others read no old bus angle and carry none of
+// the residual's sums.
+template <int ADJ, int RAMP, int WANT>
+__global__ void __launch_bounds__(kBusQBlock, kBus4MinBlocks) k_bus4(const Ctx c) {
     __shared__ __align__(16) int S[kPoolMax];
-    const bool stamp = want_res && c.stamp_lo != nullptr;
+    const bool stamp = WANT && c.stamp_lo != nullptr;
     if (stamp && threadIdx.x == 0) stamp_start(c, 0);
     const BusBlk bb = c.bus4_blk[blockIdx.x];
     // The done flag, the record copy and this thread's bus state are all issued before the
@@ -913,7 +931,8 @@ __global__ void __launch_bounds__(kBusQBlock, kBus4MinBlocks) k_bus4(const Ctx c
     const long long i = bb.e_bus + (long long)n * bb.Tp + t;
     float pb[4], uu[4], thold[4], xl[4], Ld[4], al[4];
     if (valid) {
-        ld4(X.pbar + i, pb); ld4(X.u + i, uu); ld4(X.thb + i, thold);
+        ld4(X.pbar + i, pb); ld4(X.u + i, uu);
+        if (WANT) ld4(X.thb + i, thold);
         ld4(X.xl + i, xl);
         if (ADJ) ld4(c.al + i, al);  // the adjoint needs the load only through its coefficient
         else ld4(c.load + i, Ld);
@@ -971,7 +990,7 @@ __global__ void __launch_bounds__(kBusQBlock, kBus4MinBlocks) k_bus4(const Ctx c
 #pragma unroll
                 for (int h = 0; h < 4; ++h) {
                     sum[h] += x[h];
-                    x2 += x[h] * x[h];
+                    if (WANT) x2 += x[h] * x[h];
                 }
                 continue;
             }
@@ -983,17 +1002,19 @@ __global__ void __launch_bounds__(kBusQBlock, kBus4MinBlocks) k_bus4(const Ctx c
                 if (ADJ) {
                     const float gh = a[h];  // NaN: bound active, the variable is fixed at 0
                     const bool fixed = gh != gh;
-                    xn[h] = fixed ? 0.f : (rho * v + gh) * inv_re;
-                    if (!fixed && hv[h]) gscale += (gh * inv_re) * (gh * inv_re);
+                    xn[h] = fixed ? 0.f : __fmul_rn(__fmaf_rn(rho, v, gh), inv_re);
+                    if (WANT && !fixed && hv[h]) gscale += (gh * inv_re) * (gh * inv_re);
                 } else {
                     const float cap = a[h] * etag;
-                    const float pun = (rho * v - gcost) * inv_re;
+                    const float pun = __fmul_rn(__fmaf_rn(rho, v, -gcost), inv_re);
                     xn[h] = clampf(pun, 0.f, cap);
                 }
                 if (!hv[h]) xn[h] = 0.f;
                 sum[h] += xn[h];
-                dx2[h] += (xn[h] - x[h]) * (xn[h] - x[h]);
-                x2 += xn[h] * xn[h];
+                if (WANT) {
+                    dx2[h] += (xn[h] - x[h]) * (xn[h] - x[h]);
+                    x2 += xn[h] * xn[h];
+                }
             }
             st4(X.xg + r, xn);
         }
@@ -1005,16 +1026,18 @@ __global__ void __launch_bounds__(kBusQBlock, kBus4MinBlocks) k_bus4(const Ctx c
                 if (ADJ) {
                     const float gsh = al[h];  // NaN: bound active, the variable is fixed at 0
                     const bool fixed = gsh != gsh;
-                    xn[h] = fixed ? 0.f : (rho * v + gsh) * inv_re;
-                    if (!fixed && hv[h]) gscale += (gsh * inv_re) * (gsh * inv_re);
+                    xn[h] = fixed ? 0.f : __fmul_rn(__fmaf_rn(rho, v, gsh), inv_re);
+                    if (WANT && !fixed && hv[h]) gscale += (gsh * inv_re) * (gsh * inv_re);
                 } else {
-                    const float sun = (rho * (v + Ld[h]) - c.voll) * inv_re;
+                    const float sun = __fmul_rn(__fmaf_rn(rho, __fadd_rn(v, Ld[h]), -c.voll), inv_re);
                     xn[h] = clampf(sun, 0.f, Ld[h]) - Ld[h];
                 }
                 if (!hv[h]) xn[h] = 0.f;
                 sum[h] += xn[h];
-                dx2[h] += (xn[h] - xl[h]) * (xn[h] - xl[h]);
-                x2 += xn[h] * xn[h];
+                if (WANT) {
+                    dx2[h] += (xn[h] - xl[h]) * (xn[h] - xl[h]);
+                    x2 += xn[h] * xn[h];
+                }
             }
             st4(X.xl + i, xn);
         }
@@ -1024,7 +1047,7 @@ __global__ void __launch_bounds__(kBusQBlock, kBus4MinBlocks) k_bus4(const Ctx c
 #pragma unroll
                 for (int h = 0; h < 4; ++h) {
                     sum[h] += bx[k][h];
-                    x2 += bx[k][h] * bx[k][h];
+                    if (WANT) x2 += bx[k][h] * bx[k][h];
                 }
             }
         }
@@ -1034,7 +1057,7 @@ __global__ void __launch_bounds__(kBusQBlock, kBus4MinBlocks) k_bus4(const Ctx c
 #pragma unroll
             for (int h = 0; h < 4; ++h) {
                 sum[h] += xb[h];
-                x2 += xb[h] * xb[h];
+                if (WANT) x2 += xb[h] * xb[h];
             }
         }
         float ths[4] = {0.f, 0.f, 0.f, 0.f};
@@ -1046,10 +1069,10 @@ __global__ void __launch_bounds__(kBusQBlock, kBus4MinBlocks) k_bus4(const Ctx c
                 const float beta = P.atf(kPH_EBETA, q), w = P.atf(kPH_EW, q);
 #pragma unroll
                 for (int h = 0; h < 4; ++h) {
-                    const float p = (e & 1) ? beta * ed[k][h] : -beta * ed[k][h];
-                    sum[h] += p;
-                    x2 += p * p;
-                    ths[h] += w * eq[k][h];
+                    const float p = __fmul_rn((e & 1) ? beta : -beta, ed[k][h]);
+                    sum[h] = __fadd_rn(sum[h], p);
+                    if (WANT) x2 += p * p;
+                    ths[h] = __fmaf_rn(w, eq[k][h], ths[h]);
                 }
             }
         }
@@ -1062,10 +1085,10 @@ __global__ void __launch_bounds__(kBusQBlock, kBus4MinBlocks) k_bus4(const Ctx c
             const float beta = P.atf(kPH_EBETA, q), w = P.atf(kPH_EW, q);
 #pragma unroll
             for (int h = 0; h < 4; ++h) {
-                const float p = (e & 1) ? beta * d[h] : -beta * d[h];
-                sum[h] += p;
-                x2 += p * p;
-                ths[h] += w * qv[h];
+                const float p = __fmul_rn((e & 1) ? beta : -beta, d[h]);
+                sum[h] = __fadd_rn(sum[h], p);
+                if (WANT) x2 += p * p;
+                ths[h] = __fmaf_rn(w, qv[h], ths[h]);
             }
         }
         const float icnt = P.atf(kPH_IC, nl), iws = P.atf(kPH_IW, nl), drw = P.atf(kPH_DR, nl);
@@ -1073,10 +1096,10 @@ __global__ void __launch_bounds__(kBusQBlock, kBus4MinBlocks) k_bus4(const Ctx c
         float pbn[4], un[4], thn[4];
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
-            pbn[h] = sum[h] * icnt;
-            thn[h] = ths[h] * iws;
-            un[h] = uu[h] + pbn[h];
-            if (hv[h]) {
+            pbn[h] = __fmul_rn(sum[h], icnt);
+            thn[h] = __fmul_rn(ths[h], iws);
+            un[h] = __fadd_rn(uu[h], pbn[h]);
+            if (WANT && hv[h]) {
                 const float dpb = pbn[h] - pb[h];
                 acc[0] += cnt * pbn[h] * pbn[h];
                 acc[2] += dx2[h] - cnt * dpb * dpb;
@@ -1090,7 +1113,7 @@ __global__ void __launch_bounds__(kBusQBlock, kBus4MinBlocks) k_bus4(const Ctx c
         st4(X.u + i, un);
         st4(X.thb + i, thn);
     }
-    if (want_res) {
+    if (WANT) {
         __shared__ float sh[kBusPart][kBusQBlock / 32];
         block_sum<kBusPart, kBusQBlock>(acc, sh);
         if (threadIdx.x == 0) {
@@ -1153,11 +1176,11 @@ __device__ __forceinline__ bool bulk_wait(const Ctx& c, unsigned long long* bar)
 
 // LIST: the block's copy list and done flag come from its own slot (c.bus_cpl); compiled
 // apart so that the record-path instance keeps its registers.
-template <int ADJ, int RAMP, int LIST>
-__global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) k_bus4t(const Ctx c, int want_res) {
+template <int ADJ, int RAMP, int LIST, int WANT>
+__global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) k_bus4t(const Ctx c) {
     extern __shared__ __align__(16) int S[];  // the block's record, then its row stage
     __shared__ __align__(8) unsigned long long bar;
-    const bool stamp = want_res && c.stamp_lo != nullptr;
+    const bool stamp = WANT && c.stamp_lo != nullptr;
     if (stamp && threadIdx.x == 0) stamp_start(c, 0);
     const BusBlk bb = c.bus4_blk[blockIdx.x];
     const StatePtrs X = state<ADJ>(c);
@@ -1228,7 +1251,8 @@ __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) 
     // this thread's bus state, in flight together with the row copies
     float pb[4], uu[4], thold[4], xl[4], Ld[4], al[4];
     if (valid) {
-        ld4(X.pbar + i, pb); ld4(X.u + i, uu); ld4(X.thb + i, thold);
+        ld4(X.pbar + i, pb); ld4(X.u + i, uu);
+        if (WANT) ld4(X.thb + i, thold);
         ld4(X.xl + i, xl);
         if (ADJ) ld4(c.al + i, al);  // the adjoint needs the load only through its coefficient
         else ld4(c.load + i, Ld);
@@ -1309,7 +1333,7 @@ __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) 
 #pragma unroll
                 for (int h = 0; h < 4; ++h) {
                     sum[h] += x[h];
-                    x2 += x[h] * x[h];
+                    if (WANT) x2 += x[h] * x[h];
                 }
                 continue;
             }
@@ -1331,17 +1355,19 @@ __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) 
                 if (ADJ) {
                     const float gh = a[h];  // NaN: bound active, the variable is fixed at 0
                     const bool fixed = gh != gh;
-                    xn[h] = fixed ? 0.f : (rho * v + gh) * inv_re;
-                    if (!fixed && hv[h]) gscale += (gh * inv_re) * (gh * inv_re);
+                    xn[h] = fixed ? 0.f : __fmul_rn(__fmaf_rn(rho, v, gh), inv_re);
+                    if (WANT && !fixed && hv[h]) gscale += (gh * inv_re) * (gh * inv_re);
                 } else {
                     const float cap = a[h] * etag;
-                    const float pun = (rho * v - gcost) * inv_re;
+                    const float pun = __fmul_rn(__fmaf_rn(rho, v, -gcost), inv_re);
                     xn[h] = clampf(pun, 0.f, cap);
                 }
                 if (!hv[h]) xn[h] = 0.f;
                 sum[h] += xn[h];
-                dx2[h] += (xn[h] - x[h]) * (xn[h] - x[h]);
-                x2 += xn[h] * xn[h];
+                if (WANT) {
+                    dx2[h] += (xn[h] - x[h]) * (xn[h] - x[h]);
+                    x2 += xn[h] * xn[h];
+                }
             }
             st4(X.xg + r, xn);
         }
@@ -1353,16 +1379,18 @@ __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) 
                 if (ADJ) {
                     const float gsh = al[h];  // NaN: bound active, the variable is fixed at 0
                     const bool fixed = gsh != gsh;
-                    xn[h] = fixed ? 0.f : (rho * v + gsh) * inv_re;
-                    if (!fixed && hv[h]) gscale += (gsh * inv_re) * (gsh * inv_re);
+                    xn[h] = fixed ? 0.f : __fmul_rn(__fmaf_rn(rho, v, gsh), inv_re);
+                    if (WANT && !fixed && hv[h]) gscale += (gsh * inv_re) * (gsh * inv_re);
                 } else {
-                    const float sun = (rho * (v + Ld[h]) - c.voll) * inv_re;
+                    const float sun = __fmul_rn(__fmaf_rn(rho, __fadd_rn(v, Ld[h]), -c.voll), inv_re);
                     xn[h] = clampf(sun, 0.f, Ld[h]) - Ld[h];
                 }
                 if (!hv[h]) xn[h] = 0.f;
                 sum[h] += xn[h];
-                dx2[h] += (xn[h] - xl[h]) * (xn[h] - xl[h]);
-                x2 += xn[h] * xn[h];
+                if (WANT) {
+                    dx2[h] += (xn[h] - xl[h]) * (xn[h] - xl[h]);
+                    x2 += xn[h] * xn[h];
+                }
             }
             st4(X.xl + i, xn);
         }
@@ -1377,7 +1405,7 @@ __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) 
 #pragma unroll
             for (int h = 0; h < 4; ++h) {
                 sum[h] += xb[h];
-                x2 += xb[h] * xb[h];
+                if (WANT) x2 += xb[h] * xb[h];
             }
         }
         float ths[4] = {0.f, 0.f, 0.f, 0.f};
@@ -1397,10 +1425,10 @@ __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) 
             const float beta = P.atf(kPH_EBETA, q), w = P.atf(kPH_EW, q);
 #pragma unroll
             for (int h = 0; h < 4; ++h) {
-                const float pp = (e & 1) ? beta * d[h] : -beta * d[h];
-                sum[h] += pp;
-                x2 += pp * pp;
-                ths[h] += w * qv[h];
+                const float pp = __fmul_rn((e & 1) ? beta : -beta, d[h]);
+                sum[h] = __fadd_rn(sum[h], pp);
+                if (WANT) x2 += pp * pp;
+                ths[h] = __fmaf_rn(w, qv[h], ths[h]);
             }
         }
         const float icnt = P.atf(kPH_IC, nl), iws = P.atf(kPH_IW, nl), drw = P.atf(kPH_DR, nl);
@@ -1408,10 +1436,10 @@ __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) 
         float pbn[4], un[4], thn[4];
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
-            pbn[h] = sum[h] * icnt;
-            thn[h] = ths[h] * iws;
-            un[h] = uu[h] + pbn[h];
-            if (hv[h]) {
+            pbn[h] = __fmul_rn(sum[h], icnt);
+            thn[h] = __fmul_rn(ths[h], iws);
+            un[h] = __fadd_rn(uu[h], pbn[h]);
+            if (WANT && hv[h]) {
                 const float dpb = pbn[h] - pb[h];
                 acc[0] += cnt * pbn[h] * pbn[h];
                 acc[2] += dx2[h] - cnt * dpb * dpb;
@@ -1425,7 +1453,7 @@ __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) 
         st4(X.u + i, un);
         st4(X.thb + i, thn);
     }
-    if (want_res) {
+    if (WANT) {
         __shared__ float sh[kBusPart][kBusQBlock / 32];
         block_sum<kBusPart, kBusQBlock>(acc, sh);
         if (threadIdx.x == 0) {
@@ -1813,8 +1841,15 @@ __global__ void k_plan_step(float* eta, const float* grad, const float* gamma, c
 int launch_line(const Ctx& c, int mode, int adj, int want_res, cudaStream_t st) {
     if (mode == M_INIT || c.n_line_blk <= 0) return 0;
     if (mode == M_FWD || mode == M_ADJ) {
-        if (adj) k_line4<1><<<c.n_line4_blk, kQBlock, 0, st>>>(c, want_res);
-        else k_line4<0><<<c.n_line4_blk, kQBlock, 0, st>>>(c, want_res);
+        // want_res: kWantRes the residual iteration, kWantSg the one before it, 0 any other
+        const int sg = (want_res & kWantSg) != 0;
+        if (want_res & kWantRes) {
+            if (adj) k_line4<1, 1><<<c.n_line4_blk, kQBlock, 0, st>>>(c, 1);
+            else k_line4<0, 1><<<c.n_line4_blk, kQBlock, 0, st>>>(c, 1);
+        } else {
+            if (adj) k_line4<1, 0><<<c.n_line4_blk, kQBlock, 0, st>>>(c, sg);
+            else k_line4<0, 0><<<c.n_line4_blk, kQBlock, 0, st>>>(c, sg);
+        }
         return 1;
     }
     GX_DISPATCH_MODE_SETUP(k_line, c.n_line_blk, c, want_res);
@@ -1851,6 +1886,7 @@ int launch_line(const Ctx& c, int mode, int adj, int want_res, cudaStream_t st) 
 // warp per battery (hour-strided loops).
 int launch_bat(const Ctx& c, int mode, int adj, int want_res, cudaStream_t st) {
     if (mode == M_INIT || c.n_bat_warps <= 0) return 0;
+    want_res &= kWantRes;
     const int grid = (c.n_bat_warps + kBatWarps - 1) / kBatWarps;
     const int hpl = (c.max_bat_T + 31) / 32;
     if ((mode == M_FWD || mode == M_ADJ) && hpl > 3 && c.bat_warps == 2) {
@@ -1882,28 +1918,28 @@ int launch_bus(const Ctx& c, int mode, int adj, int want_res, cudaStream_t st) {
     if (c.n_bus_blk <= 0) return 0;
     if (mode == M_FWD || mode == M_ADJ) {
         const int sm = c.bus4_smem;
-        if (c.bus_staged != 0) {
-            const bool list = c.bus_staged == 1 && c.bus_cpl != nullptr;
-#define GX_BUS4T(A, R)                                                                  \
-    do {                                                                                \
-        if (list) k_bus4t<A, R, 1><<<c.n_bus4_blk, kBusQBlock, sm, st>>>(c, want_res);  \
-        else k_bus4t<A, R, 0><<<c.n_bus4_blk, kBusQBlock, sm, st>>>(c, want_res);       \
+        const bool want = (want_res & kWantRes) != 0, ramp = c.n_ramp_warps > 0;
+        const bool list = c.bus_staged == 1 && c.bus_cpl != nullptr;
+#define GX_BUS4W(A, R, W)                                                                      \
+    do {                                                                                       \
+        if (c.bus_staged == 0) k_bus4<A, R, W><<<c.n_bus4_blk, kBusQBlock, 0, st>>>(c);        \
+        else if (list) k_bus4t<A, R, 1, W><<<c.n_bus4_blk, kBusQBlock, sm, st>>>(c);           \
+        else k_bus4t<A, R, 0, W><<<c.n_bus4_blk, kBusQBlock, sm, st>>>(c);                     \
     } while (0)
-            if (c.n_ramp_warps > 0) {
-                if (adj) GX_BUS4T(1, 1);
-                else GX_BUS4T(0, 1);
-            } else {
-                if (adj) GX_BUS4T(1, 0);
-                else GX_BUS4T(0, 0);
-            }
-#undef GX_BUS4T
-        } else if (c.n_ramp_warps > 0) {
-            if (adj) k_bus4<1, 1><<<c.n_bus4_blk, kBusQBlock, 0, st>>>(c, want_res);
-            else k_bus4<0, 1><<<c.n_bus4_blk, kBusQBlock, 0, st>>>(c, want_res);
+#define GX_BUS4R(A, R)                  \
+    do {                                \
+        if (want) GX_BUS4W(A, R, 1);    \
+        else GX_BUS4W(A, R, 0);         \
+    } while (0)
+        if (ramp) {
+            if (adj) GX_BUS4R(1, 1);
+            else GX_BUS4R(0, 1);
         } else {
-            if (adj) k_bus4<1, 0><<<c.n_bus4_blk, kBusQBlock, 0, st>>>(c, want_res);
-            else k_bus4<0, 0><<<c.n_bus4_blk, kBusQBlock, 0, st>>>(c, want_res);
+            if (adj) GX_BUS4R(1, 0);
+            else GX_BUS4R(0, 0);
         }
+#undef GX_BUS4R
+#undef GX_BUS4W
         return 1;
     }
     GX_DISPATCH_MODE_SETUP(k_bus, c.n_bus_blk, c, want_res);
@@ -1915,14 +1951,16 @@ cudaError_t bus_staged_prepare(int smem) {
     auto set = [&](const void* f) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     };
-    set((const void*)k_bus4t<0, 0, 0>);
-    set((const void*)k_bus4t<1, 0, 0>);
-    set((const void*)k_bus4t<0, 1, 0>);
-    set((const void*)k_bus4t<1, 1, 0>);
-    set((const void*)k_bus4t<0, 0, 1>);
-    set((const void*)k_bus4t<1, 0, 1>);
-    set((const void*)k_bus4t<0, 1, 1>);
-    set((const void*)k_bus4t<1, 1, 1>);
+#define GX_BUS4S(A, R)                               \
+    set((const void*)k_bus4t<A, R, 0, 0>);           \
+    set((const void*)k_bus4t<A, R, 0, 1>);           \
+    set((const void*)k_bus4t<A, R, 1, 0>);           \
+    set((const void*)k_bus4t<A, R, 1, 1>)
+    GX_BUS4S(0, 0);
+    GX_BUS4S(1, 0);
+    GX_BUS4S(0, 1);
+    GX_BUS4S(1, 1);
+#undef GX_BUS4S
     return e;
 }
 

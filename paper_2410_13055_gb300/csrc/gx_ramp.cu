@@ -262,6 +262,7 @@ __global__ void __launch_bounds__(kBatWarps * 32) k_ramp(const Ctx c, int want_r
 // longest horizon among the scenarios with ramping generators.
 int launch_ramp(const Ctx& c, int mode, int adj, int want_res, cudaStream_t st) {
     if (mode == M_INIT || c.n_ramp_warps <= 0) return 0;
+    want_res &= kWantRes;
     const int grid = (c.n_ramp_warps + kBatWarps - 1) / kBatWarps;
     const int hpl = (c.max_ramp_T + 31) / 32;
     if (hpl <= 1) GX_RAMP_HPL(1);
