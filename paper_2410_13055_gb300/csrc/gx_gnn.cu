@@ -476,6 +476,7 @@ __global__ void __launch_bounds__(256) k_relu_back(const float* __restrict__ dH,
 // walk and the gather were ten dependent loads per 256 bytes.
 // Transposed, the same pass finishes the layer below: with Z given, dZb = BF16 of
 // out * (Z > 0) and its column sums are added into db.
+// A bus block's quads are split over gridDim.y CTAs (agg_grid).
 constexpr int kAggWarps = 8;
 template <int TRANSPOSE>
 __global__ void __launch_bounds__(32 * kAggWarps) k_agg(const Ctx c, const float* __restrict__ in, float* __restrict__ out,
@@ -488,7 +489,7 @@ __global__ void __launch_bounds__(32 * kAggWarps) k_agg(const Ctx c, const float
     const int sub = lane >> 4, f = 4 * (lane & 15);  // row of the pair, first of the lane's 4 features
     const int Tq = bb.Tp >> 2;
     float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int k = warp; k < kBusQBlock; k += kAggWarps) {
+    for (int k = warp + kAggWarps * blockIdx.y; k < kBusQBlock; k += kAggWarps * gridDim.y) {
         const int local = bb.item0 + k;
         if (local >= bb.nitems) break;
         const int n = local / Tq, t = (local - n * Tq) * 4;
@@ -730,6 +731,16 @@ static gx_status encode_rows(CUtensorMap* m, void* dev, long long rows, int cols
     return GX_OK;
 }
 
+// CTAs of an aggregation: the bus blocks, each split so that the device has 16 CTAs (128 warps) per
+// SM to draw from, down to one quad per warp.  A warp walks its quads one after the other, so with
+// few rows it is the walk that takes the time: the prediction of 51k rows (534 buses, 24 h, 4
+// scenarios) took 140 us with one CTA per block and takes 86, that of 269k rows 303 and 295.
+static dim3 agg_grid(const gx_gnn* g) {
+    const int blocks = std::max(gx_internal_ctx(g->net)->n_bus4_blk, 1);
+    const int want = (16 * std::max(g->sms, 1) + blocks - 1) / blocks;
+    return dim3((unsigned)blocks, (unsigned)std::min(kBusQBlock / kAggWarps, std::max(1, want)));
+}
+
 template <int NKB, int KW, int N, int EPI>
 static cudaError_t dense_prepare() {
     return cudaFuncSetAttribute(k_dense<NKB, KW, N, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -902,7 +913,7 @@ static void gnn_forward(gx_gnn* g, const float* eta, cudaStream_t st, int* err, 
     for (int l = 0; l < kLayers; ++l) {
         float* Hl = F(g->o_Hs) + (size_t)l * M * kH;
         float* Hn = F(g->o_Hs) + (size_t)(l + 1) * M * kH;
-        k_agg<0><<<c.n_bus4_blk, 32 * kAggWarps, 0, st>>>(c, Hl, nullptr, Agb(l), nullptr, nullptr);
+        k_agg<0><<<agg_grid(g), 32 * kAggWarps, 0, st>>>(c, Hl, nullptr, Agb(l), nullptr, nullptr);
         // H_{l+1} = H_l + relu([H_l, mean] W_l + b_l); its BF16 copy feeds the next layer
         const bool last = l + 1 == kLayers;
         DenseOut ol{P + kOffL0 + l * kLayerSz + 2 * kH * kH, Hl, pred ? nullptr : F(g->o_Zs) + (size_t)l * M * kH, Hn,
@@ -982,7 +993,7 @@ gx_status gx_gnn_train_step(gx_gnn* g, const float* eta_dev, const float* target
         // which also leaves the layer below its dZ and bias gradient
         DenseOut ob{nullptr, nullptr, nullptr, nullptr, nullptr, dH, F(g->o_dAgg), err, nullptr, nullptr};
         dense_launch<1, kH, 2 * kH, kEpiBwd>(mapdZ, mapdZ, g->dev + g->o_img_bwd + (size_t)l * kImgLayer, ob, M, st);
-        k_agg<1><<<c.n_bus4_blk, 32 * kAggWarps, 0, st>>>(c, F(g->o_dAgg), dH, dZb, Z(l - 1), bias(l - 1));
+        k_agg<1><<<agg_grid(g), 32 * kAggWarps, 0, st>>>(c, F(g->o_dAgg), dH, dZb, Z(l - 1), bias(l - 1));
     }
     k_wgrad<kFin><<<wg, 128, kWSmem, st>>>(g->maps[gx_gnn::kMapXw], g->maps[gx_gnn::kMapXw], mapdZ, G + kOffWin, M,
                                              err);
