@@ -271,11 +271,12 @@ gx_status gx_network_use_graphs(gx_network* net, int on);
 
 /* Kernel schedule of the per-iteration path (not in the paper; performance only: every
  * schedule computes the same iterates, bitwise).
- *   bus_staged  how the hour-quad bus kernel reads its block's device rows.  1: bulk
- *               copies (TMA) of every row segment into shared memory, completing on an
- *               mbarrier, so all of the block's rows are in flight at once; 2: the same
- *               stage filled by per-thread 16-byte asynchronous copies; 0: each thread
- *               loads its bus's device rows itself, one generator ahead.  Until a schedule
+ *   bus_staged  how the hour-quad bus kernel reads its block's device rows.  1: where the
+ *               workspace fits the device's L2 cache, bulk copies (TMA) of every row segment into
+ *               shared memory, completing on an mbarrier, so all of the block's rows are in
+ *               flight at once; in larger workspaces as 2.  2: a ring of per-thread 16-byte
+ *               asynchronous copies, the next four devices of a thread's bus in flight.  0: each
+ *               thread loads its bus's device rows itself, one generator ahead.  Until a schedule
  *               is set, bind picks 1 when the workspace exceeds the device's L2 cache (the
  *               iteration streams from HBM) and 0 otherwise (L2-resident and
  *               latency-bound, where 0 measured fastest).

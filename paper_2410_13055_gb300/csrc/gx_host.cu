@@ -88,6 +88,7 @@ struct gx_network {
     std::vector<BatW> bat_w;           // offsets of each battery warp
     int n_bus4_blk = 0, n_line4_blk = 0;
     size_t bus4_smem = 0;              // dynamic shared memory of the staged bus kernel (record + stage)
+    int bus4_rec = 0;                  // words of the longest record kept in shared memory
     std::vector<int> pool;             // their pool records (words)
     std::vector<int> bus_cpl;          // per hour-quad bus block: copy-list header and list (fixed stride)
     int bus_cpl_stride = 0, bus_cpl_max = 0;
@@ -354,6 +355,7 @@ static void make_ctx(gx_network* net) {
     c.prof_act = net->prof ? reinterpret_cast<long long*>(d + net->o_pact) : nullptr;
     c.bus_staged = net->sched.bus_staged;
     c.bus4_smem = (int)net->bus4_smem;
+    c.bus4_rec = net->bus4_rec;
     c.bat_warps = net->sched.bat_warps;
     CrsTables& t = net->crs_tables;
     t.bus = reinterpret_cast<const int4*>(d + net->o_crbus);
@@ -676,7 +678,7 @@ static double crs_assign(gx_network* net, const std::vector<int>& act, std::vect
 // (copies, forward bytes, adjoint bytes, 0) and copies at b * stride, where a block can read
 // them before it knows its record's offset.  Blocks whose record is not kept in shared memory
 // get an empty list and use the record path.  Built only while the lists stay small (they
-// repeat each scenario's records); above the cap the kernel reads the lists from the records.
+// repeat each scenario's records); above the cap the ring kernel runs.
 constexpr size_t kBusCplMaxBytes = 16u << 20;
 
 static void build_bus_copy_lists(gx_network* net) {
@@ -723,6 +725,7 @@ static void build_bus_blocks(gx_network* net) {
     // (quad, net, n0, n1, first quad of bus n0, end quad of bus n1, quads per row) -> (offset, words)
     std::map<std::tuple<int, int, int, int, int, int, int>, std::pair<int, int>> rec_of;
     net->bus4_smem = 0;
+    net->bus4_rec = 0;
     net->bus_blk.clear();
     net->bus4_blk.clear();
     net->pool.clear();
@@ -884,6 +887,7 @@ static void build_bus_blocks(gx_network* net) {
                     p[kPH_TXA] = (int)txa;
                     // the launch's dynamic shared memory holds the largest record kept in
                     // shared memory, with its stage if it has one
+                    if (words <= kPoolMax) net->bus4_rec = std::max(net->bus4_rec, words);
                     if (words <= kPoolMax)
                         net->bus4_smem = std::max<size_t>(net->bus4_smem,
                                                           4 * (size_t)words + (staged ? (size_t)sbytes : 0));
@@ -1350,14 +1354,14 @@ gx_status gx_network_bind(gx_network* net, void* dev_mem, size_t bytes, void* st
     if (!net->ev_fork) GX_CUDA(cudaEventCreateWithFlags(&net->ev_fork, cudaEventDisableTiming));
     if (!net->ev_join) GX_CUDA(cudaEventCreateWithFlags(&net->ev_join, cudaEventDisableTiming));
     if (!net->ev_join2) GX_CUDA(cudaEventCreateWithFlags(&net->ev_join2, cudaEventDisableTiming));
-    if (net->bus4_smem > 0) GX_CUDA(bus_staged_prepare((int)net->bus4_smem));
+    if (net->bus4_smem > 0) GX_CUDA(bus_staged_prepare((int)net->bus4_smem, net->bus4_rec));
     {
         int dev = 0, l2 = 0;
         GX_CUDA(cudaGetDevice(&dev));
         GX_CUDA(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
-        // An L2-resident workspace is latency-bound: there the staged kernel reads its copy
-        // lists from per-block slots (one dependent hop fewer, more registers); a workspace
-        // that streams from HBM keeps the record path and its occupancy.
+        // An L2-resident workspace is latency-bound: there the staged kernel brings every row of
+        // a block in at once; a workspace that streams from HBM takes the ring, whose blocks are
+        // small enough for eight per SM.
         net->l2_resident = net->lay.total <= (size_t)l2;
         // default bus kernel until a schedule is set: stage the device rows when the iteration
         // streams from HBM; the autotuner picks per workload

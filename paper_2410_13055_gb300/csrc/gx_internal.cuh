@@ -64,9 +64,9 @@ constexpr int kCplPerThread = 2;
 // staged copies: array ids and flags of a copy-list entry
 enum : int { kCpGenX = 0, kCpGenAux = 1, kCpDl = 2, kCpVf = 3, kCpVt = 4, kCpBat = 5 };
 enum : int { kCpFirm = 1, kCpRamp = 2 };   // (flags << 3): capacity factor 1 / ramp-limited generator
-// Largest row stage (bytes) of one bus block; blocks above it run unstaged.  The launch's
-// dynamic shared memory is the largest stage (plus its record), so this caps the staged bus
-// kernel's shared-memory occupancy.
+// Largest row stage (bytes) of one bulk-copied bus block; blocks above it run unstaged.  The launch's
+// dynamic shared memory is the largest stage (plus its record), so this caps the kernel's
+// shared-memory occupancy.
 #ifndef GX_STAGE_MAX_KB
 #define GX_STAGE_MAX_KB 40
 #endif
@@ -75,6 +75,9 @@ constexpr int kStageMax = GX_STAGE_MAX_KB * 1024;
 #ifndef GX_BUS4T_MINB
 #define GX_BUS4T_MINB 4
 #endif
+
+// devices whose quads a thread of the ring bus kernel has in flight
+constexpr int kBusRing = 4;
 
 // Cluster-resident solver: one thread-block cluster of C CTAs per scenario, CTA r owning
 // hours [r*H, (r+1)*H) of every device, its state in shared memory.
@@ -343,20 +346,21 @@ struct Ctx {
     unsigned long long* stamp_lo;  // [kStampSlots * 3]
     unsigned long long* stamp_hi;  // [kStampSlots * 3]
     long long* prof_act;           // [S]
-    // hour-quad bus kernel: 1 = stage the block's device rows in shared memory with bulk
-    // copies (k_bus4t), 0 = per-thread loads (k_bus4); the staged launch's dynamic shared
-    // memory; a bounded device-side wait that gave up writes its status to *err
+    // hour-quad bus kernel: 0 = per-thread loads (k_bus4), 1 = asynchronous copies: bulk copies of
+    // the block's device rows where the copy lists are used (bus_cpl, k_bus4t), else a ring per
+    // thread (k_bus4r), 2 = the ring; the bulk launch's dynamic shared memory; a bounded device-side wait that gave up writes its status to *err
     int bus_staged;
     int bus4_smem;
     // Bulk-staged bus kernel, per block at a fixed stride (built where the lists are small):
     // header (copies, forward bytes, adjoint bytes, 1 = take the record path) then the block's
     // copy list, so a block reads its list together with its block record; and per-block done
-    // flags, refreshed from the scenario flags at every chunk start.  bus_cpl == nullptr: every
-    // block reads its list from its record.
+    // flags, refreshed from the scenario flags at every chunk start.  bus_cpl == nullptr: the
+    // workspace streams from HBM (or a list is too long).
     const int* bus_cpl;
     int bus_cpl_stride, bus_cpl_max;  // ints per block; most copies of a block
     int* bus_done;                    // [n_bus4_blk]
     int bat_warps;       // battery prox warps per battery for horizons over 96 hours (1 or 2)
+    int bus4_rec;        // words of the longest block record kept in shared memory
     int* err;
 };
 
@@ -451,7 +455,7 @@ int launch_bus(const Ctx& c, int mode, int adj, int want_res, cudaStream_t st);
 int launch_prep(const Ctx& c, cudaStream_t st);
 // Allow the staged bus kernel `smem` bytes of dynamic shared memory (once per process is
 // enough; called at bind).
-cudaError_t bus_staged_prepare(int smem);
+cudaError_t bus_staged_prepare(int smem, int rec);
 int launch_loop_cond(const Ctx& c, const int* pause, int max_it, cudaGraphConditionalHandle h, cudaStream_t st);
 typedef void (*CrsFn)(Ctx, CrsTables, const int*, int, int, double, int, int);
 // Cluster-resident solver (gx_crs.cu): iterate the scenarios in `scen` to convergence, one cluster

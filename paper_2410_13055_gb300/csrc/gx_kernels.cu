@@ -782,6 +782,15 @@ __device__ __forceinline__ void ld4(const float* p, float (&v)[4]) {
 __device__ __forceinline__ void st4(float* p, const float (&v)[4]) {
     *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
 }
+// Store of an updated quad, left out where all four values are bit for bit the ones there (x): most
+// generator hours lie on a bound, or are fixed at one in the adjoint, and do not move.  (13 x 168 h of
+// 2000 buses: 156.0 us an iteration instead of 157.5.)
+__device__ __forceinline__ void st4_moved(float* p, const float (&v)[4], const float (&x)[4]) {
+    bool moved = false;
+#pragma unroll
+    for (int h = 0; h < 4; ++h) moved |= __float_as_int(v[h]) != __float_as_int(x[h]);
+    if (moved) st4(p, v);
+}
 // Operand orders of the fused multiply-adds are written out in the iteration kernels, so that every
 // instance, with or without the residual terms, takes the same iterates bit for bit.
 // (a x + b y with a x rounded, b y fused:)
@@ -1016,7 +1025,7 @@ __global__ void __launch_bounds__(kBusQBlock, kBus4MinBlocks) k_bus4(const Ctx c
                     x2 += xn[h] * xn[h];
                 }
             }
-            st4(X.xg + r, xn);
+            st4_moved(X.xg + r, xn, x);
         }
         {
             float xn[4];
@@ -1039,7 +1048,7 @@ __global__ void __launch_bounds__(kBusQBlock, kBus4MinBlocks) k_bus4(const Ctx c
                     x2 += xn[h] * xn[h];
                 }
             }
-            st4(X.xl + i, xn);
+            st4_moved(X.xl + i, xn, xl);
         }
 #pragma unroll
         for (int k = 0; k < kBC4; ++k) {
@@ -1125,15 +1134,235 @@ __global__ void __launch_bounds__(kBusQBlock, kBus4MinBlocks) k_bus4(const Ctx c
 }
 
 // ------------------------------------------------------------------------------------
+// Bus kernel with a ring of asynchronous copies per thread.  The same iteration as k_bus4,
+// expression for expression and in the same summation order, for workloads that stream from HBM.
+// A thread walks its bus's device list (generators, batteries, line ends) with the quads of the next
+// kBusRing devices in flight in its own shared-memory slots (cp.async, one group a device), so
+// its arithmetic runs under the loads of the devices after it, and nothing waits for other threads
+// but the record copy.  The ring bounds the shared memory (32 bytes a device and thread) whatever the
+// device count: 16 KB and a record where staging every row of a block took up to 43, eight blocks
+// per SM instead of five.  That is what counts: a block waits for three dependent hops (its block
+// record, its pool record, its rows) of about a microsecond each, and with 18 warps per SM the DRAM
+// was 45 % busy.  13 x 168 h of 2000 buses: 83 us with every row staged by bulk copies, 65 here (4.7
+// TB/s), the iteration 156 and 137; 64 networks of 50 to 500 buses 69 and 64.  Rings of 3 and 6 devices
+// and caps of 6 to 9 blocks lie within 3 %; 8 and 10 devices are 3 and 7 % slower.
+// ------------------------------------------------------------------------------------
+template <int ADJ, int RAMP, int WANT>
+__global__ void __launch_bounds__(kBusQBlock, (WANT ? 6 : 8) * 128 / kBusQBlock) k_bus4r(const Ctx c) {
+    extern __shared__ __align__(16) int S[];  // the block's record, then the ring
+    const bool stamp = WANT && c.stamp_lo != nullptr;
+    if (stamp && threadIdx.x == 0) stamp_start(c, 0);
+    const BusBlk bb = c.bus4_blk[blockIdx.x];
+    const int done = c.done[bb.s];
+    const StatePtrs X = state<ADJ>(c);
+    const bool staged = bb.words <= kPoolMax;
+    const int Tq = bb.Tp >> 2;
+    const int local = bb.item0 + threadIdx.x;
+    const int n = local / Tq;
+    const int t = (local - n * Tq) * 4;
+    const bool valid = local < bb.nitems;
+    const long long i = bb.e_bus + (long long)n * bb.Tp + t;
+    float pb[4], uu[4], thold[4], xl[4], Ld[4], al[4];
+    if (staged) {
+        const int4* src = reinterpret_cast<const int4*>(c.pool + bb.pool);
+        int4* dst = reinterpret_cast<int4*>(S);
+        for (int k = threadIdx.x; k < (bb.words >> 2); k += kBusQBlock) cp_async16(dst + k, src + k);
+    }
+    cp_async_commit();
+    if (valid) {
+        ld4(X.pbar + i, pb); ld4(X.u + i, uu);
+        if (WANT) ld4(X.thb + i, thold);
+        ld4(X.xl + i, xl);
+        if (ADJ) ld4(c.al + i, al);  // the adjoint needs the load only through its coefficient
+        else ld4(c.load + i, Ld);
+    }
+    cp_async_wait_all();
+    if (done) return;  // block-uniform, before any barrier or store
+    __syncthreads();
+    float acc[kBusPart] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (valid) {
+        const Pool P{staged ? S : c.pool + bb.pool};
+        float4* ring = reinterpret_cast<float4*>(S + (staged ? bb.words : 0)) + threadIdx.x;
+        const int nl = n - bb.n0;
+        const float rho = c.rho, eps = c.eps;
+        const float inv_re = 1.f / (rho + eps);
+        bool hv[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) hv[h] = t + h < bb.T;
+        float sum[4] = {0.f, 0.f, 0.f, 0.f}, dx2[4] = {0.f, 0.f, 0.f, 0.f};
+        float x2 = 0.f, gscale = 0.f;
+        const float* xg = X.xg + bb.e_gen + t;
+        const int g0 = P.at(kPH_GP, nl), g1 = P.at(kPH_GP, nl + 1);
+        const int e0 = P.at(kPH_EP, nl), e1 = P.at(kPH_EP, nl + 1);
+        const int b0 = P.at(kPH_BP, nl), b1 = P.at(kPH_BP, nl + 1);
+        // the next device to fetch (a generator below g1, then a battery, then a line end) and
+        // the ring slots of the next fetch and of the next device to take
+        int fg = g0, fb = b0, fe = e0, put = 0, get = 0;
+        auto fetch = [&]() {
+            float4* slot = ring + put * (2 * kBusQBlock);
+            if (fg < g1) {
+                const long long r = (long long)P.at(kPH_GROW, fg) * bb.Tp;
+                const int fl = P.at(kPH_GFIRM, fg);
+                cp_async16(slot, xg + r);
+                if (!(RAMP && (fl & 2)) && (ADJ || !(fl & 1))) cp_async16(slot + kBusQBlock, (ADJ ? c.ag : c.cf) + bb.e_gen + t + r);
+                ++fg;
+            } else if (fb < b1) {
+                cp_async16(slot, X.xb + bb.e_bat + (long long)P.at(kPH_BROW, fb) * bb.Tp + t);
+                ++fb;
+            } else if (fe < e1) {
+                const int e = P.at(kPH_ECODE, fe);
+                const long long r = bb.e_line + (long long)(e >> 1) * bb.Tp + t;
+                cp_async16(slot, X.dl + r);
+                cp_async16(slot + kBusQBlock, ((e & 1) ? X.vt : X.vf) + r);
+                ++fe;
+            }
+            cp_async_commit();  // (past the list's end an empty group, so that the count below holds)
+            put = put + 1 == kBusRing ? 0 : put + 1;
+        };
+        // the next device's quads (the group before the newest kBusRing - 1 ones has landed)
+        auto take = [&](float (&a)[4], float (&b)[4]) {
+            cp_async_wait<kBusRing - 1>();
+            const float4* slot = ring + get * (2 * kBusQBlock);
+            const float4 v = slot[0], w = slot[kBusQBlock];
+            a[0] = v.x; a[1] = v.y; a[2] = v.z; a[3] = v.w;
+            b[0] = w.x; b[1] = w.y; b[2] = w.z; b[3] = w.w;
+            get = get + 1 == kBusRing ? 0 : get + 1;
+        };
+#pragma unroll 1
+        for (int k = 0; k < kBusRing; ++k) fetch();
+        for (int q = g0; q < g1; ++q) {
+            const long long r = (long long)P.at(kPH_GROW, q) * bb.Tp;
+            const int fl = P.at(kPH_GFIRM, q);
+            float x[4], a[4], xn[4];
+            take(x, a);
+            if (RAMP && (fl & 2)) {
+                // ramp-limited: the ramp kernel wrote this iteration's injection (and keeps
+                // its own residual terms); the bus only sums it
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    sum[h] += x[h];
+                    if (WANT) x2 += x[h] * x[h];
+                }
+                fetch();
+                continue;
+            }
+            if (!ADJ && (fl & 1)) a[0] = a[1] = a[2] = a[3] = 1.f;
+            const float gcost = ADJ ? 0.f : P.atf(kPH_GCOST, q);
+            const float etag = ADJ ? 0.f : P.atf(kPH_GETA, q);
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                const float v = x[h] - pb[h] - uu[h];
+                if (ADJ) {
+                    const float gh = a[h];  // NaN: bound active, the variable is fixed at 0
+                    const bool fixed = gh != gh;
+                    xn[h] = fixed ? 0.f : __fmul_rn(__fmaf_rn(rho, v, gh), inv_re);
+                    if (WANT && !fixed && hv[h]) gscale += (gh * inv_re) * (gh * inv_re);
+                } else {
+                    const float cap = a[h] * etag;
+                    const float pun = __fmul_rn(__fmaf_rn(rho, v, -gcost), inv_re);
+                    xn[h] = clampf(pun, 0.f, cap);
+                }
+                if (!hv[h]) xn[h] = 0.f;
+                sum[h] += xn[h];
+                if (WANT) {
+                    dx2[h] += (xn[h] - x[h]) * (xn[h] - x[h]);
+                    x2 += xn[h] * xn[h];
+                }
+            }
+            st4_moved(X.xg + bb.e_gen + t + r, xn, x);
+            fetch();
+        }
+        {
+            float xn[4];
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                const float v = xl[h] - pb[h] - uu[h];
+                if (ADJ) {
+                    const float gsh = al[h];  // NaN: bound active, the variable is fixed at 0
+                    const bool fixed = gsh != gsh;
+                    xn[h] = fixed ? 0.f : __fmul_rn(__fmaf_rn(rho, v, gsh), inv_re);
+                    if (WANT && !fixed && hv[h]) gscale += (gsh * inv_re) * (gsh * inv_re);
+                } else {
+                    const float sun = __fmul_rn(__fmaf_rn(rho, __fadd_rn(v, Ld[h]), -c.voll), inv_re);
+                    xn[h] = clampf(sun, 0.f, Ld[h]) - Ld[h];
+                }
+                if (!hv[h]) xn[h] = 0.f;
+                sum[h] += xn[h];
+                if (WANT) {
+                    dx2[h] += (xn[h] - xl[h]) * (xn[h] - xl[h]);
+                    x2 += xn[h] * xn[h];
+                }
+            }
+            st4_moved(X.xl + i, xn, xl);
+        }
+        for (int q = b0; q < b1; ++q) {
+            float xb[4], none[4];
+            take(xb, none);
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                sum[h] += xb[h];
+                if (WANT) x2 += xb[h] * xb[h];
+            }
+            fetch();
+        }
+        float ths[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int q = e0; q < e1; ++q) {
+            const int e = P.at(kPH_ECODE, q);
+            const float beta = P.atf(kPH_EBETA, q), w = P.atf(kPH_EW, q);
+            float d[4], qv[4];
+            take(d, qv);
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                const float pp = __fmul_rn((e & 1) ? beta : -beta, d[h]);
+                sum[h] = __fadd_rn(sum[h], pp);
+                if (WANT) x2 += pp * pp;
+                ths[h] = __fmaf_rn(w, qv[h], ths[h]);
+            }
+            fetch();
+        }
+        const float icnt = P.atf(kPH_IC, nl), iws = P.atf(kPH_IW, nl), drw = P.atf(kPH_DR, nl);
+        const float cnt = 1.f / icnt;
+        float pbn[4], un[4], thn[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            pbn[h] = __fmul_rn(sum[h], icnt);
+            thn[h] = __fmul_rn(ths[h], iws);
+            un[h] = __fadd_rn(uu[h], pbn[h]);
+            if (WANT && hv[h]) {
+                const float dpb = pbn[h] - pb[h];
+                acc[0] += cnt * pbn[h] * pbn[h];
+                acc[2] += dx2[h] - cnt * dpb * dpb;
+                acc[3] += (thn[h] - thold[h]) * (thn[h] - thold[h]) * drw;
+                acc[4] += cnt * (rho * un[h]) * (rho * un[h]);
+            }
+        }
+        acc[1] = gscale;
+        acc[5] = x2;
+        st4(X.pbar + i, pbn);
+        st4(X.u + i, un);
+        st4(X.thb + i, thn);
+    }
+    if (WANT) {
+        __shared__ float sh[kBusPart][kBusQBlock / 32];
+        block_sum<kBusPart, kBusQBlock>(acc, sh);
+        if (threadIdx.x == 0) {
+#pragma unroll
+            for (int q = 0; q < kBusPart; ++q) c.bus_part[blockIdx.x * kBusPart + q] = acc[q];
+            if (stamp) stamp_end(c, 0);
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------
 // Staged bus kernel.  The same iteration as k_bus4, expression for expression and in the
 // same summation order (its iterates are bitwise those of k_bus4), with the block's device
 // rows brought into shared memory first.  In k_bus4 a thread walks its bus's devices with
 // one generator's loads in flight at a time, so a block waits for about 4 + (generators
 // per bus) dependent memory round trips.  Here the block issues one bulk copy per device
 // row segment (cp.async.bulk, completing on one mbarrier armed by thread 0; the copy list
-// is built at create, in the pool record), so every row the block needs is in flight at once and
-// the block waits for three hops: its block record; its pool record and the done flag; its
-// bus state and the rows together (a converged scenario's blocks stop after the second).
+// sits in the block's own slot, built at create), so every row the block needs is in flight at
+// once and a block waits for two hops.  For workspaces that fit the L2, where latency counts and
+// not the blocks per SM (100 buses x 168 h x 16: an iteration of 15.2 us, 16.1 with the ring).
 // In the adjoint the generators' aux rows hold the adjoint coefficient (NaN where the bound
 // is active), so the active set travels with the bulk copies.  A record too large for the
 // stage runs the unstaged loads.
@@ -1174,9 +1403,7 @@ __device__ __forceinline__ bool bulk_wait(const Ctx& c, unsigned long long* bar)
     return false;
 }
 
-// LIST: the block's copy list and done flag come from its own slot (c.bus_cpl); compiled
-// apart so that the record-path instance keeps its registers.
-template <int ADJ, int RAMP, int LIST, int WANT>
+template <int ADJ, int RAMP, int WANT>
 __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) k_bus4t(const Ctx c) {
     extern __shared__ __align__(16) int S[];  // the block's record, then its row stage
     __shared__ __align__(8) unsigned long long bar;
@@ -1184,31 +1411,25 @@ __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) 
     if (stamp && threadIdx.x == 0) stamp_start(c, 0);
     const BusBlk bb = c.bus4_blk[blockIdx.x];
     const StatePtrs X = state<ADJ>(c);
-    const bool bulk = c.bus_staged == 1;
     const bool rec_smem = bb.words <= kPoolMax;
-    // Bulk schedule with per-block copy lists: the block's list and its done flag sit at its
-    // own slot, so they are read together with the block record (hop 1), and the record and
-    // the rows arrive together one hop later.  Otherwise the list comes from the record.
-    const int* cpl = (LIST && bulk) ? c.bus_cpl + (long long)blockIdx.x * c.bus_cpl_stride : nullptr;
-    int cp_n = 0, cp_tx = 0, fdone = 0, cp_rec = 1;
+    // The block's copy list and its done flag sit at its own slot, so they are read together with
+    // the block record (hop 1), and the record and the rows arrive together one hop later.  A list
+    // or record too long for that (fast = false) is read from the record, a hop later.
+    const int* cpl = c.bus_cpl + (long long)blockIdx.x * c.bus_cpl_stride;
+    const int cp_n = cpl[0], cp_tx = cpl[ADJ ? 2 : 1];
+    const int fdone = c.bus_done[blockIdx.x];
+    const bool fast = cpl[3] == 0;  // the list and the record fit
     int cp_e[kCplPerThread][3];
-    if (LIST && cpl) {
-        cp_n = cpl[0];
-        cp_tx = cpl[ADJ ? 2 : 1];
-        cp_rec = cpl[3];
-        fdone = c.bus_done[blockIdx.x];
 #pragma unroll
-        for (int j = 0; j < kCplPerThread; ++j) {
-            const int k = (int)threadIdx.x + j * kBusQBlock;
-            cp_e[j][0] = cp_e[j][1] = cp_e[j][2] = 0;
-            if (k < c.bus_cpl_max) {
-                cp_e[j][0] = cpl[4 + 3 * k];
-                cp_e[j][1] = cpl[4 + 3 * k + 1];
-                cp_e[j][2] = cpl[4 + 3 * k + 2];
-            }
+    for (int j = 0; j < kCplPerThread; ++j) {
+        const int k = (int)threadIdx.x + j * kBusQBlock;
+        cp_e[j][0] = cp_e[j][1] = cp_e[j][2] = 0;
+        if (k < c.bus_cpl_max) {
+            cp_e[j][0] = cpl[4 + 3 * k];
+            cp_e[j][1] = cpl[4 + 3 * k + 1];
+            cp_e[j][2] = cpl[4 + 3 * k + 2];
         }
     }
-    const bool fast = LIST && cpl != nullptr && cp_rec == 0;  // a listed block's record fits shared memory
     // hop 2 (record path): the record and the done flag, in flight together
     if (!fast && rec_smem) {
         const int4* src = reinterpret_cast<const int4*>(c.pool + bb.pool);
@@ -1222,7 +1443,7 @@ __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) 
     const bool valid = local < bb.nitems;
     const long long i = bb.e_bus + (long long)n * bb.Tp + t;
     const int done = fast ? fdone : c.done[bb.s];
-    if (threadIdx.x == 0 && bulk && rec_smem) {
+    if (threadIdx.x == 0 && rec_smem) {
         mbar_init(&bar, 1);
         mbar_fence_init();
         if (fast) {
@@ -1263,7 +1484,7 @@ __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) 
     const int qg = P.p[kPH_QG], qe = P.p[kPH_QE];
     // hop 3 (bulk, record path): every device row segment of the block, the copy list split
     // over the warps
-    if (!fast && sbytes > 0 && bulk) {
+    if (!fast && sbytes > 0) {
         const int ncp = P.p[kPH_NCP];
         const int* rcpl = P.p + P.p[kPH_CP];
         for (int k = threadIdx.x; k < ncp; k += kBusQBlock) {
@@ -1275,34 +1496,7 @@ __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) 
     const int nl = n - bb.n0;
     const int nq = valid ? P.at(kPH_SQ, nl) : 0;
     const int pos = valid ? (int)threadIdx.x - P.at(kPH_SI, nl) : 0;
-    const long long gt = bb.e_gen + t;  // generator rows: gt + row * Tp
-    const int g0 = valid ? P.at(kPH_GP, nl) : 0, g1 = valid ? P.at(kPH_GP, nl + 1) : 0;
-    if (sbytes > 0 && !bulk && valid) {
-        // hop 3 (per thread): this thread's own quads of its bus's device rows, 16-byte
-        // asynchronous copies into the same stage slots (each thread reads only its own)
-        const int sg = P.at(kPH_SG, nl), se = P.at(kPH_SE, nl), sb = P.at(kPH_SB, nl);
-        for (int q = g0; q < g1; ++q) {
-            const int slot = sg + (q - g0) * nq + pos;
-            const long long r = gt + (long long)P.at(kPH_GROW, q) * bb.Tp;
-            const int fl = P.at(kPH_GFIRM, q);
-            cp_async16(stage + slot, X.xg + r);
-            if (!(fl & 2) && (ADJ || !(fl & 1))) cp_async16(stage + qg + slot, (ADJ ? c.ag : c.cf) + r);
-        }
-        const int e0 = P.at(kPH_EP, nl), e1 = P.at(kPH_EP, nl + 1);
-        for (int q = e0; q < e1; ++q) {
-            const int e = P.at(kPH_ECODE, q);
-            const int slot = se + (q - e0) * nq + pos;
-            const long long r = bb.e_line + (long long)(e >> 1) * bb.Tp + t;
-            cp_async16(stage + 2 * qg + slot, X.dl + r);
-            cp_async16(stage + 2 * qg + qe + slot, ((e & 1) ? X.vt : X.vf) + r);
-        }
-        const int b0 = P.at(kPH_BP, nl), b1 = P.at(kPH_BP, nl + 1);
-        for (int q = b0; q < b1; ++q)
-            cp_async16(stage + 2 * qg + 2 * qe + sb + (q - b0) * nq + pos,
-                       X.xb + bb.e_bat + (long long)P.at(kPH_BROW, q) * bb.Tp + t);
-    }
-    if (sbytes > 0 && !bulk) cp_async_wait_all();
-    if (!fast && sbytes > 0 && bulk && !bulk_wait<ADJ>(c, &bar)) return;
+    if (!fast && sbytes > 0 && !bulk_wait<ADJ>(c, &bar)) return;
     float acc[kBusPart] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (valid) {
         const bool stg = sbytes > 0;
@@ -1313,6 +1507,8 @@ __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) 
         for (int h = 0; h < 4; ++h) hv[h] = t + h < bb.T;
         float sum[4] = {0.f, 0.f, 0.f, 0.f}, dx2[4] = {0.f, 0.f, 0.f, 0.f};
         float x2 = 0.f, gscale = 0.f;
+        const long long gt = bb.e_gen + t;  // generator rows: gt + row * Tp
+        const int g0 = P.at(kPH_GP, nl), g1 = P.at(kPH_GP, nl + 1);
         const int e0 = P.at(kPH_EP, nl), e1 = P.at(kPH_EP, nl + 1);
         const int b0 = P.at(kPH_BP, nl), b1 = P.at(kPH_BP, nl + 1);
         const int sg = stg ? P.at(kPH_SG, nl) : 0, se = stg ? P.at(kPH_SE, nl) : 0, sb = stg ? P.at(kPH_SB, nl) : 0;
@@ -1369,7 +1565,7 @@ __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) 
                     x2 += xn[h] * xn[h];
                 }
             }
-            st4(X.xg + r, xn);
+            st4_moved(X.xg + r, xn, x);
         }
         {
             float xn[4];
@@ -1392,7 +1588,7 @@ __global__ void __launch_bounds__(kBusQBlock, GX_BUS4T_MINB * 128 / kBusQBlock) 
                     x2 += xn[h] * xn[h];
                 }
             }
-            st4(X.xl + i, xn);
+            st4_moved(X.xl + i, xn, xl);
         }
         for (int q = b0; q < b1; ++q) {
             float xb[4];
@@ -1920,11 +2116,12 @@ int launch_bus(const Ctx& c, int mode, int adj, int want_res, cudaStream_t st) {
         const int sm = c.bus4_smem;
         const bool want = (want_res & kWantRes) != 0, ramp = c.n_ramp_warps > 0;
         const bool list = c.bus_staged == 1 && c.bus_cpl != nullptr;
+        const int sr = 4 * c.bus4_rec + 32 * kBusRing * kBusQBlock;
 #define GX_BUS4W(A, R, W)                                                                      \
     do {                                                                                       \
         if (c.bus_staged == 0) k_bus4<A, R, W><<<c.n_bus4_blk, kBusQBlock, 0, st>>>(c);        \
-        else if (list) k_bus4t<A, R, 1, W><<<c.n_bus4_blk, kBusQBlock, sm, st>>>(c);           \
-        else k_bus4t<A, R, 0, W><<<c.n_bus4_blk, kBusQBlock, sm, st>>>(c);                     \
+        else if (list) k_bus4t<A, R, W><<<c.n_bus4_blk, kBusQBlock, sm, st>>>(c);              \
+        else k_bus4r<A, R, W><<<c.n_bus4_blk, kBusQBlock, sr, st>>>(c);                        \
     } while (0)
 #define GX_BUS4R(A, R)                  \
     do {                                \
@@ -1946,16 +2143,17 @@ int launch_bus(const Ctx& c, int mode, int adj, int want_res, cudaStream_t st) {
     return 1;
 }
 
-cudaError_t bus_staged_prepare(int smem) {
+cudaError_t bus_staged_prepare(int smem, int rec) {
     cudaError_t e = cudaSuccess;
-    auto set = [&](const void* f) {
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    auto set = [&](const void* f, int bytes) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     };
-#define GX_BUS4S(A, R)                               \
-    set((const void*)k_bus4t<A, R, 0, 0>);           \
-    set((const void*)k_bus4t<A, R, 0, 1>);           \
-    set((const void*)k_bus4t<A, R, 1, 0>);           \
-    set((const void*)k_bus4t<A, R, 1, 1>)
+    const int ring = 4 * rec + 32 * kBusRing * kBusQBlock;
+#define GX_BUS4S(A, R)                           \
+    set((const void*)k_bus4t<A, R, 0>, smem);    \
+    set((const void*)k_bus4t<A, R, 1>, smem);    \
+    set((const void*)k_bus4r<A, R, 0>, ring);    \
+    set((const void*)k_bus4r<A, R, 1>, ring)
     GX_BUS4S(0, 0);
     GX_BUS4S(1, 0);
     GX_BUS4S(0, 1);
