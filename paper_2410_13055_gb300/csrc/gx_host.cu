@@ -121,7 +121,7 @@ struct gx_network {
     long long bus_el = 0, gen_el = 0, line_el = 0, bat_el = 0;
     int n_bus_blk = 0, n_line_blk = 0, n_bat_warps = 0, n_cost_blk = 0, n_gwarps = 0, gs_total = 0;
     int tot_gen = 0, tot_line = 0, tot_bat = 0, tot_bus = 0, tot_ptr = 0, tot_ramp = 0;
-    std::vector<int> ramp_warp_scen;   // scenario of each ramp-kernel warp
+    std::vector<RampW> ramp_w;         // offsets of each ramp-kernel warp
     int n_ramp_warps = 0;
     long long ramp_el = 0;             // ramp state rows x Tp over all scenarios
     int max_ramp_T = 1;
@@ -284,7 +284,7 @@ static void make_ctx(gx_network* net) {
     c.bus_cpl_max = net->bus_cpl_max;
     c.bus_done = reinterpret_cast<int*>(d + net->o_busdone);
     c.n_ramp_warps = net->n_ramp_warps;
-    c.ramp_warp_scen = I(net->o_rws);
+    c.ramp_w = reinterpret_cast<const RampW*>(d + net->o_rws);
     c.r_gen = I(net->o_rgen);
     c.r_rate = F(net->o_rrate);
     c.g_ramp = I(net->o_gramp);
@@ -1069,7 +1069,16 @@ gx_status gx_network_create(const gx_network_desc* nets, int n_nets, const gx_sc
         sd.e_ramp = net->ramp_el;
         net->ramp_el += (long long)sd.R * sh.Tp;
         sd.ramp_w0 = net->n_ramp_warps;
-        for (int r = 0; r < sd.R; ++r) net->ramp_warp_scen.push_back(s);
+        for (int r = 0; r < sd.R; ++r) {
+            const int g = h.ramp_gens[r];
+            RampW w{};
+            w.row0 = sd.e_ramp + (long long)r * sh.Tp;
+            w.grow0 = sd.e_gen + (long long)g * sh.Tp;
+            w.brow0 = sd.e_bus + (long long)h.gen_bus[g] * sh.Tp;
+            w.s = s; w.T = sh.T; w.Tp = sh.Tp; w.gg = h.gen0 + g;
+            w.eta_g = h.eta0 + g; w.rate = h.ramp0 + r;
+            net->ramp_w.push_back(w);
+        }
         net->n_ramp_warps += sd.R;
         if (sd.R > 0) net->max_ramp_T = std::max(net->max_ramp_T, sh.T);
         sd.weight = (float)d.weight;
@@ -1191,7 +1200,7 @@ gx_status gx_network_create(const gx_network_desc* nets, int n_nets, const gx_sc
     net->o_rgen = L.add(I4(net->tot_ramp));
     net->o_rrate = L.add(F4(net->tot_ramp));
     net->o_gramp = L.add(I4(gen0));
-    net->o_rws = L.add(I4(net->n_ramp_warps));
+    net->o_rws = L.add(sizeof(RampW) * std::max<size_t>(net->ramp_w.size(), 1));
     net->o_rdd = L.add(F4(net->ramp_el));
     net->o_ardd = L.add(F4(net->ramp_el));
     net->o_scl = L.add(I4((long long)net->sc_line.size()));
@@ -1331,7 +1340,7 @@ gx_status gx_network_bind(gx_network* net, void* dev_mem, size_t bytes, void* st
         put(net->o_rgen, rgen.data(), 4 * rgen.size());
         put(net->o_rrate, rrate.data(), 4 * rrate.size());
         put(net->o_gramp, gramp.data(), 4 * (size_t)net->tot_gen);
-        put(net->o_rws, net->ramp_warp_scen.data(), 4 * net->ramp_warp_scen.size());
+        put(net->o_rws, net->ramp_w.data(), sizeof(RampW) * net->ramp_w.size());
     }
     GX_CUDA(cudaMemcpyAsync(net->dev, h.data(), net->static_end, cudaMemcpyHostToDevice, st));
     GX_CUDA(cudaMemsetAsync(net->dev + net->static_end, 0, net->lay.total - net->static_end, st));

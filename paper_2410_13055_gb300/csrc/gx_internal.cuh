@@ -197,6 +197,11 @@ struct BatW {
     int s, bg, T, Tp;          // scenario, battery (global index), true / padded horizon
     int eta_b, pad0, pad1, pad2;  // plan index of the battery's power
 };
+struct RampW {  // one per ramp-limited generator and scenario
+    long long row0, grow0, brow0;  // its ramp state row, its generator row, its bus's row
+    int s, T, Tp, gg;              // scenario, true / padded horizon, generator (global index)
+    int eta_g, rate;               // plan index of its capacity, index of its ramp rate
+};
 
 // Kernel modes.  FWD/ADJ advance the forward or adjoint message passing by one
 // iteration; RESET/INIT prepare a cold or user start; MASK records the active set.
@@ -259,7 +264,7 @@ struct Ctx {
     const int* line4_blk_scen; // [n_line4_blk]
     const LineBlk* line4_blk;  // [n_line4_blk]
     const BatW* bat_w;         // [n_bat_warps]
-    const int* ramp_warp_scen; // [n_ramp_warps]
+    const RampW* ramp_w;       // [n_ramp_warps]
     const int* r_gen;          // [ramping generators] generator index within its network
     const float* r_rate;       // [ramping generators] ramp limit / capacity per hour
     const int* g_ramp;         // [generators] index among its network's ramping generators, -1 if none
