@@ -131,9 +131,11 @@ __global__ void __launch_bounds__(kBusQBlock) k_features(const Ctx c, const floa
 // Epilogues: kEpiFwd  Z = D + b;  H = relu(Z) (+ resid);  and a BF16 copy of H for the next
 //                     layer's operand;
 //            kEpiBwd  dH[:, 0:64] += D[:, 0:64];  dAgg = D[:, 64:128]   (D = dZ W^T);
-//            kEpiHead the last layer of a prediction: H as in kEpiFwd, of which only the output
-//                     layer y = H W_out + b_out leaves the CTA, as prices ($/MWh) and angles.
-// A prediction needs no Z (kept for the backward pass alone): o.Z is null there.
+//            kEpiHead the last layer: as kEpiFwd, and the output layer y = H W_out + b_out: a
+//                     prediction's prices ($/MWh) and angles, or a training step's Y.
+// What only the backward pass reads (Z, the last layer's H) is null in a prediction.
+// Bound by HBM: a hidden layer's tile moves 128 rows of 768 bytes (1,024 with Z).  268,800 rows: 39 us
+// (57 with the epilogue's reads among its stores), in training 48 (63), backward 36 (63).
 enum : int { kEpiFwd = 0, kEpiBwd = 1, kEpiHead = 2 };
 
 struct DenseOut {
@@ -145,8 +147,9 @@ struct DenseOut {
     float* dH;
     float* dAgg;
     int* err;
-    const float* head;  // kEpiHead: W_out [64][2], b_out [2]; predictions, prices then angles
-    float* pred;
+    const float* head;  // kEpiHead: W_out [64][2], b_out [2]
+    float* pred;        // predictions, prices then angles, or (nullptr)
+    float* Y;           // a training step's outputs
 };
 
 template <int NKB, int KW, int N>
@@ -198,6 +201,21 @@ __global__ void __launch_bounds__(128) k_dense(const __grid_constant__ CUtensorM
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *holder;
+    // The FP32 rows that the epilogue adds to (the residual input, or dH), 32 columns ahead of
+    // the stores: read in the loop that stores, each row's load waited for the store before it, 16
+    // round trips a tile.  They do not wait for the tile's operands either.
+    const int cq = lane & 7, rq = lane >> 3;
+    const float* add = EPI == kEpiBwd ? o.dH : o.resid;
+    float4 pre[8];
+    auto ahead = [&](int c) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const long long r = row0 + warp * 32 + 4 * i + rq;
+            pre[i] = add && r < M ? *reinterpret_cast<const float4*>(add + r * kH + 32 * c + 4 * cq)
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    ahead(0);
     if (tid == 0) {
         mbar_expect_tx(&bar[0], Sh::TX);
         bulk_g2s(sB, bimg, Sh::BBYTES, &bar[0]);
@@ -232,11 +250,10 @@ __global__ void __launch_bounds__(128) k_dense(const __grid_constant__ CUtensorM
             // its shared-memory stage, and writes rows as 128-byte segments: lane l takes
             // columns 4 (l % 8) .. +3 of rows 4 i + l / 8, i = 0..7.
             const uint32_t tq = tmem + ((uint32_t)(warp * 32) << 16);
-            const int cq = lane & 7, rq = lane >> 3;
             float y0[8], y1[8];  // kEpiHead: the lane's share of its rows' outputs
 #pragma unroll
             for (int i = 0; i < 8; ++i) y0[i] = y1[i] = 0.f;
-#pragma unroll 1
+#pragma unroll
             for (int c = 0; c < N / 32; ++c) {
                 float v[32];
                 tmem_ld32(tq + 32u * c, v);  // warp-collective: rows past M take part too
@@ -252,6 +269,10 @@ __global__ void __launch_bounds__(128) k_dense(const __grid_constant__ CUtensorM
                     w0 = *reinterpret_cast<const float4*>(o.head + 2 * col);
                     w1 = *reinterpret_cast<const float4*>(o.head + 2 * col + 4);
                 }
+                float4 acc[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[i] = pre[i];
+                if (c + 1 < kH / 32) ahead(c + 1);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const int lr = 4 * i + rq;
@@ -260,16 +281,16 @@ __global__ void __launch_bounds__(128) k_dense(const __grid_constant__ CUtensorM
                     const float4 d = *reinterpret_cast<const float4*>(sE + lr * Sh::EPITCH + 4 * cq);
                     if (EPI != kEpiBwd) {
                         const float4 z = make_float4(d.x + b.x, d.y + b.y, d.z + b.z, d.w + b.w);
-                        if (EPI == kEpiFwd && o.Z) *reinterpret_cast<float4*>(o.Z + r * N + col) = z;
+                        if (o.Z) *reinterpret_cast<float4*>(o.Z + r * N + col) = z;
                         float4 h = make_float4(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f), fmaxf(z.z, 0.f), fmaxf(z.w, 0.f));
                         if (o.resid) {
-                            const float4 a = *reinterpret_cast<const float4*>(o.resid + r * N + col);
+                            const float4 a = acc[i];
                             h.x += a.x; h.y += a.y; h.z += a.z; h.w += a.w;
                         }
                         if (EPI == kEpiHead) {
                             y0[i] += h.x * w0.x + h.y * w0.z + h.z * w1.x + h.w * w1.z;
                             y1[i] += h.x * w0.y + h.y * w0.w + h.z * w1.y + h.w * w1.w;
-                            continue;
+                            if (!o.H) continue;
                         }
                         *reinterpret_cast<float4*>(o.H + r * N + col) = h;
                         if (o.Hb) {
@@ -280,7 +301,7 @@ __global__ void __launch_bounds__(128) k_dense(const __grid_constant__ CUtensorM
                     } else if (c < 2) {
                         // columns [0, 64): the direct half, added into dH
                         float4* p = reinterpret_cast<float4*>(o.dH + r * kH + col);
-                        const float4 a = *p;
+                        const float4 a = acc[i];
                         *p = make_float4(a.x + d.x, a.y + d.y, a.z + d.z, a.w + d.w);
                     } else {
                         // columns [64, 128): the neighbour half
@@ -299,8 +320,13 @@ __global__ void __launch_bounds__(128) k_dense(const __grid_constant__ CUtensorM
                     }
                     const long long r = row0 + warp * 32 + 4 * i + rq;
                     if (cq == 0 && r < M) {
-                        o.pred[r] = 100.f * (y0[i] + o.head[2 * kH]);
-                        o.pred[M + r] = y1[i] + o.head[2 * kH + 1];
+                        const float2 y = make_float2(y0[i] + o.head[2 * kH], y1[i] + o.head[2 * kH + 1]);
+                        if (o.pred) {
+                            o.pred[r] = 100.f * y.x;
+                            o.pred[M + r] = y.y;
+                        } else {
+                            reinterpret_cast<float2*>(o.Y)[r] = y;
+                        }
                     }
                 }
             }
@@ -447,25 +473,6 @@ __device__ __forceinline__ void add_colsum(float* sh, const float4& v, int f, fl
     for (int i = threadIdx.x; i < kH; i += blockDim.x) atomicAdd(&db[i], sh[i]);
 }
 
-// The top layer's dZ = dH * (Z > 0): its BF16 copy (the operand of dZ W^T and of the weight
-// gradient) and its column sums (the bias gradient, from the FP32 values); the layers below get
-// theirs from the transposed aggregation.  Streams dH and Z once, 16 bytes a load; dZ itself is
-// not stored.
-constexpr int kReluBlocks = 1216;
-__global__ void __launch_bounds__(256) k_relu_back(const float* __restrict__ dH, const float* __restrict__ Z,
-                                                   __nv_bfloat16* __restrict__ dZb, float* __restrict__ db, long long M) {
-    __shared__ float sh[kH];
-    const int f = 4 * (threadIdx.x & 15);
-    float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (long long r = (long long)blockIdx.x * 16 + (threadIdx.x >> 4); r < M; r += (long long)gridDim.x * 16) {
-        float4 d = *reinterpret_cast<const float4*>(dH + r * kH + f);
-        relu_mask(d, *reinterpret_cast<const float4*>(Z + r * kH + f));
-        store_bf16x4(dZb + r * kH + f, d);
-        cs.x += d.x; cs.y += d.y; cs.z += d.z; cs.w += d.w;
-    }
-    add_colsum(sh, cs, f, db);
-}
-
 // ---------------------------------------------------------------- aggregation
 // outb[i] = BF16 of the mean over neighbour buses m of in[(m, t)] (the next layer's operand), or
 // (transpose) out[i] += sum over neighbours m of in[(m, t)] / deg(m).  A block takes the hour quads
@@ -538,26 +545,6 @@ __global__ void __launch_bounds__(32 * kAggWarps) k_agg(const Ctx c, const float
     if (TRANSPOSE) add_colsum(sh, cs, f, db);
 }
 
-// ---------------------------------------------------------------- head, loss, backward head
-__global__ void k_head(const float* __restrict__ H, const float* __restrict__ P, float* __restrict__ Y, long long M) {
-    const long long i = (long long)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-    if (i >= M) return;
-    const int lane = threadIdx.x & 31;
-    const float2 h = reinterpret_cast<const float2*>(H + i * kH)[lane];
-    const float* W = P + kOffWout;
-    float y0 = h.x * W[(2 * lane) * 2 + 0] + h.y * W[(2 * lane + 1) * 2 + 0];
-    float y1 = h.x * W[(2 * lane) * 2 + 1] + h.y * W[(2 * lane + 1) * 2 + 1];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        y0 += __shfl_xor_sync(0xffffffffu, y0, o);
-        y1 += __shfl_xor_sync(0xffffffffu, y1, o);
-    }
-    if (lane == 0) {
-        Y[2 * i] = y0 + P[kOffBout];
-        Y[2 * i + 1] = y1 + P[kOffBout + 1];
-    }
-}
-
 // loss over valid nodes (hour < T); dY = d loss / d y; target layout [prices | angles]
 __global__ void k_loss(const Ctx c, const float* __restrict__ Y, const float* __restrict__ tgt, long long M,
                        double inv_count, float w_theta, float* __restrict__ dY, double* __restrict__ loss) {
@@ -579,46 +566,85 @@ __global__ void k_loss(const Ctx c, const float* __restrict__ Y, const float* __
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0 && l != 0.0) atomicAdd(loss, l * inv_count);
+    // one atomic a block, 15 us at 268,800 rows (one a warp, all on one address: 20)
+    __shared__ double sh[8];
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = l;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) t += sh[w];
+        if (t != 0.0) atomicAdd(loss, t * inv_count);
+    }
 }
 
-// dW_out += H^T dY, db_out += sum dY, dH = dY W_out^T.  Warps stride over nodes (lane l owns
-// hidden units 2l, 2l + 1); the block sums its warps' partial weight gradients in shared
-// memory and adds them with one atomic per weight.
+// dW_out += H^T dY, db_out += sum dY, dH = dY W_out^T, and of the last layer dZb = BF16 of
+// dH * (Z > 0) with its column sums added into db.  Warps stride over nodes (lane l owns hidden
+// units 2l, 2l + 1); the block sums its warps' partial gradients in shared memory and adds them
+// with one atomic per weight.  Bound by HBM: 896 bytes a row, 45 us for
+// 268,800 rows.  With the masking in a pass of its own it was 25 + 32 us.
 constexpr int kHeadBlocks = 1024;
+constexpr int kHeadRed = 3 * kH + 2;
+constexpr int kHeadRows = 4;  // rows a warp has in flight (one at a time: 59 us)
 __global__ void __launch_bounds__(256) k_head_back(const float* __restrict__ H, const float* __restrict__ dY,
-                                                   const float* __restrict__ P, float* __restrict__ G,
-                                                   float* __restrict__ dH, long long M) {
-    __shared__ float red[8][2 * kH + 2];
+                                                   const float* __restrict__ P, const float* __restrict__ Z,
+                                                   float* __restrict__ G, float* __restrict__ dH,
+                                                   __nv_bfloat16* __restrict__ dZb, float* __restrict__ db, long long M) {
+    __shared__ float red[8][kHeadRed];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float* W = P + kOffWout;
     const float w00 = W[(2 * lane) * 2], w01 = W[(2 * lane) * 2 + 1];
     const float w10 = W[(2 * lane + 1) * 2], w11 = W[(2 * lane + 1) * 2 + 1];
+    float2 cs = make_float2(0.f, 0.f);
     float g00 = 0.f, g01 = 0.f, g10 = 0.f, g11 = 0.f, b0 = 0.f, b1 = 0.f;
-    for (long long i = (long long)blockIdx.x * 8 + warp; i < M; i += (long long)gridDim.x * 8) {
-        const float2 h = reinterpret_cast<const float2*>(H + i * kH)[lane];
-        const float d0 = dY[2 * i], d1 = dY[2 * i + 1];
-        g00 += h.x * d0; g01 += h.x * d1;
-        g10 += h.y * d0; g11 += h.y * d1;
-        b0 += d0; b1 += d1;
-        reinterpret_cast<float2*>(dH + i * kH)[lane] = make_float2(d0 * w00 + d1 * w01, d0 * w10 + d1 * w11);
+    for (long long i0 = ((long long)blockIdx.x * 8 + warp) * kHeadRows; i0 < M; i0 += (long long)gridDim.x * 8 * kHeadRows) {
+        float2 h[kHeadRows], z[kHeadRows], y[kHeadRows];
+#pragma unroll
+        for (int k = 0; k < kHeadRows; ++k) {
+            const long long i = i0 + k;
+            h[k] = z[k] = y[k] = make_float2(0.f, 0.f);
+            if (i < M) {
+                h[k] = reinterpret_cast<const float2*>(H + i * kH)[lane];
+                z[k] = reinterpret_cast<const float2*>(Z + i * kH)[lane];
+                y[k] = reinterpret_cast<const float2*>(dY)[i];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kHeadRows; ++k) {
+            const long long i = i0 + k;
+            if (i >= M) break;
+            const float d0 = y[k].x, d1 = y[k].y;
+            g00 += h[k].x * d0; g01 += h[k].x * d1;
+            g10 += h[k].y * d0; g11 += h[k].y * d1;
+            b0 += d0; b1 += d1;
+            float2 d = make_float2(d0 * w00 + d1 * w01, d0 * w10 + d1 * w11);
+            reinterpret_cast<float2*>(dH + i * kH)[lane] = d;
+            d.x = z[k].x > 0.f ? d.x : 0.f;
+            d.y = z[k].y > 0.f ? d.y : 0.f;
+            reinterpret_cast<__nv_bfloat162*>(dZb + i * kH)[lane] = __floats2bfloat162_rn(d.x, d.y);
+            cs.x += d.x;
+            cs.y += d.y;
+        }
     }
     red[warp][4 * lane] = g00;
     red[warp][4 * lane + 1] = g01;
     red[warp][4 * lane + 2] = g10;
     red[warp][4 * lane + 3] = g11;
+    red[warp][2 * kH + 2 + 2 * lane] = cs.x;
+    red[warp][2 * kH + 3 + 2 * lane] = cs.y;
     if (lane == 0) {
         red[warp][2 * kH] = b0;
         red[warp][2 * kH + 1] = b1;
     }
     __syncthreads();
     // red[w][4 l + 2 u + o] is the gradient of W_out[2 l + u][o] = GW[(2 l + u) * 2 + o]
-    for (int k = threadIdx.x; k < 2 * kH + 2; k += blockDim.x) {
+    for (int k = threadIdx.x; k < kHeadRed; k += blockDim.x) {
         float t = 0.f;
 #pragma unroll
         for (int w = 0; w < 8; ++w) t += red[w][k];
         if (k < 2 * kH) atomicAdd(&G[kOffWout + k], t);
-        else atomicAdd(&G[kOffBout + k - 2 * kH], t);
+        else if (k < 2 * kH + 2) atomicAdd(&G[kOffBout + k - 2 * kH], t);
+        else atomicAdd(&db[k - 2 * kH - 2], t);
     }
 }
 
@@ -907,7 +933,7 @@ static void gnn_forward(gx_gnn* g, const float* eta, cudaStream_t st, int* err, 
     auto Agb = [&](int l) { return Bf(g->o_Agb) + (size_t)l * M * kH; };
     k_features<<<c.n_bus4_blk, kBusQBlock, 0, st>>>(c, eta, Bf(g->o_Xb));
     float* H0 = F(g->o_Hs);
-    DenseOut o{P + kOffBin, nullptr, pred ? nullptr : F(g->o_Z0), H0, Hb(0), nullptr, nullptr, err, nullptr, nullptr};
+    DenseOut o{P + kOffBin, nullptr, pred ? nullptr : F(g->o_Z0), H0, Hb(0), nullptr, nullptr, err, nullptr, nullptr, nullptr};
     dense_launch<1, kFin, kH, kEpiFwd>(g->maps[gx_gnn::kMapX], g->maps[gx_gnn::kMapX], g->dev + g->o_img_in, o, M,
                                         st);
     for (int l = 0; l < kLayers; ++l) {
@@ -916,14 +942,14 @@ static void gnn_forward(gx_gnn* g, const float* eta, cudaStream_t st, int* err, 
         k_agg<0><<<agg_grid(g), 32 * kAggWarps, 0, st>>>(c, Hl, nullptr, Agb(l), nullptr, nullptr);
         // H_{l+1} = H_l + relu([H_l, mean] W_l + b_l); its BF16 copy feeds the next layer
         const bool last = l + 1 == kLayers;
-        DenseOut ol{P + kOffL0 + l * kLayerSz + 2 * kH * kH, Hl, pred ? nullptr : F(g->o_Zs) + (size_t)l * M * kH, Hn,
-                    last ? nullptr : Hb(l + 1), nullptr, nullptr, err, P + kOffWout, pred};
+        DenseOut ol{P + kOffL0 + l * kLayerSz + 2 * kH * kH, Hl, pred ? nullptr : F(g->o_Zs) + (size_t)l * M * kH,
+                    pred && last ? nullptr : Hn, last ? nullptr : Hb(l + 1), nullptr, nullptr, err, P + kOffWout, pred,
+                    F(g->o_Y)};
         const CUtensorMap &mh = g->maps[gx_gnn::kMapH + l], &ma = g->maps[gx_gnn::kMapAg + l];
         const uint8_t* img = g->dev + g->o_img_fwd + (size_t)l * kImgLayer;
-        if (pred && last) dense_launch<2, kH, kH, kEpiHead>(mh, ma, img, ol, M, st);
+        if (last) dense_launch<2, kH, kH, kEpiHead>(mh, ma, img, ol, M, st);
         else dense_launch<2, kH, kH, kEpiFwd>(mh, ma, img, ol, M, st);
     }
-    if (!pred) k_head<<<(unsigned)((M + 7) / 8), 256, 0, st>>>(F(g->o_Hs) + (size_t)kLayers * M * kH, P, F(g->o_Y), M);
 }
 
 gx_status gx_gnn_predict(gx_gnn* g, const float* eta_dev, float* out_dev, void* stream) {
@@ -975,23 +1001,21 @@ gx_status gx_gnn_train_step(gx_gnn* g, const float* eta_dev, const float* target
     k_loss<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(c, F(g->o_Y), target_dev, M, 1.0 / g->valid, w_theta,
                                                         F(g->o_dY), reinterpret_cast<double*>(g->dev + g->o_loss));
     float* dH = F(g->o_dH);
-    k_head_back<<<(unsigned)std::min<long long>((M + 7) / 8, kHeadBlocks), 256, 0, st>>>(
-        F(g->o_Hs) + (size_t)kLayers * M * kH, F(g->o_dY), P, G, dH, M);
     // persistent weight-gradient CTAs: one per SM, none without a row tile
     const long long ntiles = (M + 127) / 128;
     const unsigned wg = (unsigned)std::min<long long>(ntiles, std::max(g->sms, 1));
     const CUtensorMap& mapdZ = g->maps[gx_gnn::kMapdZ];
     auto bias = [&](int l) { return l < 0 ? G + kOffBin : G + kOffL0 + l * kLayerSz + 2 * kH * kH; };
     auto Z = [&](int l) { return l < 0 ? F(g->o_Z0) : F(g->o_Zs) + (size_t)l * M * kH; };
-    k_relu_back<<<(unsigned)std::min<long long>((M + 15) / 16, kReluBlocks), 256, 0, st>>>(
-        dH, Z(kLayers - 1), dZb, bias(kLayers - 1), M);
+    k_head_back<<<(unsigned)std::min<long long>((M + 8 * kHeadRows - 1) / (8 * kHeadRows), kHeadBlocks), 256, 0, st>>>(
+        F(g->o_Hs) + (size_t)kLayers * M * kH, F(g->o_dY), P, Z(kLayers - 1), G, dH, dZb, bias(kLayers - 1), M);
     for (int l = kLayers - 1; l >= 0; --l) {
         k_wgrad<2 * kH><<<wg, 128, kWSmem, st>>>(g->maps[gx_gnn::kMapH + l], g->maps[gx_gnn::kMapAg + l], mapdZ,
                                                    G + kOffL0 + l * kLayerSz, M, err);
         // [dH_direct, dAgg] = dZ W_l^T on the tensor cores; the residual keeps dH, the direct
         // half is added into it, the neighbour half goes through the transposed aggregation,
         // which also leaves the layer below its dZ and bias gradient
-        DenseOut ob{nullptr, nullptr, nullptr, nullptr, nullptr, dH, F(g->o_dAgg), err, nullptr, nullptr};
+        DenseOut ob{nullptr, nullptr, nullptr, nullptr, nullptr, dH, F(g->o_dAgg), err, nullptr, nullptr, nullptr};
         dense_launch<1, kH, 2 * kH, kEpiBwd>(mapdZ, mapdZ, g->dev + g->o_img_bwd + (size_t)l * kImgLayer, ob, M, st);
         k_agg<1><<<agg_grid(g), 32 * kAggWarps, 0, st>>>(c, F(g->o_dAgg), dH, dZb, Z(l - 1), bias(l - 1));
     }
