@@ -131,7 +131,7 @@ struct gx_network {
     size_t o_crbus, o_crgen, o_crend, o_crline, o_crbat, o_crcls, o_crrep;
     size_t o_bus4blk, o_l4bs, o_l4blk, o_batw, o_buscpl, o_busdone;
     size_t o_scl, o_sce, o_scb, o_scbm, o_scp, o_scd, o_scdl, o_scgw;
-    size_t o_rgen, o_rrate, o_gramp, o_rws, o_rdd, o_ardd, o_rf[4], o_ra[4], o_rpart;
+    size_t o_rrate, o_gramp, o_rws, o_rdd, o_ardd, o_rf[4], o_ra[4], o_rpart;
     size_t o_gbus, o_gcost, o_gemis, o_gfirm, o_lfrom, o_lto, o_lbeta, o_ldth, o_lw, o_bbus, o_bdur, o_beffc, o_beffd;
     size_t o_gptr, o_gidx, o_bptr, o_bidx, o_eptr, o_eidx, o_icnt, o_iwsum, o_dresw;
     size_t o_load, o_cf, o_dd, o_add;
@@ -285,7 +285,6 @@ static void make_ctx(gx_network* net) {
     c.bus_done = reinterpret_cast<int*>(d + net->o_busdone);
     c.n_ramp_warps = net->n_ramp_warps;
     c.ramp_w = reinterpret_cast<const RampW*>(d + net->o_rws);
-    c.r_gen = I(net->o_rgen);
     c.r_rate = F(net->o_rrate);
     c.g_ramp = I(net->o_gramp);
     c.ramp_dd = F(net->o_rdd);
@@ -1197,7 +1196,6 @@ gx_status gx_network_create(const gx_network_desc* nets, int n_nets, const gx_sc
     net->o_icnt = L.add(F4(bus0)); net->o_iwsum = L.add(F4(bus0)); net->o_dresw = L.add(F4(bus0));
     net->o_load = L.add(F4(eb)); net->o_cf = L.add(F4(eg)); net->o_dd = L.add(F4(ebt));
     net->o_add = L.add(F4(ebt));
-    net->o_rgen = L.add(I4(net->tot_ramp));
     net->o_rrate = L.add(F4(net->tot_ramp));
     net->o_gramp = L.add(I4(gen0));
     net->o_rws = L.add(sizeof(RampW) * std::max<size_t>(net->ramp_w.size(), 1));
@@ -1328,16 +1326,12 @@ gx_status gx_network_bind(gx_network* net, void* dev_mem, size_t bytes, void* st
     put_v(net->o_rdd, net->rdd_host, 0);
     put_v(net->o_ardd, net->ardd_host, 0);
     {
-        std::vector<int> rgen, gramp(std::max(net->tot_gen, 1), -1);
+        std::vector<int> gramp(std::max(net->tot_gen, 1), -1);
         std::vector<float> rrate;
         for (const NetH& n : net->nets) {
-            for (int r = 0; r < (int)n.ramp_gens.size(); ++r) {
-                rgen.push_back(n.ramp_gens[r]);
-                rrate.push_back((float)n.gen_ramp[n.ramp_gens[r]]);
-            }
+            for (int g : n.ramp_gens) rrate.push_back((float)n.gen_ramp[g]);
             for (int g = 0; g < n.G; ++g) gramp[n.gen0 + g] = n.g_ramp[g];
         }
-        put(net->o_rgen, rgen.data(), 4 * rgen.size());
         put(net->o_rrate, rrate.data(), 4 * rrate.size());
         put(net->o_gramp, gramp.data(), 4 * (size_t)net->tot_gen);
         put(net->o_rws, net->ramp_w.data(), sizeof(RampW) * net->ramp_w.size());

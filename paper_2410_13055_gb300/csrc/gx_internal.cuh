@@ -265,7 +265,6 @@ struct Ctx {
     const LineBlk* line4_blk;  // [n_line4_blk]
     const BatW* bat_w;         // [n_bat_warps]
     const RampW* ramp_w;       // [n_ramp_warps]
-    const int* r_gen;          // [ramping generators] generator index within its network
     const float* r_rate;       // [ramping generators] ramp limit / capacity per hour
     const int* g_ramp;         // [generators] index among its network's ramping generators, -1 if none
     int* pool;                 // bus-block pool records (generator plan values refreshed per call)

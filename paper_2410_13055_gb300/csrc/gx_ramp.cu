@@ -49,6 +49,9 @@ __device__ __forceinline__ RampPtrs ramp_state(const Ctx& c) {
 
 template <int MODE, int ADJ, int kHpl>
 __global__ void __launch_bounds__(kBatWarps * 32) k_ramp(const Ctx c, int want_res) {
+    // (up to 32 hours, one a lane, the kernel before this one fused the backward sweep's last sum the
+    // other way round: its iterates are kept)
+    constexpr bool kSecond = kHpl == 1;
     const int lane = threadIdx.x & 31;
     const int gw = blockIdx.x * kBatWarps + (threadIdx.x >> 5);
     if (gw >= c.n_ramp_warps) return;
@@ -216,7 +219,11 @@ __global__ void __launch_bounds__(kBatWarps * 32) k_ramp(const Ctx c, int want_r
             const int t = t0 + j;
             const bool ok = (j < hpl) && (t < T);
             px[j] = 0.f;
-            if (ok) { pn = __fmaf_rn(__fmul_rn(ri, ba[j]), pn, __fmul_rn(ba[j], bp[j])); px[j] = pn; }
+            if (ok) {
+                const float g = __fmul_rn(ri, ba[j]);
+                pn = kSecond ? __fmaf_rn(ba[j], bp[j], __fmul_rn(g, pn)) : __fmaf_rn(g, pn, __fmul_rn(ba[j], bp[j]));
+                px[j] = pn;
+            }
         }
         // box and ramp projections, inner dual steps; the chunk's first hour reads the
         // previous lane's last p
