@@ -150,7 +150,7 @@ struct Sm {
     int4* busr;      // [N] generator rows, first line-end slot, first battery slot, counts (12, 12, 8 bits)
     float4* busf;    // [N] 1/terminals, 1/sum of phase weights, dual-residual weight
     int2* genr;      // [G] bus row offset, cost
-    int4* endr;      // [2L] line row offset, signed beta, phase weight
+    int4* endr;      // [2L + 1] line row offset, signed beta, phase weight; a zero entry
     int4* liner;     // [L] from / to bus row offsets, from / to end row offsets
     float4* linef;   // [L] beta, rho beta, rho_theta / 2, denominator
     float4* linec;   // [L] flow / angle cap, phase weight, 1 / denominator
@@ -603,7 +603,8 @@ __device__ __forceinline__ void res_bus(const Ctx& c, const Sm& m, float rho, in
     const int ng = br.w & 0xfff, ne = (br.w >> 12) & 0xfff, nb = (int)((unsigned)br.w >> 24);
     // The lists are walked in batches whose loads are all issued before the first sum, without
     // branches: an entry past a list's end reads the list's last one with factor 0 (an empty
-    // list reads the next bus's first), so the lanes of a warp stay together whatever their lengths.
+    // list the next bus's first, or the zero entry past the last), so the lanes of a warp stay
+    // together whatever their lengths.
     constexpr int kGB = kV == 4 ? 3 : 4, kEB = kV == 4 ? 2 : 4;
     const float* xg = m.xg + br.x + hl;
     const float* xbr = m.xb + br.z * HS + hl;
@@ -752,6 +753,12 @@ __global__ void __launch_bounds__(kCrsMaxThreads, 1)
         m.busf[n] = make_float4(c.bus_inv_cnt[nb], c.bus_inv_wsum[nb], c.bus_dres_w[nb], 0.f);
         for (int g = r.x; g < r1.x; ++g)
             m.genr[g] = make_int2(n * HS, __float_as_int(c.g_cost[sd.gen0 + R.gen[sd.gen0 + g]]));
+    }
+    // the entry past the last list is zero, and so are the rows that it leads to
+    if (tid == 0) m.endr[2 * L] = make_int4(0, 0, 0, 0);
+    for (int h = tid; h < HS; h += nt) {
+        m.q[2 * L * HS + h] = 0.f;
+        if (L == 0) m.dl[h] = 0.f;
     }
     for (int e = tid; e < 2 * L; e += nt) {
         const int code = R.end[2 * sd.line0 + e], lg = sd.line0 + (code >> 1);

@@ -124,7 +124,7 @@ struct CrsOff {
     size_t red, wred, xch, bar, flag, busr, busf, genr, endr, liner, linef, linec, bslot, batr, batg, idd, scan;
     size_t pbar, u, thb, xl, ld;  // [N][HS] bus-hours (ld: load, or the adjoint coefficient, NaN if fixed)
     size_t xg, cap;               // [G][HS] (cap: forward capacity, adjoint coefficient or NaN)
-    size_t dl, q;                 // [L][HS], [2L][HS] phase copies by end slot
+    size_t dl, q;                 // [max(L, 1)][HS], [2L + 1][HS] phase copies by end slot, one zero row
     size_t xb;                    // [B][HS]
     size_t vrow;                  // [nbo][TR] owned batteries' prox targets (then their new injections)
     size_t bst;                   // [nbo][6][T] owned batteries' state
@@ -150,17 +150,20 @@ __host__ __device__ inline CrsOff crs_offsets(int N, int G, int L, int B, int HS
     o.flag = crs_take(p, 16);
     o.busr = crs_take(p, 16 * (size_t)N); o.busf = crs_take(p, 16 * (size_t)N);
     o.genr = crs_take(p, 8 * (size_t)G);
-    o.endr = crs_take(p, 32 * (size_t)L + 16);  // (and one entry read past an empty last list)
+    o.endr = crs_take(p, 32 * (size_t)L + 16);  // (and a zero entry, read where the last lists are empty)
     o.liner = crs_take(p, 16 * (size_t)L); o.linef = crs_take(p, 16 * (size_t)L); o.linec = crs_take(p, 16 * (size_t)L);
     o.bslot = crs_take(p, 8 * (size_t)B);
     o.batr = crs_take(p, 32 * (size_t)nbo); o.batg = crs_take(p, 8 * (size_t)nbo);
     o.idd = crs_take(p, 4 * (size_t)dd_rows * T);
     o.scan = crs_take(p, 4 * (size_t)dd_rows * 12 * 32 * kw);
-    const size_t nb = (size_t)N * HS * 4, ng = (size_t)G * HS * 4, nl = (size_t)L * HS * 4;
+    const size_t nb = (size_t)N * HS * 4, ng = (size_t)G * HS * 4, row = (size_t)HS * 4;
     o.pbar = crs_take(p, nb); o.u = crs_take(p, nb); o.thb = crs_take(p, nb);
     o.xl = crs_take(p, nb); o.ld = crs_take(p, nb);
     o.xg = crs_take(p, ng); o.cap = crs_take(p, ng);
-    o.dl = crs_take(p, nl); o.q = crs_take(p, 2 * nl);
+    // The bus step reads the first batch of a list whatever its length: from an empty list at the end
+    // of the order the row past the line ends, row 0 of the lines, and the row past the generators
+    // (that of the next array).  Those rows are here even without lines or generators.
+    o.dl = crs_take(p, (L > 0 ? L : 1) * row); o.q = crs_take(p, (2 * (size_t)L + 1) * row);
     o.xb = crs_take(p, (size_t)B * HS * 4);
     o.vrow = crs_take(p, 4 * (size_t)nbo * crs_row(T));
     o.bst = crs_take(p, bat_smem ? (size_t)nbo * 6 * T * 4 : 0);
