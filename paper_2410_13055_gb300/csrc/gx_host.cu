@@ -15,7 +15,6 @@ using namespace gx;
 
 namespace {
 
-constexpr int kNoCluster = 1 << 16;  // weight in the active count of a scenario that fits no cluster
 constexpr int kCrsStreams = 8;  // launch groups of the resident path run side by side
 
 thread_local std::string g_err;
@@ -113,7 +112,7 @@ struct gx_network {
     std::vector<int2> crs_bat;
     std::vector<int> crs_gen, crs_end, crs_cls, crs_rep;
     std::vector<int> done_loop;        // done flags of the per-iteration loop (cluster-resident ones set)
-    bool actw_set = false;             // the scenarios' weights in the active count are in the workspace
+    bool nocl_set = false;             // the marks of the scenarios without a cluster are in the workspace
     int thr_dev = -1;                  // what the loop graphs' pause threshold in the workspace holds
     int use_crs = -1;                  // 1 on, 0 off, -1 not chosen: by rule (crs_active)
     cudaStream_t crs_streams[kCrsStreams] = {};
@@ -159,7 +158,7 @@ struct gx_network {
     int graph_next = 0;
     cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr, cap_stream3 = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
-    int* h_nact = nullptr;  // pinned: [0] active-scenario count, [1] iteration counter, [2] pause threshold
+    int* h_nact = nullptr;  // pinned: [0, 1] active-scenario counts, [2] iteration counter, [3] pause threshold
     int use_graphs = 2;     // 0 eager launches, 1 one graph per chunk, 2 the whole loop as one graph
     gx_schedule sched{1, 2};  // kernel schedule (gx_network_set_schedule)
     bool sched_set = false;   // the caller chose the schedule (else bind picks it by workspace size)
@@ -384,13 +383,12 @@ static void make_ctx(gx_network* net) {
 
 namespace gx {
 // Condition of the device-side loop (a conditional WHILE node around one residual-check
-// chunk): run another chunk while more than *pause scenarios are still iterating and the cap is
-// not reached (0: until all have stopped).
+// chunk): run another chunk unless the loop may stop or pause (loop_goes_on) or has reached its cap.
 // The reduction marks every scenario done once the counter reaches the cap, so the loop
 // ends after at most cap / chunk bodies.
 __global__ void k_loop_cond(const int* n_active, const int* iter_ctr, const int* pause, int max_it,
                             cudaGraphConditionalHandle h) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) cudaGraphSetConditional(h, (*n_active > *pause && *iter_ctr < max_it) ? 1u : 0u);
+    if (threadIdx.x == 0 && blockIdx.x == 0) cudaGraphSetConditional(h, (loop_goes_on(n_active, *pause) && *iter_ctr < max_it) ? 1u : 0u);
 }
 
 int launch_loop_cond(const Ctx& c, const int* pause, int max_it, cudaGraphConditionalHandle h, cudaStream_t st) {
@@ -1233,7 +1231,7 @@ gx_status gx_network_create(const gx_network_desc* nets, int n_nets, const gx_sc
     net->o_btpart = L.add(F4((long long)net->n_bat_warps * kDevPart));
     net->o_rpart = L.add(F4((long long)net->n_ramp_warps * kDevPart));
     net->o_cpart = L.add(D8(2LL * net->n_cost_blk));
-    net->o_nact = L.add(I4(1 + S));
+    net->o_nact = L.add(I4(2 + S));
     // the resident path's tables, uploaded by a copy of their own
     net->crs_begin = L.total;
     net->o_crbus = L.add(16 * std::max<size_t>(net->crs_bus.size(), 1));
@@ -1374,7 +1372,7 @@ gx_status gx_network_bind(gx_network* net, void* dev_mem, size_t bytes, void* st
     // clusters of C CTAs, one per SM, that the device holds at once
     net->crs_choices.clear();
     net->thr_dev = 0;  // (the workspace starts zeroed)
-    net->actw_set = false;
+    net->nocl_set = false;
     CrsShape probe;
     probe.threads = kCrsMaxThreads;
     for (int C = 1; C <= kCrsMaxC; ++C) {
@@ -1505,9 +1503,9 @@ static gx_status enqueue_iters(gx_network* net, const Ctx& c, int adj, int chunk
         *launches += nl + nb + nu;
     }
     if (reduce) {
-        GX_CUDA(cudaMemsetAsync(c.n_active, 0, sizeof(int), st));
+        GX_CUDA(cudaMemsetAsync(c.n_active, 0, 2 * sizeof(int), st));
         *launches += launch_reduce(c, adj, tol, st);
-        if (to_host) GX_CUDA(cudaMemcpyAsync(net->h_nact, c.n_active, sizeof(int), cudaMemcpyDeviceToHost, st));
+        if (to_host) GX_CUDA(cudaMemcpyAsync(net->h_nact, c.n_active, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
     }
     return GX_OK;
 }
@@ -1696,17 +1694,17 @@ static gx_status run_loop(gx_network* net, int adj, cudaStream_t st, int* launch
     if (it0 > 0) *launches += launch_tick(c, it0, st);
     if (net->use_graphs == 2 && max_it % every == 0) {
         if (net->thr_dev != pause_at) {
-            net->h_nact[2] = pause_at;
-            GX_CUDA(cudaMemcpyAsync(net->dev + net->o_thr, net->h_nact + 2, sizeof(int), cudaMemcpyHostToDevice, st));
+            net->h_nact[3] = pause_at;
+            GX_CUDA(cudaMemcpyAsync(net->dev + net->o_thr, net->h_nact + 3, sizeof(int), cudaMemcpyHostToDevice, st));
             net->thr_dev = pause_at;
         }
         cudaGraphExec_t exec = nullptr;
         if (gx_status e = loop_graph(net, c, adj, every, max_it, &exec)) return e;
         GX_CUDA(cudaGraphLaunch(exec, st));
-        GX_CUDA(cudaMemcpyAsync(net->h_nact + 1, c.iter_ctr, sizeof(int), cudaMemcpyDeviceToHost, st));
+        GX_CUDA(cudaMemcpyAsync(net->h_nact + 2, c.iter_ctr, sizeof(int), cudaMemcpyDeviceToHost, st));
         GX_CUDA(cudaGetLastError());
         GX_CUDA(cudaStreamSynchronize(st));
-        it = net->h_nact[1];
+        it = net->h_nact[2];
         // per body: tick, the iterations, the reduction and the condition kernel
         *launches += ((it - it0) / every) * (3 + every * per_it);
         *iters_out = it;
@@ -1735,7 +1733,7 @@ static gx_status run_loop(gx_network* net, int adj, cudaStream_t st, int* launch
         ++nch;
         GX_CUDA(cudaGetLastError());
         GX_CUDA(cudaStreamSynchronize(st));
-        if (*net->h_nact <= pause_at) break;
+        if (!loop_goes_on(net->h_nact, pause_at)) break;
     }
     *iters_out = it;
     if (net->prof) {
@@ -1786,13 +1784,12 @@ static gx_status iterate(gx_network* net, int adj, cudaStream_t st, int* launche
         if (gx_status e = still_active(net, st, act)) return e;
         if (act.empty() || it0 >= max_it) return GX_OK;
     }
-    if (!net->actw_set) {
-        std::vector<int> w(net->S, 1);
-        for (int s = 0; s < net->S; ++s)
-            if (crs_choices(net, s).empty()) w[s] = kNoCluster;
-        GX_CUDA(cudaMemcpyAsync(net->dev + net->o_nact + sizeof(int), w.data(), 4 * (size_t)net->S, cudaMemcpyHostToDevice, st));
+    if (!net->nocl_set) {
+        std::vector<int> w(net->S, 0);
+        for (int s = 0; s < net->S; ++s) w[s] = crs_choices(net, s).empty();
+        GX_CUDA(cudaMemcpyAsync(net->dev + net->o_nact + 2 * sizeof(int), w.data(), 4 * (size_t)net->S, cudaMemcpyHostToDevice, st));
         GX_CUDA(cudaStreamSynchronize(st));  // `w` is local
-        net->actw_set = true;
+        net->nocl_set = true;
     }
     std::vector<CrsShape> shapes;
     const bool asked = net->use_crs == 1;  // every scenario that fits a cluster runs in it
@@ -1824,8 +1821,8 @@ static gx_status iterate(gx_network* net, int adj, cudaStream_t st, int* launche
         double us = 0;
         if (n_fit == n) us = crs_assign(net, act, &shapes, &fits);
         if (!resident && !asked && !(fits && us < 0.95 * stream_cost(net, act))) {
-            // Pause once no scenario without a cluster is left (they count kNoCluster each) and as
-            // many others as fit for certain: the most for which the largest ones fit.
+            // Pause once no scenario without a cluster is left and as many others as fit for
+            // certain: the most for which the largest ones fit.
             std::vector<int> big;
             for (int s : act)
                 if (!crs_choices(net, s).empty()) big.push_back(s);

@@ -331,8 +331,7 @@ struct Ctx {
     int* iters;         // [S]
     int* status;        // [S]
     int* adj_iters;     // [S]
-    // [0] the scenarios still iterating, each with its weight, [1 + s] the weight of scenario s (0: 1)
-    int* n_active;
+    int* n_active;      // [0] scenarios still iterating, [1] those of them that fit no cluster, [2 + s] scenario s does not
     double* resid;      // [S*2]
     double* rbest;      // [S] smallest max(primal, dual) residual of the current solve
     double* cost;       // [S]
@@ -449,6 +448,14 @@ __device__ __forceinline__ void cost_share(const Ctx& c, const ScenDev& sc, long
             if ((int)(t0 + h) < sc.T) a += 0.5f * eps * fv[h] * fv[h];
         cs += (double)a;
     }
+}
+
+// Whether the per-iteration loop goes on after a residual check.  n_active: the scenarios still
+// iterating, and how many of them fit no cluster; pause: with at most that many left, and all of
+// those in clusters, the loop pauses (0: it runs until all have stopped).  (Two counts, not one with
+// a large weight for those without a cluster: 32,768 scenarios of weight 65,536 are -2^31.)
+__host__ __device__ inline bool loop_goes_on(const int* n_active, int pause) {
+    return n_active[0] > pause || n_active[1] > 0;
 }
 
 // want_res of an iteration's launches: the chunk's residual iteration, the one before it

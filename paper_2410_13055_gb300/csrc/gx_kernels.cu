@@ -1699,7 +1699,7 @@ __global__ void __launch_bounds__(kBlock) k_reduce(const Ctx c, int adj, double 
     if (c.prof_act != nullptr && threadIdx.x == 0) c.prof_act[s] += 1;
     const int it = *c.iter_ctr;
     const int final_ = it >= c.max_it;
-    const int weight = max(c.n_active[1 + s], 1);
+    const int no_cluster = c.n_active[2 + s];
     const ScenDev sc = c.scen[s];
     double a[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     for (int b = threadIdx.x; b < sc.bus4_nblk; b += kBlock) {
@@ -1767,7 +1767,8 @@ __global__ void __launch_bounds__(kBlock) k_reduce(const Ctx c, int adj, double 
             c.done[s] = 1;
             itp[s] = it;
         } else {
-            atomicAdd(c.n_active, weight);
+            atomicAdd(c.n_active, 1);
+            if (no_cluster) atomicAdd(c.n_active + 1, 1);
         }
     }
 }
