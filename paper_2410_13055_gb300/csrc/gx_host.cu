@@ -1,6 +1,7 @@
 // Host side of the C ABI (include/gx.h): descriptor validation, workspace layout,
 // bind (upload of static data), and the drivers of the solve, gradient and plan step.
 #include "gx_internal.cuh"
+#include "gx_paths.h"
 
 #include <algorithm>
 #include <cmath>
@@ -100,19 +101,17 @@ struct gx_network {
     std::vector<int2> sc_pool, sc_dres_l;
     std::vector<ScaleDres> sc_dres, sc_dres_pool;  // bus_dres_w targets; pool-word targets
     // cluster-resident solver: the launch shapes a scenario can take, by (network, horizon)
-    struct CrsChoice {
-        CrsShape shape;
-        double us = 0;    // estimated time per iteration
-        double room = 0;  // share of the device one such cluster takes
-    };
     std::map<std::pair<int, int>, std::vector<CrsChoice>> crs_choices;
+    std::map<std::tuple<int, int, int, int>, bool> crs_ready;  // kernel instances asked for at bind: launchable
+    std::vector<const std::vector<CrsChoice>*> crs_of;  // per scenario: its choices
+    std::vector<double> crs_dh;                         // per scenario: its device-hours
+    std::vector<int> crs_by_room, crs_by_us;  // scenarios that have choices, by their smallest cluster's room / time, descending
     int crs_clusters[kCrsMaxC + 1] = {};  // clusters of C whole-SM CTAs the device holds (set at bind)
     std::vector<int4> crs_bus, crs_line;
     CrsTables crs_tables{};            // their places in the workspace
     std::vector<int2> crs_bat;
     std::vector<int> crs_gen, crs_end, crs_cls, crs_rep;
     std::vector<int> done_loop;        // done flags of the per-iteration loop (cluster-resident ones set)
-    bool nocl_set = false;             // the marks of the scenarios without a cluster are in the workspace
     int thr_dev = -1;                  // what the loop graphs' pause threshold in the workspace holds
     int use_crs = -1;                  // 1 on, 0 off, -1 not chosen: by rule (crs_active)
     cudaStream_t crs_streams[kCrsStreams] = {};
@@ -580,16 +579,16 @@ static double crs_cost(const ScenDev& sd, const CrsShape& p) {
 // ascending, those that gain nothing over a smaller one left out.  Empty: the scenario runs on
 // the per-iteration kernels only.  Battery lanes are split as in the battery kernel (two warps
 // where the batch's longest horizon exceeds 96 hours).
-static const std::vector<gx_network::CrsChoice>& crs_choices(gx_network* net, int s) {
+static const std::vector<CrsChoice>& crs_choices(gx_network* net, int s) {
     const ScenDev& sd = net->sdev[s];
     const auto key = std::make_pair(sd.net, sd.T);
     const auto it = net->crs_choices.find(key);
     if (it != net->crs_choices.end()) return it->second;
-    std::vector<gx_network::CrsChoice>& out = net->crs_choices[key];
+    std::vector<CrsChoice>& out = net->crs_choices[key];
     // ramping generators run on the per-iteration kernels; a bus's counts are 12 and 8 bits
     if (sd.R > 0 || !net->nets[sd.net].crs_ok) return out;
     for (int C = 1; C <= kCrsMaxC; ++C) {
-        gx_network::CrsChoice best;
+        CrsChoice best;
         if (net->crs_clusters[C] < 1) continue;
         for (int V : {4, 1}) {
             if (crs_hours(sd.T, C, V) * (C - 1) >= sd.T) continue;  // an empty rank
@@ -609,7 +608,7 @@ static const std::vector<gx_network::CrsChoice>& crs_choices(gx_network* net, in
                     }
                 const size_t image = std::max(p.smem[0], p.smem[1]);
                 if (image > kCrsSmemMax) continue;
-                gx_network::CrsChoice ch;
+                CrsChoice ch;
                 ch.shape = p;
                 ch.us = crs_cost(sd, p);
                 // CTAs that share an SM: its registers (96 per thread) and shared memory
@@ -619,53 +618,53 @@ static const std::vector<gx_network::CrsChoice>& crs_choices(gx_network* net, in
             }
         }
         if (!best.shape.C || (!out.empty() && best.us > 0.97 * out.back().us)) continue;
-        bool ok = true;
-        for (int adj = 0; adj < 2 && ok; ++adj) ok = crs_prepare(adj, best.shape) == cudaSuccess;
-        cudaGetLastError();
-        if (ok) out.push_back(best);
+        const CrsShape& p = best.shape;
+        const auto ready = net->crs_ready.emplace(std::make_tuple(p.V, p.kw, p.hpl, p.reg), true);
+        if (ready.second) {
+            for (int adj = 0; adj < 2; ++adj) ready.first->second &= crs_prepare(adj, p) == cudaSuccess;
+            cudaGetLastError();
+        }
+        if (ready.first->second) out.push_back(best);
     }
     return out;
 }
 
-// Launch shapes for the scenarios `act`, all of which have choices: each starts from its
-// smallest cluster, then the slowest is enlarged while the device still holds all of them side by
-// side (scenarios of one size take one cluster size).  Returns the estimated time per iteration, that
-// of the slowest; *fits: whether the smallest clusters already fit side by side.
-static double crs_assign(gx_network* net, const std::vector<int>& act, std::vector<CrsShape>* shapes, bool* fits) {
-    const size_t n = act.size();
-    std::vector<const std::vector<gx_network::CrsChoice>*> ch(n);
-    std::vector<size_t> at(n, 0);
-    double room = 0;
-    bool one = true;
-    for (size_t i = 0; i < n; ++i) {
-        ch[i] = &crs_choices(net, act[i]);
-        one = one && ch[i] == ch[0];
-        room += (*ch[i])[0].room;
+// The launch choices of every scenario, and the orders that the searches before a loop need, once
+// per bind.
+static void build_crs_choices(gx_network* net) {
+    net->crs_choices.clear();
+    net->crs_ready.clear();
+    net->crs_of.resize(net->S);
+    net->crs_dh.resize(net->S);
+    net->crs_by_room.clear();
+    for (int s = 0; s < net->S; ++s) {
+        const ScenDev& sd = net->sdev[s];
+        net->crs_of[s] = &crs_choices(net, s);
+        net->crs_dh[s] = (double)sd.T * (sd.N + sd.G + sd.L + sd.B);
+        if (!net->crs_of[s]->empty()) net->crs_by_room.push_back(s);
     }
-    // clusters of mixed sizes leave gaps in the processing clusters that hold them
-    const double limit = one ? 1.0 + 1e-9 : 0.9;
-    *fits = room <= limit;
-    if (one) {
-        for (size_t k = 1; k < ch[0]->size(); ++k)
-            if ((double)n * (*ch[0])[k].room <= limit) std::fill(at.begin(), at.end(), k);
-    } else if (*fits) {
-        for (;;) {
-            size_t w = 0;
-            for (size_t i = 1; i < n; ++i)
-                if ((*ch[i])[at[i]].us > (*ch[w])[at[w]].us) w = i;
-            if (at[w] + 1 >= ch[w]->size()) break;
-            const double more = (*ch[w])[at[w] + 1].room - (*ch[w])[at[w]].room;
-            if (room + more > limit) break;
-            room += more;
-            ++at[w];
-        }
-    }
-    double us = 0;
-    if (shapes) shapes->resize(n);
-    for (size_t i = 0; i < n; ++i) {
-        us = std::max(us, (*ch[i])[at[i]].us);
-        if (shapes) (*shapes)[i] = (*ch[i])[at[i]].shape;
-    }
+    net->crs_by_us = net->crs_by_room;
+    const auto& of = net->crs_of;
+    std::stable_sort(net->crs_by_room.begin(), net->crs_by_room.end(),
+                     [&](int a, int b) { return of[a]->front().room > of[b]->front().room; });
+    std::stable_sort(net->crs_by_us.begin(), net->crs_by_us.end(),
+                     [&](int a, int b) { return of[a]->front().us > of[b]->front().us; });
+}
+
+static std::vector<const std::vector<CrsChoice>*> crs_lists(const gx_network* net, const std::vector<int>& scen) {
+    std::vector<const std::vector<CrsChoice>*> ch;
+    ch.reserve(scen.size());
+    for (int s : scen) ch.push_back(net->crs_of[s]);
+    return ch;
+}
+
+// Launch shapes for the scenarios `act` (crs_assign); returns the estimated time per iteration.
+static double crs_shapes(const gx_network* net, const std::vector<int>& act, std::vector<CrsShape>* shapes, bool* fits) {
+    const auto ch = crs_lists(net, act);
+    std::vector<size_t> at;
+    const double us = crs_assign(ch, act.size(), at, fits);
+    shapes->resize(act.size());
+    for (size_t i = 0; i < act.size(); ++i) (*shapes)[i] = (*ch[i])[at[i]].shape;
     return us;
 }
 
@@ -1370,9 +1369,7 @@ gx_status gx_network_bind(gx_network* net, void* dev_mem, size_t bytes, void* st
     }
     make_ctx(net);
     // clusters of C CTAs, one per SM, that the device holds at once
-    net->crs_choices.clear();
     net->thr_dev = 0;  // (the workspace starts zeroed)
-    net->nocl_set = false;
     CrsShape probe;
     probe.threads = kCrsMaxThreads;
     for (int C = 1; C <= kCrsMaxC; ++C) {
@@ -1380,6 +1377,11 @@ gx_status gx_network_bind(gx_network* net, void* dev_mem, size_t bytes, void* st
         net->crs_clusters[C] = crs_prepare(0, probe) == cudaSuccess ? crs_max_clusters(0, probe, 200 * 1024) : 0;
     }
     cudaGetLastError();
+    build_crs_choices(net);
+    std::vector<int> none(net->S);  // marks of the scenarios without a cluster
+    for (int s = 0; s < net->S; ++s) none[s] = net->crs_of[s]->empty();
+    GX_CUDA(cudaMemcpyAsync(net->dev + net->o_nact + 2 * sizeof(int), none.data(), 4 * (size_t)net->S, cudaMemcpyHostToDevice, st));
+    GX_CUDA(cudaStreamSynchronize(st));  // (`none` is local)
     net->solved = false;
     net->adj_ready = false;
     return GX_OK;
@@ -1757,13 +1759,14 @@ static gx_status still_active(gx_network* net, cudaStream_t st, std::vector<int>
     return GX_OK;
 }
 
-// Estimated microseconds of one iteration of the per-iteration kernels with `act` iterating: three
-// dependent launches (10 to 11 us for one scenario of any size here), then 3.3 to 3.6 us per million
-// device-hours (100 buses, 168 h: 10.9 us for 2 scenarios, 15.4 for 16).
-static double stream_cost(const gx_network* net, const std::vector<int>& act) {
-    double dh = 0;
-    for (int s : act) dh += (double)net->sdev[s].T * (net->sdev[s].N + net->sdev[s].G + net->sdev[s].L + net->sdev[s].B);
-    return 10.0 + 3.5e-6 * dh;
+// Of the order `by`, the scenarios of `act`.
+static std::vector<int> crs_sorted(const gx_network* net, const std::vector<int>& by, const std::vector<int>& act) {
+    std::vector<char> in(net->S, 0);
+    for (int s : act) in[s] = 1;
+    std::vector<int> out;
+    for (int s : by)
+        if (in[s]) out.push_back(s);
+    return out;
 }
 
 // Iterate the batch's scenarios to their stops on whichever path is estimated faster for those
@@ -1784,28 +1787,21 @@ static gx_status iterate(gx_network* net, int adj, cudaStream_t st, int* launche
         if (gx_status e = still_active(net, st, act)) return e;
         if (act.empty() || it0 >= max_it) return GX_OK;
     }
-    if (!net->nocl_set) {
-        std::vector<int> w(net->S, 0);
-        for (int s = 0; s < net->S; ++s) w[s] = crs_choices(net, s).empty();
-        GX_CUDA(cudaMemcpyAsync(net->dev + net->o_nact + 2 * sizeof(int), w.data(), 4 * (size_t)net->S, cudaMemcpyHostToDevice, st));
-        GX_CUDA(cudaStreamSynchronize(st));  // `w` is local
-        net->nocl_set = true;
-    }
     std::vector<CrsShape> shapes;
     const bool asked = net->use_crs == 1;  // every scenario that fits a cluster runs in it
     if (asked) {
         std::vector<int> res;
         for (int s : act)
-            if (!crs_choices(net, s).empty()) res.push_back(s);
+            if (!net->crs_of[s]->empty()) res.push_back(s);
         const bool mixed = res.size() < act.size();
         if (res.empty() || (mixed && it0 > 0)) return run_loop(net, adj, st, launches, &it, it0);
         if (mixed) {  // the others on the per-iteration kernels beside them
             net->done_loop.assign(net->S, 1);
             for (int s : act)
-                if (crs_choices(net, s).empty()) net->done_loop[s] = 0;
+                if (net->crs_of[s]->empty()) net->done_loop[s] = 0;
             GX_CUDA(cudaMemcpyAsync(net->dev + net->o_done, net->done_loop.data(), 4 * net->S, cudaMemcpyHostToDevice, st));
             bool fits;
-            crs_assign(net, res, &shapes, &fits);
+            crs_shapes(net, res, &shapes, &fits);
             if (gx_status e = crs_launch(net, adj, res, shapes, it0, 0, false, st, launches, &used)) return e;
             const gx_status le = run_loop(net, adj, st, launches, &it, it0);
             if (gx_status e = crs_wait(net, used, st)) return e;
@@ -1816,23 +1812,21 @@ static gx_status iterate(gx_network* net, int adj, cudaStream_t st, int* launche
     for (;;) {
         const int n = (int)act.size();
         int n_fit = 0;
-        for (int s : act) n_fit += !crs_choices(net, s).empty();
+        double dh = 0;
+        for (int s : act) {
+            n_fit += !net->crs_of[s]->empty();
+            dh += net->crs_dh[s];
+        }
         bool fits = false;
         double us = 0;
-        if (n_fit == n) us = crs_assign(net, act, &shapes, &fits);
-        if (!resident && !asked && !(fits && us < 0.95 * stream_cost(net, act))) {
+        if (n_fit == n) us = crs_shapes(net, act, &shapes, &fits);
+        if (!resident && !asked && !(fits && us < 0.95 * stream_us(dh))) {
             // Pause once no scenario without a cluster is left and as many others as fit for
             // certain: the most for which the largest ones fit.
-            std::vector<int> big;
-            for (int s : act)
-                if (!crs_choices(net, s).empty()) big.push_back(s);
-            std::sort(big.begin(), big.end(), [&](int a, int b) { return crs_choices(net, a)[0].room > crs_choices(net, b)[0].room; });
-            int pause_at = 0;
-            for (size_t k = std::min<size_t>(big.size(), (size_t)n - 1); k >= 1 && pause_at == 0; --k) {
-                big.resize(k);
-                bool f;
-                if (crs_assign(net, big, nullptr, &f) < 0.95 * stream_cost(net, big) && f) pause_at = (int)k;
-            }
+            const std::vector<int> big = crs_sorted(net, net->crs_by_room, act);
+            std::vector<double> big_dh;
+            for (int s : big) big_dh.push_back(net->crs_dh[s]);
+            const int pause_at = (int)crs_pause_at(crs_lists(net, big), big_dh, (size_t)n - 1);
             if (gx_status e = run_loop(net, adj, st, launches, &it, it, pause_at)) return e;
             if (pause_at == 0 || it >= max_it) return GX_OK;
             if (gx_status e = still_active(net, st, act)) return e;
@@ -1841,14 +1835,7 @@ static gx_status iterate(gx_network* net, int adj, cudaStream_t st, int* launche
         }
         // the largest count of remaining scenarios at which larger clusters pay for the pause
         // (estimated on the slowest of them, for whichever remain)
-        int pause_at = 0;
-        std::vector<int> big = act;
-        std::sort(big.begin(), big.end(), [&](int a, int b) { return crs_choices(net, a)[0].us > crs_choices(net, b)[0].us; });
-        for (int k = net->prof ? 0 : n - 1; k >= 1 && pause_at == 0; k = k > 8 ? k * 7 / 8 : k - 1) {
-            big.resize(k);
-            bool f;
-            if (crs_assign(net, big, nullptr, &f) < 0.9 * us && f) pause_at = k;
-        }
+        const int pause_at = net->prof ? 0 : (int)crs_regroup_at(crs_lists(net, crs_sorted(net, net->crs_by_us, act)), us);
         if (gx_status e = crs_launch(net, adj, act, shapes, resident ? -1 : it, pause_at, true, st, launches, &used)) return e;
         if (gx_status e = crs_wait(net, used, st)) return e;
         if (pause_at == 0) return GX_OK;
@@ -2166,13 +2153,12 @@ gx_status gx_network_persistent_info(const gx_network* net, int scen, int* clust
     if (scen < 0 || scen >= net->S) return fail(GX_ERR_INVALID_ARG, "scenario out of range");
     *cluster_ctas = 0;
     if (!net->dev || !crs_active(net)) return GX_OK;
-    gx_network* nn = const_cast<gx_network*>(net);  // (the shapes are worked out on first use)
     std::vector<int> fit;
     for (int s = 0; s < net->S; ++s)
-        if (!crs_choices(nn, s).empty()) fit.push_back(s);
+        if (!net->crs_of[s]->empty()) fit.push_back(s);
     std::vector<CrsShape> shapes;
     bool fits;
-    if (!fit.empty()) crs_assign(nn, fit, &shapes, &fits);
+    crs_shapes(net, fit, &shapes, &fits);
     for (size_t i = 0; i < fit.size(); ++i)
         if (fit[i] == scen) *cluster_ctas = shapes[i].C;
     return GX_OK;

@@ -100,6 +100,13 @@ struct CrsShape {
     size_t smem[2] = {0, 0};
 };
 
+// One of a scenario's ways to run on the resident path.
+struct CrsChoice {
+    CrsShape shape;
+    double us = 0;    // estimated time per iteration
+    double room = 0;  // share of the device one such cluster takes
+};
+
 // Static tables of the resident path, per network (concatenated over networks): buses sorted
 // by device count, and the devices renumbered so that a bus's are consecutive.
 struct CrsTables {
