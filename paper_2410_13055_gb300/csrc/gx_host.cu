@@ -595,8 +595,10 @@ static const std::vector<CrsChoice>& crs_choices(gx_network* net, int s) {
             for (int threads : {128, 256, 384, 512, 640}) {
                 CrsShape p;
                 p.C = C; p.V = V; p.threads = threads;
-                p.kw = net->ctx.max_bat_T > 96 && sd.T > 32 ? 2 : 1;
-                p.hpl = (sd.T + 32 * p.kw - 1) / (32 * p.kw);
+                if (sd.B > 0) {  // (without batteries no horizon is too long)
+                    p.kw = net->ctx.max_bat_T > 96 && sd.T > 32 ? 2 : 1;
+                    p.hpl = (sd.T + 32 * p.kw - 1) / (32 * p.kw);
+                }
                 if (p.hpl > 3) continue;
                 const int HS = crs_hours(sd.T, C, V), nbo = (sd.B + C - 1) / C;
                 p.reg = p.kw == 2 && nbo * 64 <= threads;

@@ -1,0 +1,34 @@
+"""Which horizons the cluster-resident loops take: any without batteries, up to 192 hours with them
+by the library's choice."""
+import numpy as np
+import pytest
+
+from gpu_util import eta_tensor, gpu_net
+from paper_2410_13055_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(net, sc, persistent):
+    import torch
+    h = gpu_net([net], sc, kappa=50.0, tol=1e-4, adj_tol=1e-4, max_iter=400, adj_max_iter=400, check_every=20)
+    if persistent is not None:
+        h.use_persistent(persistent)
+    e = eta_tensor(net["eta_min"] * 1.05)
+    h.solve(e)
+    g = h.grad(e).clone()
+    torch.cuda.synchronize()
+    return h, [h.state(False), h.state(True), g, h.array("iters"), h.array("adj_iters")]
+
+
+@pytest.mark.parametrize("T", [97, 200, 256])
+@pytest.mark.parametrize("S", [1, 3])
+def test_long_horizons_without_batteries_take_clusters_bitwise(T, S):
+    import torch
+    net, sc = synth.custom(12, 18, 30, 0, T, S=S, seed=T)
+    _, a = _run(net, sc, False)
+    for persistent in (None, True):
+        h, b = _run(net, sc, persistent)
+        assert min(h.persistent_info()) > 0
+        for k, (x, y) in enumerate(zip(a, b)):
+            assert torch.equal(x, y), (persistent, k)
