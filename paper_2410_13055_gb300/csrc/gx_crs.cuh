@@ -38,7 +38,8 @@
 //
 // The arithmetic of every step is that of the per-iteration kernels (gx_kernels.cu), in the same
 // order, so a scenario takes bitwise the same iterates on either path; only the residual
-// partials are summed in another order (FP32 within a thread's items, then FP64 over CTAs).
+// partials are summed in another order: FP32 within an item (at most four hours of a device or bus),
+// pairs of floats over a thread's items and a warp's lanes (about 48 bits), FP64 from there on.
 // State is read from and written back to the workspace rows at entry and exit, so the reset,
 // mask, extraction and gradient kernels work unchanged.
 #pragma once
@@ -56,12 +57,6 @@ namespace gx {
 namespace {
 
 __device__ __forceinline__ float clampf(float x, float lo, float hi) { return fminf(fmaxf(x, lo), hi); }
-
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
 
 // ---------------------------------------------------------------- cluster primitives
 __device__ __forceinline__ unsigned map_rank(unsigned a, int rank) {
@@ -136,6 +131,43 @@ __device__ __forceinline__ float quotient(float a, float b, float r) {
     return __fmaf_rn(__fmaf_rn(-b, q, a), r, q);
 }
 
+// A residual sum: the rounding errors of hi, each exact (Knuth's two-sum), are summed in lo.  Most
+// of a scenario's terms meet in one CTA, so plain FP32 sums would round some 40 times on the way to
+// the total where the per-iteration kernels go to FP64 after 128 threads; and the dual residual's
+// device and bus parts, which cancel, are two sums here.
+struct Sum2 {
+    float hi, lo;
+    __device__ __forceinline__ void add(float v) {
+        const float s = __fadd_rn(hi, v), b = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(v, b)));
+        hi = s;
+    }
+    __device__ __forceinline__ void add(float h, float l) {
+        add(h);
+        lo = __fadd_rn(lo, l);
+    }
+};
+
+// The warp's total of sum q, in lanes 2 q and 2 q + 1: each step halves the sums that a lane carries.
+__device__ __forceinline__ Sum2 warp_sums(const Sum2 (&acc)[9], int lane) {
+    Sum2 v[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) v[q] = q < 9 ? acc[q < 9 ? q : 0] : Sum2{0.f, 0.f};
+#pragma unroll
+    for (int n = 8; n >= 1; n >>= 1) {
+        const int bit = 2 * n;
+        const bool up = lane & bit;
+#pragma unroll
+        for (int q = 0; q < n; ++q) {
+            const Sum2 out = up ? v[q] : v[q + n];
+            if (up) v[q] = v[q + n];
+            v[q].add(__shfl_xor_sync(0xffffffffu, out.hi, bit), __shfl_xor_sync(0xffffffffu, out.lo, bit));
+        }
+    }
+    v[0].add(__shfl_xor_sync(0xffffffffu, v[0].hi, 1), __shfl_xor_sync(0xffffffffu, v[0].lo, 1));
+    return v[0];
+}
+
 struct GState {
     float *xg, *xl, *dl, *sg, *vf, *vt, *xb, *zc, *u, *pbar, *thb;
     long long zstride;  // zc, zd, zs, yc, yd, ys lie this many floats apart
@@ -143,7 +175,7 @@ struct GState {
 
 struct Sm {
     double* red;     // [2][C][kCrsRed] residual partials of every rank (two chunks' slots)
-    float* wred;     // [warps][kCrsRed]
+    double* wred;    // [warps][kCrsRed]
     float* xch;      // [warps][8] two-warp exchange of the battery prox
     unsigned long long* bar;  // [0] battery injections have arrived, [1] prox targets have arrived
     int* flag;       // [0] stop, [1] a bounded wait gave up, [2] this rank's marks at a residual check
@@ -166,7 +198,7 @@ struct Sm {
 __device__ __forceinline__ Sm sm_at(unsigned char* b, const CrsOff& o) {
     Sm m;
     m.red = reinterpret_cast<double*>(b + o.red);
-    m.wred = reinterpret_cast<float*>(b + o.wred);
+    m.wred = reinterpret_cast<double*>(b + o.wred);
     m.xch = reinterpret_cast<float*>(b + o.xch);
     m.bar = reinterpret_cast<unsigned long long*>(b + o.bar);
     m.flag = reinterpret_cast<int*>(b + o.flag);
@@ -231,7 +263,7 @@ __device__ __forceinline__ void res_battery(const Ctx& c, const Sm& m, const Bat
                                             const unsigned (&qa)[kV == 4 ? 1 : kHpl],
                                             const unsigned (&qb)[kV == 4 ? 1 : kHpl], int slot, int group,
                                             float (&s6)[6][kHpl], float* st, long long sstride, long long row0,
-                                            float& dx2_acc, float& x2_acc) {
+                                            Sum2 (&acc)[9]) {
     constexpr int NL = 32 * kW;
     const int Lx = threadIdx.x & (NL - 1);
     const int lane = Lx & 31, wb = Lx >> 5;
@@ -416,14 +448,17 @@ __device__ __forceinline__ void res_battery(const Ctx& c, const Sm& m, const Bat
                 for (int r = 0; r < 6; ++r) st[r * sstride + t0 + j] = s6[r][j];
     float* xl = m.xb + br.x;  // local row of the battery's injections (multi: this rank's hours)
     if (WANT) {
+        float dx2 = 0.f, x2 = 0.f;
 #pragma unroll
         for (int j = 0; j < kHpl; ++j) {
             if (j >= nv) continue;
             const int t = t0 + j, rk = t / HS;
             const float old = multi ? ld_cluster(map_rank(smem_addr(xl + (t - rk * HS)), rk)) : xl[t];
-            dx2_acc += (xn[j] - old) * (xn[j] - old);
-            x2_acc += xn[j] * xn[j];
+            dx2 += (xn[j] - old) * (xn[j] - old);
+            x2 += xn[j] * xn[j];
         }
+        acc[6].add(dx2);
+        acc[7].add(x2);
         sync();  // every lane has read the old injections before a lane of another order sends new ones
     }
     if (!multi) {
@@ -474,7 +509,8 @@ __device__ __forceinline__ void res_scan_table(const float* ird, float* sc, int 
 // and in the residual iteration.
 template <int WANT, int ADJ, int kV>
 __device__ __forceinline__ void res_line(const Ctx& c, const Sm& m, float* sg, long long row, int HS, int l, int hq,
-                                         int store_sg, float (&acc)[9]) {
+                                         int store_sg, Sum2 (&acc)[9]) {
+    float dx2 = 0.f, x2 = 0.f, th2 = 0.f;
     const int hl = hq * kV;
     const int4 lr = m.liner[l];
     const float4 lf = m.linef[l];
@@ -501,7 +537,7 @@ __device__ __forceinline__ void res_line(const Ctx& c, const Sm& m, float* sg, l
         const float vf = qf[h] - zf[h], vt = qt[h] - zt[h];
         if (WANT && !dc) {
             const float ef = 0.5f * (g[h] + d[h]) - zf[h], et = 0.5f * (g[h] - d[h]) - zt[h];
-            acc[8] += beta * beta * (ef * ef + et * et);
+            th2 += beta * beta * (ef * ef + et * et);
         }
         const float wf = zf[h] - vf, wt = zt[h] - vt;
         const float tf = __fsub_rn(__fmaf_rn(-beta, d[h], -pbf[h]), uf[h]);
@@ -516,9 +552,14 @@ __device__ __forceinline__ void res_line(const Ctx& c, const Sm& m, float* sg, l
         nt[h] = __fmaf_rn(0.5f, __fsub_rn(gn[h], dn[h]), vt);
         if (WANT) {
             const float dd = dn[h] - d[h];
-            acc[6] += 2.f * beta * beta * dd * dd;
-            acc[7] += 2.f * beta * beta * dn[h] * dn[h];
+            dx2 += 2.f * beta * beta * dd * dd;
+            x2 += 2.f * beta * beta * dn[h] * dn[h];
         }
+    }
+    if (WANT) {
+        acc[6].add(dx2);
+        acc[7].add(x2);
+        acc[8].add(th2);
     }
     stv<kV>(pd, dn); stv<kV>(pqf, nf); stv<kV>(pqt, nt);
     if (WANT || store_sg) stv<kV>(sg + gr, gn);
@@ -526,7 +567,8 @@ __device__ __forceinline__ void res_line(const Ctx& c, const Sm& m, float* sg, l
 
 // One generator item: clip (forward) or masked step (adjoint).
 template <int WANT, int ADJ, int kV>
-__device__ __forceinline__ void res_gen(const Sm& m, float rho, float inv_re, int HS, int g, int hl, float (&acc)[9]) {
+__device__ __forceinline__ void res_gen(const Sm& m, float rho, float inv_re, int HS, int g, int hl, Sum2 (&acc)[9]) {
+    float dx2 = 0.f, x2 = 0.f, scale = 0.f;
     const int2 gr = m.genr[g];
     const float cost = __int_as_float(gr.y);
     float x[kV], a[kV], pb[kV], uu[kV], xn[kV];
@@ -540,21 +582,27 @@ __device__ __forceinline__ void res_gen(const Sm& m, float rho, float inv_re, in
             const float gh = a[h];  // NaN: bound active, the variable is fixed at 0
             const bool fixed = gh != gh;
             xn[h] = fixed ? 0.f : __fmul_rn(__fmaf_rn(rho, v, gh), inv_re);
-            if (WANT && !fixed) acc[1] += (gh * inv_re) * (gh * inv_re);
+            if (WANT && !fixed) scale += (gh * inv_re) * (gh * inv_re);
         } else {
             xn[h] = clampf(__fmul_rn(__fmaf_rn(rho, v, -cost), inv_re), 0.f, a[h]);
         }
         if (WANT) {
-            acc[2] += (xn[h] - x[h]) * (xn[h] - x[h]);
-            acc[5] += xn[h] * xn[h];
+            dx2 += (xn[h] - x[h]) * (xn[h] - x[h]);
+            x2 += xn[h] * xn[h];
         }
+    }
+    if (WANT) {
+        if (ADJ) acc[1].add(scale);
+        acc[2].add(dx2);
+        acc[5].add(x2);
     }
     stv<kV>(px, xn);
 }
 
 // One load item (shed variable; terminal injection shed - L).
 template <int WANT, int ADJ, int kV>
-__device__ __forceinline__ void res_load(const Sm& m, float rho, float inv_re, float voll, int i, float (&acc)[9]) {
+__device__ __forceinline__ void res_load(const Sm& m, float rho, float inv_re, float voll, int i, Sum2 (&acc)[9]) {
+    float dx2 = 0.f, x2 = 0.f, scale = 0.f;
     float x[kV], Ld[kV], pb[kV], uu[kV], xn[kV];
     ldv<kV>(m.xl + i, x); ldv<kV>(m.ld + i, Ld); ldv<kV>(m.pbar + i, pb); ldv<kV>(m.u + i, uu);
 #pragma unroll
@@ -564,14 +612,19 @@ __device__ __forceinline__ void res_load(const Sm& m, float rho, float inv_re, f
             const float gsh = Ld[h];  // adjoint coefficient; NaN: bound active
             const bool fixed = gsh != gsh;
             xn[h] = fixed ? 0.f : __fmul_rn(__fmaf_rn(rho, v, gsh), inv_re);
-            if (WANT && !fixed) acc[1] += (gsh * inv_re) * (gsh * inv_re);
+            if (WANT && !fixed) scale += (gsh * inv_re) * (gsh * inv_re);
         } else {
             xn[h] = clampf(__fmul_rn(__fmaf_rn(rho, __fadd_rn(v, Ld[h]), -voll), inv_re), 0.f, Ld[h]) - Ld[h];
         }
         if (WANT) {
-            acc[2] += (xn[h] - x[h]) * (xn[h] - x[h]);
-            acc[5] += xn[h] * xn[h];
+            dx2 += (xn[h] - x[h]) * (xn[h] - x[h]);
+            x2 += xn[h] * xn[h];
         }
+    }
+    if (WANT) {
+        if (ADJ) acc[1].add(scale);
+        acc[2].add(dx2);
+        acc[5].add(x2);
     }
     stv<kV>(m.xl + i, xn);
 }
@@ -596,7 +649,7 @@ __device__ __forceinline__ void push_targets(const Sm& m, int HS, int t, bool mu
 // kernels' order), then the consensus and the dual update.
 template <int WANT, int kV>
 __device__ __forceinline__ void res_bus(const Ctx& c, const Sm& m, float rho, int HS, int n, int hl, int t, bool multi,
-                                        float (&acc)[9]) {
+                                        Sum2 (&acc)[9]) {
     const int i = n * HS + hl;
     const int4 br = m.busr[n];
     const float4 bf = m.busf[n];
@@ -684,18 +737,23 @@ __device__ __forceinline__ void res_bus(const Ctx& c, const Sm& m, float rho, in
     }
     if (WANT) {
         const float cnt = 1.f / bf.x;
+        float p2 = 0.f, dp2 = 0.f, dth2 = 0.f, u2 = 0.f;
         float pb[kV], th[kV];
         ldv<kV>(m.pbar + i, pb);
         ldv<kV>(m.thb + i, th);
 #pragma unroll
         for (int h = 0; h < kV; ++h) {
             const float dpb = pbn[h] - pb[h];
-            acc[0] += cnt * pbn[h] * pbn[h];
-            acc[2] -= cnt * dpb * dpb;
-            acc[3] += (thn[h] - th[h]) * (thn[h] - th[h]) * bf.z;
-            acc[4] += cnt * (rho * un[h]) * (rho * un[h]);
+            p2 += cnt * pbn[h] * pbn[h];
+            dp2 += cnt * dpb * dpb;
+            dth2 += (thn[h] - th[h]) * (thn[h] - th[h]) * bf.z;
+            u2 += cnt * (rho * un[h]) * (rho * un[h]);
         }
-        acc[5] += x2;
+        acc[0].add(p2);
+        acc[2].add(-dp2);
+        acc[3].add(dth2);
+        acc[4].add(u2);
+        acc[5].add(x2);
     }
     push_targets<kV>(m, HS, t, multi, br.z, nb, xbr, pbn, un);
     stv<kV>(m.pbar + i, pbn);
@@ -923,7 +981,7 @@ __global__ void __launch_bounds__(kCrsMaxThreads, 1)
     int it = it0, slot = 0;
     unsigned ph = 0;  // iterations of this launch: the barriers' phases
     double best = it0 > 0 ? c.rbest[s] : 0.0;
-    auto iterate = [&](auto want_c, int store_sg, float (&acc)[9]) {
+    auto iterate = [&](auto want_c, int store_sg, Sum2 (&acc)[9]) {
         constexpr int W = decltype(want_c)::value;
         if (tid == 0 && wait_x) mbar_expect_tx(m.bar, bytes_x);
         // A: batteries first (the longest chain), then chunks of the other devices
@@ -934,7 +992,7 @@ __global__ void __launch_bounds__(kCrsMaxThreads, 1)
                 const long long row0 = sd.e_bat + (long long)(rank + j * C) * sd.Tp;
                 float* st = bat_smem ? m.bst + (size_t)j * 6 * T : X.zc + row0;
                 res_battery<W, ADJ, kHpl, kW, kV, kReg>(c, m, K, T, TR, HS, multi, qa, qb, j, group, s6, st,
-                                                        bat_smem ? T : X.zstride, row0, acc[6], acc[7]);
+                                                        bat_smem ? T : X.zstride, row0, acc);
             }
         }
         for (int k = k0; k < k1; ++k) {
@@ -969,14 +1027,13 @@ __global__ void __launch_bounds__(kCrsMaxThreads, 1)
     };
     for (;;) {
         const int chunk = min(every, max_it - it);
-        float acc[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        Sum2 acc[9];  // (the residual iteration's alone)
         for (int jt = 0; jt < chunk - 1; ++jt) iterate(std::integral_constant<int, 0>{}, jt == chunk - 2, acc);
-        iterate(std::integral_constant<int, 1>{}, 1, acc);
 #pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            const float w = warp_sum(acc[q]);
-            if (lane == 0) m.wred[warp * kCrsRed + q] = w;
-        }
+        for (int q = 0; q < 9; ++q) acc[q] = Sum2{0.f, 0.f};
+        iterate(std::integral_constant<int, 1>{}, 1, acc);
+        const Sum2 w = warp_sums(acc, lane);
+        if (lane < 18 && (lane & 1) == 0) m.wred[warp * kCrsRed + (lane >> 1)] = (double)w.hi + (double)w.lo;
         if (tid == 0)  // (one reading for all ranks)
             m.flag[2] = (m.flag[1] ? 1 : 0) +
                         (rank == 0 && pause_at > 0 && *reinterpret_cast<volatile int*>(c.n_active) <= pause_at ? 64 : 0);
@@ -985,10 +1042,10 @@ __global__ void __launch_bounds__(kCrsMaxThreads, 1)
         // failure flag and, from rank 0, whether to pause
         for (int k = tid; k < kCrsRed * C; k += nt) {
             const int r = k / kCrsRed, q = k - kCrsRed * r;
-            float tot = 0.f;
+            double tot = 0.0;
             if (q < 9) for (int w = 0; w < nt / 32; ++w) tot += m.wred[w * kCrsRed + q];
-            else tot = (float)m.flag[2];
-            cl.map_shared_rank(m.red, r)[(slot * C + rank) * kCrsRed + q] = (double)tot;
+            else tot = (double)m.flag[2];
+            cl.map_shared_rank(m.red, r)[(slot * C + rank) * kCrsRed + q] = tot;
         }
         cl.sync();
         it += chunk;

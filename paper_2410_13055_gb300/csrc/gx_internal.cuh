@@ -151,7 +151,7 @@ __host__ __device__ inline CrsOff crs_offsets(int N, int G, int L, int B, int HS
     size_t p = 0;
     const int nbo = (B + C - 1) / C;
     o.red = crs_take(p, sizeof(double) * 2 * C * kCrsRed);
-    o.wred = crs_take(p, 4 * (size_t)(threads / 32) * kCrsRed);
+    o.wred = crs_take(p, sizeof(double) * (size_t)(threads / 32) * kCrsRed);
     o.xch = crs_take(p, 4 * 8 * (size_t)(threads / 32));
     o.bar = crs_take(p, 16);
     o.flag = crs_take(p, 16);
