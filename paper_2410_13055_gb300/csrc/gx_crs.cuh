@@ -148,14 +148,21 @@ struct Sum2 {
     }
 };
 
-// The warp's total of sum q, in lanes 2 q and 2 q + 1: each step halves the sums that a lane carries.
-__device__ __forceinline__ Sum2 warp_sums(const Sum2 (&acc)[9], int lane) {
-    Sum2 v[16];
+// The sums of a residual check: |n| pbar^2 and the phase mismatch; the adjoint scale; |z^k - z^{k-1}|^2
+// (devices' dx^2 less the buses' part); dthbar^2 w; |rho u|^2; and x^2, which is there for the test
+// of finiteness alone and so a plain FP32 sum.
+struct ResSums {
+    Sum2 n, scale, dz, dth, u;
+    float x;
+};
+
+// The warp's totals, sum k of ResSums in lanes 4 k to 4 k + 3: a step that can halves the sums that
+// a lane carries.
+__device__ __forceinline__ Sum2 warp_sums(const ResSums& a, int lane) {
+    Sum2 v[8] = {a.n, a.scale, a.dz, a.dth, a.u, Sum2{a.x, 0.f}, Sum2{0.f, 0.f}, Sum2{0.f, 0.f}};
 #pragma unroll
-    for (int q = 0; q < 16; ++q) v[q] = q < 9 ? acc[q < 9 ? q : 0] : Sum2{0.f, 0.f};
-#pragma unroll
-    for (int n = 8; n >= 1; n >>= 1) {
-        const int bit = 2 * n;
+    for (int n = 4; n >= 1; n >>= 1) {
+        const int bit = 4 * n;
         const bool up = lane & bit;
 #pragma unroll
         for (int q = 0; q < n; ++q) {
@@ -164,7 +171,9 @@ __device__ __forceinline__ Sum2 warp_sums(const Sum2 (&acc)[9], int lane) {
             v[q].add(__shfl_xor_sync(0xffffffffu, out.hi, bit), __shfl_xor_sync(0xffffffffu, out.lo, bit));
         }
     }
-    v[0].add(__shfl_xor_sync(0xffffffffu, v[0].hi, 1), __shfl_xor_sync(0xffffffffu, v[0].lo, 1));
+#pragma unroll
+    for (int bit = 2; bit >= 1; bit >>= 1)
+        v[0].add(__shfl_xor_sync(0xffffffffu, v[0].hi, bit), __shfl_xor_sync(0xffffffffu, v[0].lo, bit));
     return v[0];
 }
 
@@ -175,7 +184,7 @@ struct GState {
 
 struct Sm {
     double* red;     // [2][C][kCrsRed] residual partials of every rank (two chunks' slots)
-    double* wred;    // [warps][kCrsRed]
+    Sum2* wred;      // [warps][kCrsRed - 1]
     float* xch;      // [warps][8] two-warp exchange of the battery prox
     unsigned long long* bar;  // [0] battery injections have arrived, [1] prox targets have arrived
     int* flag;       // [0] stop, [1] a bounded wait gave up, [2] this rank's marks at a residual check
@@ -198,7 +207,7 @@ struct Sm {
 __device__ __forceinline__ Sm sm_at(unsigned char* b, const CrsOff& o) {
     Sm m;
     m.red = reinterpret_cast<double*>(b + o.red);
-    m.wred = reinterpret_cast<double*>(b + o.wred);
+    m.wred = reinterpret_cast<Sum2*>(b + o.wred);
     m.xch = reinterpret_cast<float*>(b + o.xch);
     m.bar = reinterpret_cast<unsigned long long*>(b + o.bar);
     m.flag = reinterpret_cast<int*>(b + o.flag);
@@ -263,7 +272,7 @@ __device__ __forceinline__ void res_battery(const Ctx& c, const Sm& m, const Bat
                                             const unsigned (&qa)[kV == 4 ? 1 : kHpl],
                                             const unsigned (&qb)[kV == 4 ? 1 : kHpl], int slot, int group,
                                             float (&s6)[6][kHpl], float* st, long long sstride, long long row0,
-                                            Sum2 (&acc)[9]) {
+                                            ResSums& acc) {
     constexpr int NL = 32 * kW;
     const int Lx = threadIdx.x & (NL - 1);
     const int lane = Lx & 31, wb = Lx >> 5;
@@ -457,8 +466,8 @@ __device__ __forceinline__ void res_battery(const Ctx& c, const Sm& m, const Bat
             dx2 += (xn[j] - old) * (xn[j] - old);
             x2 += xn[j] * xn[j];
         }
-        acc[6].add(dx2);
-        acc[7].add(x2);
+        acc.dz.add(dx2);
+        acc.x += x2;
         sync();  // every lane has read the old injections before a lane of another order sends new ones
     }
     if (!multi) {
@@ -509,7 +518,7 @@ __device__ __forceinline__ void res_scan_table(const float* ird, float* sc, int 
 // and in the residual iteration.
 template <int WANT, int ADJ, int kV>
 __device__ __forceinline__ void res_line(const Ctx& c, const Sm& m, float* sg, long long row, int HS, int l, int hq,
-                                         int store_sg, Sum2 (&acc)[9]) {
+                                         int store_sg, ResSums& acc) {
     float dx2 = 0.f, x2 = 0.f, th2 = 0.f;
     const int hl = hq * kV;
     const int4 lr = m.liner[l];
@@ -557,9 +566,9 @@ __device__ __forceinline__ void res_line(const Ctx& c, const Sm& m, float* sg, l
         }
     }
     if (WANT) {
-        acc[6].add(dx2);
-        acc[7].add(x2);
-        acc[8].add(th2);
+        acc.dz.add(dx2);
+        acc.x += x2;
+        acc.n.add(th2);
     }
     stv<kV>(pd, dn); stv<kV>(pqf, nf); stv<kV>(pqt, nt);
     if (WANT || store_sg) stv<kV>(sg + gr, gn);
@@ -567,7 +576,7 @@ __device__ __forceinline__ void res_line(const Ctx& c, const Sm& m, float* sg, l
 
 // One generator item: clip (forward) or masked step (adjoint).
 template <int WANT, int ADJ, int kV>
-__device__ __forceinline__ void res_gen(const Sm& m, float rho, float inv_re, int HS, int g, int hl, Sum2 (&acc)[9]) {
+__device__ __forceinline__ void res_gen(const Sm& m, float rho, float inv_re, int HS, int g, int hl, ResSums& acc) {
     float dx2 = 0.f, x2 = 0.f, scale = 0.f;
     const int2 gr = m.genr[g];
     const float cost = __int_as_float(gr.y);
@@ -592,16 +601,16 @@ __device__ __forceinline__ void res_gen(const Sm& m, float rho, float inv_re, in
         }
     }
     if (WANT) {
-        if (ADJ) acc[1].add(scale);
-        acc[2].add(dx2);
-        acc[5].add(x2);
+        if (ADJ) acc.scale.add(scale);
+        acc.dz.add(dx2);
+        acc.x += x2;
     }
     stv<kV>(px, xn);
 }
 
 // One load item (shed variable; terminal injection shed - L).
 template <int WANT, int ADJ, int kV>
-__device__ __forceinline__ void res_load(const Sm& m, float rho, float inv_re, float voll, int i, Sum2 (&acc)[9]) {
+__device__ __forceinline__ void res_load(const Sm& m, float rho, float inv_re, float voll, int i, ResSums& acc) {
     float dx2 = 0.f, x2 = 0.f, scale = 0.f;
     float x[kV], Ld[kV], pb[kV], uu[kV], xn[kV];
     ldv<kV>(m.xl + i, x); ldv<kV>(m.ld + i, Ld); ldv<kV>(m.pbar + i, pb); ldv<kV>(m.u + i, uu);
@@ -622,9 +631,9 @@ __device__ __forceinline__ void res_load(const Sm& m, float rho, float inv_re, f
         }
     }
     if (WANT) {
-        if (ADJ) acc[1].add(scale);
-        acc[2].add(dx2);
-        acc[5].add(x2);
+        if (ADJ) acc.scale.add(scale);
+        acc.dz.add(dx2);
+        acc.x += x2;
     }
     stv<kV>(m.xl + i, xn);
 }
@@ -649,7 +658,7 @@ __device__ __forceinline__ void push_targets(const Sm& m, int HS, int t, bool mu
 // kernels' order), then the consensus and the dual update.
 template <int WANT, int kV>
 __device__ __forceinline__ void res_bus(const Ctx& c, const Sm& m, float rho, int HS, int n, int hl, int t, bool multi,
-                                        Sum2 (&acc)[9]) {
+                                        ResSums& acc) {
     const int i = n * HS + hl;
     const int4 br = m.busr[n];
     const float4 bf = m.busf[n];
@@ -749,11 +758,11 @@ __device__ __forceinline__ void res_bus(const Ctx& c, const Sm& m, float rho, in
             dth2 += (thn[h] - th[h]) * (thn[h] - th[h]) * bf.z;
             u2 += cnt * (rho * un[h]) * (rho * un[h]);
         }
-        acc[0].add(p2);
-        acc[2].add(-dp2);
-        acc[3].add(dth2);
-        acc[4].add(u2);
-        acc[5].add(x2);
+        acc.n.add(p2);
+        acc.dz.add(-dp2);
+        acc.dth.add(dth2);
+        acc.u.add(u2);
+        acc.x += x2;
     }
     push_targets<kV>(m, HS, t, multi, br.z, nb, xbr, pbn, un);
     stv<kV>(m.pbar + i, pbn);
@@ -981,7 +990,7 @@ __global__ void __launch_bounds__(kCrsMaxThreads, 1)
     int it = it0, slot = 0;
     unsigned ph = 0;  // iterations of this launch: the barriers' phases
     double best = it0 > 0 ? c.rbest[s] : 0.0;
-    auto iterate = [&](auto want_c, int store_sg, Sum2 (&acc)[9]) {
+    auto iterate = [&](auto want_c, int store_sg, ResSums& acc) {
         constexpr int W = decltype(want_c)::value;
         if (tid == 0 && wait_x) mbar_expect_tx(m.bar, bytes_x);
         // A: batteries first (the longest chain), then chunks of the other devices
@@ -1027,25 +1036,25 @@ __global__ void __launch_bounds__(kCrsMaxThreads, 1)
     };
     for (;;) {
         const int chunk = min(every, max_it - it);
-        Sum2 acc[9];  // (the residual iteration's alone)
+        ResSums acc;  // (the residual iteration's alone)
         for (int jt = 0; jt < chunk - 1; ++jt) iterate(std::integral_constant<int, 0>{}, jt == chunk - 2, acc);
-#pragma unroll
-        for (int q = 0; q < 9; ++q) acc[q] = Sum2{0.f, 0.f};
+        acc = ResSums{};
         iterate(std::integral_constant<int, 1>{}, 1, acc);
         const Sum2 w = warp_sums(acc, lane);
-        if (lane < 18 && (lane & 1) == 0) m.wred[warp * kCrsRed + (lane >> 1)] = (double)w.hi + (double)w.lo;
+        if (lane < 4 * (kCrsRed - 1) && (lane & 3) == 0) m.wred[warp * (kCrsRed - 1) + (lane >> 2)] = w;
         if (tid == 0)  // (one reading for all ranks)
             m.flag[2] = (m.flag[1] ? 1 : 0) +
                         (rank == 0 && pause_at > 0 && *reinterpret_cast<volatile int*>(c.n_active) <= pause_at ? 64 : 0);
         __syncthreads();
-        // this rank's partial sums into every rank's reduction slots; the last slot carries its
+        // this rank's sums, a warp each, into every rank's reduction slots; the last slot carries its
         // failure flag and, from rank 0, whether to pause
-        for (int k = tid; k < kCrsRed * C; k += nt) {
-            const int r = k / kCrsRed, q = k - kCrsRed * r;
-            double tot = 0.0;
-            if (q < 9) for (int w = 0; w < nt / 32; ++w) tot += m.wred[w * kCrsRed + q];
-            else tot = (double)m.flag[2];
-            cl.map_shared_rank(m.red, r)[(slot * C + rank) * kCrsRed + q] = tot;
+        for (int q = warp; q < kCrsRed; q += nt / 32) {
+            Sum2 t = lane < nt / 32 && q < kCrsRed - 1 ? m.wred[lane * (kCrsRed - 1) + q] : Sum2{0.f, 0.f};
+#pragma unroll
+            for (int bit = 16; bit >= 1; bit >>= 1)
+                t.add(__shfl_xor_sync(0xffffffffu, t.hi, bit), __shfl_xor_sync(0xffffffffu, t.lo, bit));
+            const double tot = q < kCrsRed - 1 ? (double)t.hi + (double)t.lo : (double)m.flag[2];
+            if (lane < C) cl.map_shared_rank(m.red, lane)[(slot * C + rank) * kCrsRed + q] = tot;
         }
         cl.sync();
         it += chunk;
@@ -1059,8 +1068,8 @@ __global__ void __launch_bounds__(kCrsMaxThreads, 1)
             // NaN / inf test on the raw sums, before the clamps (fmax would turn a NaN into 0)
             const bool finite = __all_sync(0xffffffffu, isfinite(a));
             auto sum = [&](int q) { return __shfl_sync(0xffffffffu, a, q); };
-            const double s0 = sum(0) + sum(8), s1 = sum(1), dz2 = fmax(sum(2) + sum(6), 0.0), s3 = sum(3), s4 = sum(4);
-            const double marks = sum(9);
+            const double s0 = sum(0), s1 = sum(1), dz2 = fmax(sum(2), 0.0), s3 = sum(3), s4 = sum(4);
+            const double marks = sum(kCrsRed - 1);
             const bool pause = marks >= 64.0, bad = marks != (pause ? 64.0 : 0.0);
             const double rhod = c.rho, rth = c.rth_c;
             const double arg = lane == 0 ? fmax(s0, 0.0) : lane == 1 ? s1 : lane == 2 ? rhod * rhod * dz2 + rth * rth * s3 : s4;

@@ -83,7 +83,7 @@ constexpr int kBusRing = 4;
 // hours [r*H, (r+1)*H) of every device, its state in shared memory.
 constexpr int kCrsMaxThreads = 640;  // 20 warps of at most 96 registers
 constexpr int kCrsMaxC = 16;
-constexpr int kCrsRed = 10;          // residual partial sums per rank (9 used)
+constexpr int kCrsRed = 7;           // residual sums per rank, and its marks
 constexpr size_t kCrsSmemMax = 227 * 1024;
 constexpr int kCrsMaxEnds = 4095;    // generators or line ends of one bus (12-bit counts)
 constexpr int kCrsMaxBats = 255;     // batteries of one bus (8-bit count)
@@ -151,7 +151,7 @@ __host__ __device__ inline CrsOff crs_offsets(int N, int G, int L, int B, int HS
     size_t p = 0;
     const int nbo = (B + C - 1) / C;
     o.red = crs_take(p, sizeof(double) * 2 * C * kCrsRed);
-    o.wred = crs_take(p, sizeof(double) * (size_t)(threads / 32) * kCrsRed);
+    o.wred = crs_take(p, 8 * (size_t)(threads / 32) * (kCrsRed - 1));
     o.xch = crs_take(p, 4 * 8 * (size_t)(threads / 32));
     o.bar = crs_take(p, 16);
     o.flag = crs_take(p, 16);
