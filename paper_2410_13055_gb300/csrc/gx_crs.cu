@@ -53,13 +53,12 @@ int crs_max_clusters(int adj, const CrsShape& p, size_t smem) {
     return n;
 }
 
-int launch_crs(const Ctx& c, const CrsTables& tab, int adj, const int* scen, int n, const CrsShape& p, double tol, int it0, int pause_at,
-               cudaStream_t st) {
+int launch_crs(const Ctx& c, const CrsTables& tab, int adj, const int4* runs, int n, const CrsShape& p, double tol, cudaStream_t st) {
     if (n <= 0) return 0;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[1];
     crs_config(cfg, at, n, p.C, p.threads, p.smem[adj], st);
-    cudaLaunchKernelEx(&cfg, crs_kernel(adj, p), c, tab, scen, p.C, p.bat_smem[adj], tol, it0, pause_at);
+    cudaLaunchKernelEx(&cfg, crs_kernel(adj, p), c, tab, runs, p.C, p.bat_smem[adj], tol);
     return 1;
 }
 

@@ -187,7 +187,7 @@ struct Sm {
     Sum2* wred;      // [warps][kCrsRed - 1]
     float* xch;      // [warps][8] two-warp exchange of the battery prox
     unsigned long long* bar;  // [0] battery injections have arrived, [1] prox targets have arrived
-    int* flag;       // [0] stop, [1] a bounded wait gave up, [2] this rank's marks at a residual check
+    int* flag;       // [0] stop, [1] a bounded wait gave up, [2] that as of a residual check
     int4* busr;      // [N] generator rows, first line-end slot, first battery slot, counts (12, 12, 8 bits)
     float4* busf;    // [N] 1/terminals, 1/sum of phase weights, dual-residual weight
     int2* genr;      // [G] bus row offset, cost
@@ -772,12 +772,12 @@ __device__ __forceinline__ void res_bus(const Ctx& c, const Sm& m, float rho, in
 
 template <int ADJ, int kHpl, int kW, int kV, int kReg>
 __global__ void __launch_bounds__(kCrsMaxThreads, 1)
-    k_crs(const Ctx c, const CrsTables R, const int* __restrict__ scen, int C, int bat_smem, double tol, int it0_arg, int pause_at) {
+    k_crs(const Ctx c, const CrsTables R, const int4* __restrict__ runs, int C, int bat_smem, double tol) {
     extern __shared__ __align__(16) unsigned char smem[];
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
-    const int s = scen[blockIdx.x / C];
-    const int it0 = it0_arg >= 0 ? it0_arg : (ADJ ? c.adj_iters : c.iters)[s];  // iterations already run
+    const int4 run = runs[blockIdx.x / C];
+    const int s = run.x, it0 = run.y, it_end = run.z;  // iterations already run; pause once it_end have
     const ScenDev sd = c.scen[s];
     const int T = sd.T, N = sd.N, G = sd.G, L = sd.L, B = sd.B;
     const int HS = crs_hours(T, C, kV);
@@ -1042,12 +1042,10 @@ __global__ void __launch_bounds__(kCrsMaxThreads, 1)
         iterate(std::integral_constant<int, 1>{}, 1, acc);
         const Sum2 w = warp_sums(acc, lane);
         if (lane < 4 * (kCrsRed - 1) && (lane & 3) == 0) m.wred[warp * (kCrsRed - 1) + (lane >> 2)] = w;
-        if (tid == 0)  // (one reading for all ranks)
-            m.flag[2] = (m.flag[1] ? 1 : 0) +
-                        (rank == 0 && pause_at > 0 && *reinterpret_cast<volatile int*>(c.n_active) <= pause_at ? 64 : 0);
+        if (tid == 0) m.flag[2] = m.flag[1] ? 1 : 0;  // (one reading for all ranks)
         __syncthreads();
         // this rank's sums, a warp each, into every rank's reduction slots; the last slot carries its
-        // failure flag and, from rank 0, whether to pause
+        // failure flag
         for (int q = warp; q < kCrsRed; q += nt / 32) {
             Sum2 t = lane < nt / 32 && q < kCrsRed - 1 ? m.wred[lane * (kCrsRed - 1) + q] : Sum2{0.f, 0.f};
 #pragma unroll
@@ -1070,7 +1068,7 @@ __global__ void __launch_bounds__(kCrsMaxThreads, 1)
             auto sum = [&](int q) { return __shfl_sync(0xffffffffu, a, q); };
             const double s0 = sum(0), s1 = sum(1), dz2 = fmax(sum(2), 0.0), s3 = sum(3), s4 = sum(4);
             const double marks = sum(kCrsRed - 1);
-            const bool pause = marks >= 64.0, bad = marks != (pause ? 64.0 : 0.0);
+            const bool pause = it >= it_end, bad = marks != 0.0;
             const double rhod = c.rho, rth = c.rth_c;
             const double arg = lane == 0 ? fmax(s0, 0.0) : lane == 1 ? s1 : lane == 2 ? rhod * rhod * dz2 + rth * rth * s3 : s4;
             const double root = sqrt(arg);
@@ -1095,11 +1093,7 @@ __global__ void __launch_bounds__(kCrsMaxThreads, 1)
                     (ADJ ? c.adj_iters : c.iters)[s] = it;
                     c.rbest[s] = best;
                 }
-                if (rank == 0 && stop && pause_at > 0) atomicSub(c.n_active, 1);
-                if (rank == 0 && !stop && pause) {
-                    (ADJ ? c.adj_iters : c.iters)[s] = it;
-                    c.rbest[s] = best;
-                }
+                if (rank == 0 && !stop && pause) c.rbest[s] = best;
                 m.flag[0] = stop || pause;
             }
         }

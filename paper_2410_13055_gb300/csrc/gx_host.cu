@@ -660,13 +660,13 @@ static std::vector<const std::vector<CrsChoice>*> crs_lists(const gx_network* ne
     return ch;
 }
 
-// Launch shapes for the scenarios `act` (crs_assign); returns the estimated time per iteration.
-static double crs_shapes(const gx_network* net, const std::vector<int>& act, std::vector<CrsShape>* shapes, bool* fits) {
+// A choice for each of the scenarios `act` (crs_assign); returns the estimated time per iteration.
+static double crs_pick(const gx_network* net, const std::vector<int>& act, std::vector<const CrsChoice*>* pick, bool* fits) {
     const auto ch = crs_lists(net, act);
     std::vector<size_t> at;
     const double us = crs_assign(ch, act.size(), at, fits);
-    shapes->resize(act.size());
-    for (size_t i = 0; i < act.size(); ++i) (*shapes)[i] = (*ch[i])[at[i]].shape;
+    pick->resize(act.size());
+    for (size_t i = 0; i < act.size(); ++i) (*pick)[i] = &(*ch[i])[at[i]];
     return us;
 }
 
@@ -1176,7 +1176,7 @@ gx_status gx_network_create(const gx_network_desc* nets, int n_nets, const gx_sc
     net->o_busblk = L.add(sizeof(BusBlk) * std::max<size_t>(net->bus_blk.size(), 1));
     net->o_pool = L.add(I4((long long)net->pool.size()));
     net->o_prep = L.add(8 * std::max<size_t>(net->prep.size(), 1));
-    net->o_crs = L.add(I4(S));
+    net->o_crs = L.add(sizeof(int4) * (size_t)S);
     net->o_bus4blk = L.add(sizeof(BusBlk) * std::max<size_t>(net->bus4_blk.size(), 1));
     net->o_buscpl = L.add(I4(std::max<long long>((long long)net->bus_cpl.size(), 1)));
     net->o_busdone = L.add(I4(std::max<long long>((long long)net->bus4_blk.size(), 1)));
@@ -1604,43 +1604,39 @@ static bool crs_active(const gx_network* net) {
 }
 
 // Launch the resident loops of the scenarios `act` (one launch per group of equal shape, the
-// groups on streams of their own unless there is one).  it0 >= 0: iterations already run by all
-// of them, -1: by each what its iteration count says; pause_at: stop at the next residual check
-// once at most that many are still iterating (0: run all to their end).  What follows on `st`
-// waits for them (crs_wait).
-static gx_status crs_launch(gx_network* net, int adj, const std::vector<int>& act, const std::vector<CrsShape>& shapes, int it0,
-                            int pause_at, bool alone, cudaStream_t st, int* launches, int* used) {
+// groups on streams of their own unless there is one).  its: per scenario of the network the
+// iterations already run; ends: per scenario of `act` the iterations at which it pauses.  What
+// follows on `st` waits for them (crs_wait).
+static gx_status crs_launch(gx_network* net, int adj, const std::vector<int>& act, const std::vector<const CrsChoice*>& pick,
+                            const std::vector<int>& its, const std::vector<int>& ends, bool alone, cudaStream_t st,
+                            int* launches, int* used) {
     const Ctx& c = adj ? net->actx : net->ctx;
     const double tol = adj ? net->opts.adj_tol : net->opts.tol;
     *used = 0;
     struct Group { CrsShape shape; int first, n; };
     std::vector<Group> groups;
-    std::vector<int> list;
+    std::vector<int4> list;
     // (largest clusters first: they need the most contiguous room)
     typedef std::tuple<int, int, int, int, int, int, int, int> Key;
     std::map<Key, std::vector<size_t>> by;
     for (size_t i = 0; i < act.size(); ++i) {
-        const CrsShape& p = shapes[i];
+        const CrsShape& p = pick[i]->shape;
         by[Key(-p.C, p.V, p.threads, p.kw, p.hpl, p.reg, p.bat_smem[0], p.bat_smem[1])].push_back(i);
     }
     for (const auto& kv : by) {
-        Group g{shapes[kv.second[0]], (int)list.size(), (int)kv.second.size()};
+        Group g{pick[kv.second[0]]->shape, (int)list.size(), (int)kv.second.size()};
         for (size_t i : kv.second) {
-            for (int k = 0; k < 2; ++k) g.shape.smem[k] = std::max(g.shape.smem[k], shapes[i].smem[k]);
-            list.push_back(act[i]);
+            for (int k = 0; k < 2; ++k) g.shape.smem[k] = std::max(g.shape.smem[k], pick[i]->shape.smem[k]);
+            list.push_back(make_int4(act[i], its[act[i]], ends[i], 0));
         }
         groups.push_back(g);
     }
-    int* dlist = reinterpret_cast<int*>(net->dev + net->o_crs);
-    GX_CUDA(cudaMemcpyAsync(dlist, list.data(), 4 * list.size(), cudaMemcpyHostToDevice, st));
-    if (pause_at > 0) {
-        const int n = (int)act.size();
-        GX_CUDA(cudaMemcpyAsync(c.n_active, &n, sizeof(int), cudaMemcpyHostToDevice, st));
-    }
+    int4* dlist = reinterpret_cast<int4*>(net->dev + net->o_crs);
+    GX_CUDA(cudaMemcpyAsync(dlist, list.data(), sizeof(int4) * list.size(), cudaMemcpyHostToDevice, st));
     if (net->prof) GX_CUDA(cudaEventRecord(net->ev[0], st));
     int nl = 0;
     if (groups.size() == 1 && alone) {
-        nl += launch_crs(c, net->crs_tables, adj, dlist, groups[0].n, groups[0].shape, tol, it0, pause_at, st);
+        nl += launch_crs(c, net->crs_tables, adj, dlist, groups[0].n, groups[0].shape, tol, st);
     } else {
         if (!net->crs_fork) GX_CUDA(cudaEventCreateWithFlags(&net->crs_fork, cudaEventDisableTiming));
         GX_CUDA(cudaEventRecord(net->crs_fork, st));
@@ -1651,8 +1647,7 @@ static gx_status crs_launch(gx_network* net, int adj, const std::vector<int>& ac
             GX_CUDA(cudaStreamWaitEvent(net->crs_streams[k], net->crs_fork, 0));
         }
         for (size_t k = 0; k < groups.size(); ++k)
-            nl += launch_crs(c, net->crs_tables, adj, dlist + groups[k].first, groups[k].n, groups[k].shape, tol, it0, pause_at,
-                             net->crs_streams[k % ns]);
+            nl += launch_crs(c, net->crs_tables, adj, dlist + groups[k].first, groups[k].n, groups[k].shape, tol, net->crs_streams[k % ns]);
         for (int k = 0; k < ns; ++k) GX_CUDA(cudaEventRecord(net->crs_join[k], net->crs_streams[k]));
         *used = ns;
     }
@@ -1772,12 +1767,19 @@ static std::vector<int> crs_sorted(const gx_network* net, const std::vector<int>
 }
 
 // Iterate the batch's scenarios to their stops on whichever path is estimated faster for those
-// still iterating.  Both take bitwise the same iterates and test the same residuals at the same
-// iterations, so a change of path or of cluster size at a residual check changes no result:
+// still iterating:
 //  * while the scenarios do not fit the device's shared memory side by side, or one of them fits
 //    no cluster, the per-iteration kernels run them all, and pause once the rest fit;
-//  * once they fit and a resident iteration is estimated shorter, each runs in its cluster; as
-//    scenarios stop, the rest pause and take larger clusters where that is worth a tenth.
+//  * once they fit and a resident iteration is estimated shorter, each runs in its cluster; while
+//    fewer of them would gain a tenth from larger clusters, they pause from time to time, and those
+//    left are given clusters anew.
+// Both paths take bitwise the same iterates and test the residual at the same iterations, but add up
+// its terms in another order: a residual within rounding of its tolerance (2^-24 between the paths,
+// about 2^-45 between cluster sizes of one item width) can stop a check earlier or later.  Which path
+// and which cluster runs an iteration depends on the inputs and the estimates alone: every pause is a
+// number of iterations fixed beforehand, or a count of scenarios at a check of the per-iteration
+// kernels, whose scenarios are in step.  So two equal calls take equal steps.  (A pause as soon as few
+// enough clusters were left depended on how far the others had got.)
 static gx_status iterate(gx_network* net, int adj, cudaStream_t st, int* launches, int it0 = 0) {
     int it = it0, used = 0;
     if (!crs_active(net)) return run_loop(net, adj, st, launches, &it, it0);
@@ -1789,7 +1791,8 @@ static gx_status iterate(gx_network* net, int adj, cudaStream_t st, int* launche
         if (gx_status e = still_active(net, st, act)) return e;
         if (act.empty() || it0 >= max_it) return GX_OK;
     }
-    std::vector<CrsShape> shapes;
+    std::vector<const CrsChoice*> pick;
+    std::vector<int> its(net->S, it0), ends;  // iterations run, by scenario; the next pauses, as `act`
     const bool asked = net->use_crs == 1;  // every scenario that fits a cluster runs in it
     if (asked) {
         std::vector<int> res;
@@ -1803,14 +1806,16 @@ static gx_status iterate(gx_network* net, int adj, cudaStream_t st, int* launche
                 if (net->crs_of[s]->empty()) net->done_loop[s] = 0;
             GX_CUDA(cudaMemcpyAsync(net->dev + net->o_done, net->done_loop.data(), 4 * net->S, cudaMemcpyHostToDevice, st));
             bool fits;
-            crs_shapes(net, res, &shapes, &fits);
-            if (gx_status e = crs_launch(net, adj, res, shapes, it0, 0, false, st, launches, &used)) return e;
+            crs_pick(net, res, &pick, &fits);
+            ends.assign(res.size(), max_it);
+            if (gx_status e = crs_launch(net, adj, res, pick, its, ends, false, st, launches, &used)) return e;
             const gx_status le = run_loop(net, adj, st, launches, &it, it0);
             if (gx_status e = crs_wait(net, used, st)) return e;
             return le;
         }
     }
     bool resident = false;
+    double spent = 0;  // estimated time so far
     for (;;) {
         const int n = (int)act.size();
         int n_fit = 0;
@@ -1821,7 +1826,7 @@ static gx_status iterate(gx_network* net, int adj, cudaStream_t st, int* launche
         }
         bool fits = false;
         double us = 0;
-        if (n_fit == n) us = crs_shapes(net, act, &shapes, &fits);
+        if (n_fit == n) us = crs_pick(net, act, &pick, &fits);
         if (!resident && !asked && !(fits && us < 0.95 * stream_us(dh))) {
             // Pause once no scenario without a cluster is left and as many others as fit for
             // certain: the most for which the largest ones fit.
@@ -1829,20 +1834,32 @@ static gx_status iterate(gx_network* net, int adj, cudaStream_t st, int* launche
             std::vector<double> big_dh;
             for (int s : big) big_dh.push_back(net->crs_dh[s]);
             const int pause_at = (int)crs_pause_at(crs_lists(net, big), big_dh, (size_t)n - 1);
+            const int from = it;
             if (gx_status e = run_loop(net, adj, st, launches, &it, it, pause_at)) return e;
             if (pause_at == 0 || it >= max_it) return GX_OK;
+            spent += (it - from) * stream_us(dh);
+            for (int s : act) its[s] = it;
             if (gx_status e = still_active(net, st, act)) return e;
             if (act.empty()) return GX_OK;
             continue;
         }
-        // the largest count of remaining scenarios at which larger clusters pay for the pause
-        // (estimated on the slowest of them, for whichever remain)
-        const int pause_at = net->prof ? 0 : (int)crs_regroup_at(crs_lists(net, crs_sorted(net, net->crs_by_us, act)), us);
-        if (gx_status e = crs_launch(net, adj, act, shapes, resident ? -1 : it, pause_at, true, st, launches, &used)) return e;
+        // Where fewer scenarios would gain from larger clusters, each pauses after a share of the time
+        // spent so far (by the estimates, so that all pause together).
+        const bool pause = !net->prof && crs_regroup_at(crs_lists(net, crs_sorted(net, net->crs_by_us, act)), us) > 0;
+        const double part = std::max(kCrsPause, spent * kCrsPauseShare);
+        bool last = true;
+        ends.assign(act.size(), max_it);
+        for (size_t i = 0; pause && i < act.size(); ++i) {
+            ends[i] = crs_pause_end(its[act[i]], pick[i]->us, part, net->opts.check_every, max_it);
+            last = last && ends[i] == max_it;
+        }
+        if (gx_status e = crs_launch(net, adj, act, pick, its, ends, true, st, launches, &used)) return e;
         if (gx_status e = crs_wait(net, used, st)) return e;
-        if (pause_at == 0) return GX_OK;
+        if (last) return GX_OK;
+        for (size_t i = 0; i < act.size(); ++i) its[act[i]] = ends[i];
         if (gx_status e = still_active(net, st, act)) return e;
         if (act.empty()) return GX_OK;
+        spent += part;
         resident = true;
     }
 }
@@ -2158,11 +2175,11 @@ gx_status gx_network_persistent_info(const gx_network* net, int scen, int* clust
     std::vector<int> fit;
     for (int s = 0; s < net->S; ++s)
         if (!net->crs_of[s]->empty()) fit.push_back(s);
-    std::vector<CrsShape> shapes;
+    std::vector<const CrsChoice*> pick;
     bool fits;
-    crs_shapes(net, fit, &shapes, &fits);
+    crs_pick(net, fit, &pick, &fits);
     for (size_t i = 0; i < fit.size(); ++i)
-        if (fit[i] == scen) *cluster_ctas = shapes[i].C;
+        if (fit[i] == scen) *cluster_ctas = pick[i]->shape.C;
     return GX_OK;
 }
 

@@ -83,7 +83,7 @@ constexpr int kBusRing = 4;
 // hours [r*H, (r+1)*H) of every device, its state in shared memory.
 constexpr int kCrsMaxThreads = 640;  // 20 warps of at most 96 registers
 constexpr int kCrsMaxC = 16;
-constexpr int kCrsRed = 7;           // residual sums per rank, and its marks
+constexpr int kCrsRed = 7;           // residual sums per rank, and its failure flag
 constexpr size_t kCrsSmemMax = 227 * 1024;
 constexpr int kCrsMaxEnds = 4095;    // generators or line ends of one bus (12-bit counts)
 constexpr int kCrsMaxBats = 255;     // batteries of one bus (8-bit count)
@@ -478,14 +478,12 @@ int launch_prep(const Ctx& c, cudaStream_t st);
 // enough; called at bind).
 cudaError_t bus_staged_prepare(int smem, int rec);
 int launch_loop_cond(const Ctx& c, const int* pause, int max_it, cudaGraphConditionalHandle h, cudaStream_t st);
-typedef void (*CrsFn)(Ctx, CrsTables, const int*, int, int, double, int, int);
-// Cluster-resident solver (gx_crs.cu): iterate the scenarios in `scen` to convergence, one cluster
-// each; it0 >= 0: iterations already run, -1: each scenario's own count; pause_at > 0: stop at the
-// next residual check once at most that many scenarios (counted down in n_active) are iterating.
+typedef void (*CrsFn)(Ctx, CrsTables, const int4*, int, int, double);
+// Cluster-resident solver (gx_crs.cu): iterate the scenarios in `runs` (scenario, iterations already
+// run, iterations after which it pauses) to convergence or their pause, one cluster each.
 cudaError_t crs_prepare(int adj, const CrsShape& p);
 int crs_max_clusters(int adj, const CrsShape& p, size_t smem);
-int launch_crs(const Ctx& c, const CrsTables& tab, int adj, const int* scen, int n, const CrsShape& p, double tol, int it0, int pause_at,
-               cudaStream_t st);
+int launch_crs(const Ctx& c, const CrsTables& tab, int adj, const int4* runs, int n, const CrsShape& p, double tol, cudaStream_t st);
 int launch_reduce(const Ctx& c, int adj, double tol, cudaStream_t st);
 int launch_tick(const Ctx& c, int chunk, cudaStream_t st);
 int launch_extract(const Ctx& c, const int* in_batch, cudaStream_t st);

@@ -6,6 +6,7 @@
 // every loop, so none of them may grow with the square of the scenario count.
 #pragma once
 #include <algorithm>
+#include <cmath>
 #include <cstddef>
 #include <queue>
 #include <utility>
@@ -17,6 +18,16 @@ namespace gx {
 // dependent launches (10 to 11 us for one scenario of any size here), then 3.3 to 3.6 us per million
 // device-hours (100 buses, 168 h: 10.9 us for 2 scenarios, 15.4 for 16).
 inline double stream_us(double dh) { return 10.0 + 3.5e-6 * dh; }
+
+// The time between two pauses of resident loops.  A pause costs 25 to 55 us (a launch, the state out
+// and in, a look at the done flags), so it comes after at least
+constexpr double kCrsPause = 800.0;
+// microseconds, and a share of the time spent so far, as what is left to gain shrinks against it.
+constexpr double kCrsPauseShare = 0.125;
+// 16 x 168 h of 100 buses, five sets of inputs, plan steps and dispatches from nothing: 72.0 and 77.9 ms;
+// 300 us 73.3 and 81.1, 500 us 72.4 and 79.3, 1,200 us 73.0 and 79.0, a share of 0.2 71.9 and 78.6, no
+// pauses 99.0 and 86.4.  (A pause as soon as few enough were left, which depended on how far each
+// cluster had got: 70.5 and 75.4.)
 
 // Clusters of mixed sizes leave gaps in the processing clusters that hold them.
 inline double crs_room_limit(bool one_list) { return one_list ? 1.0 + 1e-9 : 0.9; }
@@ -105,6 +116,13 @@ size_t crs_regroup_at(const std::vector<const std::vector<Choice>*>& ch, double 
     for (size_t k = std::min(ch.size() - 1, crs_fit_prefix(ch)); k >= 1; k = k > 8 ? k * 7 / 8 : k - 1)
         if (crs_assign(ch, k, at, &fits) < 0.9 * us && fits) return k;
     return 0;
+}
+
+// Where a scenario pauses: after `part` microseconds at `us` an iteration, rounded up to residual
+// checks, and at the cap at the latest.
+inline int crs_pause_end(int it, double us, double part, int every, int max_it) {
+    const double checks = std::max(1.0, std::ceil(part / (us * every)));
+    return checks * every < (double)(max_it - it) ? it + (int)checks * every : max_it;
 }
 
 }  // namespace gx

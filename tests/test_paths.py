@@ -84,6 +84,13 @@ int main() {
         if (k >= ch.size() && k) ++bad;
         if (k && !(assign(ch, k, a, &fa) < 0.9 * uc && fa)) ++bad;
     }
+    // pauses lie on residual checks, after at least the given time, and at the cap at the latest
+    for (int trial = 0; trial < 1000; ++trial) {
+        const int every = 1 + (int)uni(0, 40), it = every * (int)uni(0, 50), max_it = it + 1 + (int)uni(0, 5000);
+        const double us = uni(0.5, 20), part = uni(1, 3000);
+        const int e = crs_pause_end(it, us, part, every, max_it);
+        if (e <= it || e > max_it || (e < max_it && ((e - it) % every || (e - it) * us < part * (1 - 1e-9)))) ++bad;
+    }
     double worst = 0;  // milliseconds of the searches before one loop over 8,192 scenarios
     for (double us0 : {2.0, 60.0}) for (int keys : {1, 20, 8192}) for (double room0 : {1.0 / 700, 1.0 / 20}) {
         const std::vector<List> v = lists(keys, room0, us0);
