@@ -1356,7 +1356,7 @@ gx_status gx_network_bind(gx_network* net, void* dev_mem, size_t bytes, void* st
     if (!net->ev_fork) GX_CUDA(cudaEventCreateWithFlags(&net->ev_fork, cudaEventDisableTiming));
     if (!net->ev_join) GX_CUDA(cudaEventCreateWithFlags(&net->ev_join, cudaEventDisableTiming));
     if (!net->ev_join2) GX_CUDA(cudaEventCreateWithFlags(&net->ev_join2, cudaEventDisableTiming));
-    if (net->bus4_smem > 0) GX_CUDA(bus_staged_prepare((int)net->bus4_smem, net->bus4_rec));
+    GX_CUDA(bus_staged_prepare());
     {
         int dev = 0, l2 = 0;
         GX_CUDA(cudaGetDevice(&dev));

@@ -474,9 +474,8 @@ int launch_bat(const Ctx& c, int mode, int adj, int want_res, cudaStream_t st);
 int launch_ramp(const Ctx& c, int mode, int adj, int want_res, cudaStream_t st);
 int launch_bus(const Ctx& c, int mode, int adj, int want_res, cudaStream_t st);
 int launch_prep(const Ctx& c, cudaStream_t st);
-// Allow the staged bus kernel `smem` bytes of dynamic shared memory (once per process is
-// enough; called at bind).
-cudaError_t bus_staged_prepare(int smem, int rec);
+// Allow the staged bus kernels the dynamic shared memory of any network (called at bind).
+cudaError_t bus_staged_prepare();
 int launch_loop_cond(const Ctx& c, const int* pause, int max_it, cudaGraphConditionalHandle h, cudaStream_t st);
 typedef void (*CrsFn)(Ctx, CrsTables, const int4*, int, int, double);
 // Cluster-resident solver (gx_crs.cu): iterate the scenarios in `runs` (scenario, iterations already

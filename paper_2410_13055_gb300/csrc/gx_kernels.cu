@@ -2144,12 +2144,15 @@ int launch_bus(const Ctx& c, int mode, int adj, int want_res, cudaStream_t st) {
     return 1;
 }
 
-cudaError_t bus_staged_prepare(int smem, int rec) {
+// The attribute belongs to the function, not to a network: it is the most that any network's launch
+// can ask for (the longest record and the largest stage, or the ring), so that a network bound later
+// does not lower it for this one.
+cudaError_t bus_staged_prepare() {
     cudaError_t e = cudaSuccess;
     auto set = [&](const void* f, int bytes) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     };
-    const int ring = 4 * rec + 32 * kBusRing * kBusQBlock;
+    const int smem = 4 * kPoolMax + kStageMax, ring = 4 * kPoolMax + 32 * kBusRing * kBusQBlock;
 #define GX_BUS4S(A, R)                           \
     set((const void*)k_bus4t<A, R, 0>, smem);    \
     set((const void*)k_bus4t<A, R, 1>, smem);    \
