@@ -297,13 +297,17 @@ gx_status gx_network_get_schedule(const gx_network* net, gx_schedule* sched);
  * persistent launch that tests its own convergence.  on != 0: every such scenario does; 0: none,
  * all run on the per-iteration kernels.  Until this is called the library decides, per loop and
  * again as scenarios stop, by estimated time: scenarios go to clusters while all that are still
- * iterating fit the device side by side; never after a call of gx_network_set_schedule or another
- * launch mode than 2, nor while gx_profile_enable is on.  The two paths take bitwise the same
- * iterates for horizons up to 192 hours (longer ones always run on the per-iteration kernels
- * where they have batteries); only the residual partials are summed in another order, so that a
- * scenario may stop at another residual check on the other path.  Equal calls take equal steps: which
+ * iterating fit the device side by side; never after a call of gx_network_set_schedule (until
+ * gx_network_auto_path) or in another launch mode than 2, nor while gx_profile_enable is on.  The two
+ * paths take bitwise the same iterates for horizons up to 192 hours (longer ones always run on the
+ * per-iteration kernels where they have batteries); only the residual partials are summed in another
+ * order, so that a scenario may stop at another residual check on the other path.  Equal calls take equal steps: which
  * path and cluster runs an iteration follows from the inputs and the device alone, not from timing. */
 gx_status gx_network_use_persistent(gx_network* net, int on);
+/* Give the choice of path back to the library after gx_network_use_persistent or
+ * gx_network_set_schedule.  The schedule stays as it was set, for what runs on the per-iteration
+ * kernels. */
+gx_status gx_network_auto_path(gx_network* net);
 /* *cluster_ctas: CTAs of the cluster scenario `scen` runs on, 0 if it runs on the
  * per-iteration kernels (not resident, not launchable on this device, or switched off). */
 gx_status gx_network_persistent_info(const gx_network* net, int scen, int* cluster_ctas);

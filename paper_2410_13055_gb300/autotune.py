@@ -7,8 +7,8 @@ planner objective stays within `h_tol` of a tight reference solve at the same pl
 whose gradient there is no less accurate than the defaults' (within a factor `g_slack`)
 against a tight reference gradient (equal residual tolerances do not give equal
 accuracy across penalties; the adjoint penalty changes the gradient and not h).  Parameters:
-the execution path (per-iteration kernels replayed as CUDA graphs, or one persistent
-cluster-resident launch per loop for the scenarios that fit), the kernel schedule (how
+the execution path (the library's own choice, per-iteration kernels replayed as CUDA graphs, or
+persistent cluster-resident launches for the scenarios that fit), the kernel schedule (how
 the bus kernel brings its device rows in: per-thread loads, bulk copies into shared
 memory, or per-thread asynchronous copies; one or two warps per battery), residual-check
 chunk length (the CUDA-graph size), power penalty rho, phase penalty scale, adjoint
@@ -17,7 +17,9 @@ scenarios) rounded to powers of two.
 
 ``tune_schedule`` is the quick form for the kernel schedule alone: schedules do not change
 the iterates (the bus kernel variants are bitwise equal), so it times a fixed number of
-iterations per candidate and keeps the fastest.
+iterations per candidate and keeps the fastest.  Where the library chooses the path when a tuner
+is called, it does so again afterwards (unless the timed steps were slower that way), and the tuned
+schedule serves what it runs on the per-iteration kernels.
 """
 from __future__ import annotations
 
@@ -37,7 +39,7 @@ if TYPE_CHECKING:  # the library is loaded by the functions that run it
 SCHEDULE = {"bus_staged": [0, 1, 2], "bat_warps": [2, 1]}
 
 SPACE = {
-    "persistent": [False, True],
+    "persistent": [None, False, True],  # None: the library chooses the path
     "bus_staged": SCHEDULE["bus_staged"],
     "bat_warps": SCHEDULE["bat_warps"],
     "check_every": [10, 20, 40],
@@ -91,21 +93,29 @@ def _grad_err(net, eta, g_ref):
 def _apply(net, opts):
     """Options, execution path and kernel schedule of a setting."""
     net.set_opts(**{k: v for k, v in opts.items() if k not in ("persistent",) and k not in SCHEDULE})
-    if "persistent" in opts:
+    if opts.get("persistent") is not None:
         net.use_persistent(bool(opts["persistent"]))
     sched = {k: int(v) for k, v in opts.items() if k in SCHEDULE}
     if sched:
         net.set_schedule(**sched)
+    if "persistent" in opts and opts["persistent"] is None:
+        net.auto_path()
+
+
+def _path_is_auto(net):
+    return getattr(net, "path_is_auto", lambda: False)()
 
 
 def tune_schedule(net: gx.Network, eta, iters=200, space=None, log=None):
     """Pick the fastest kernel schedule for `net` at plan `eta`: for each candidate, time
     `iters` forward and `iters` adjoint iterations with every scenario iterating (the
     tolerances are set out of reach for the timing, then restored).  The schedules
-    compute the same iterates, so only time decides.  Leaves the state of the last
-    timing run in the workspace (callers start their solves cold).  Returns
+    compute the same iterates, so only time decides.  Every candidate runs on the per-iteration
+    kernels; afterwards the library chooses the path again if it did before.  Leaves the state of
+    the last timing run in the workspace (callers start their solves cold).  Returns
     dict(best=..., trials=[...])."""
     space = space or SCHEDULE
+    auto = _path_is_auto(net)
     keep = {k: getattr(net.opts, k) for k in ("tol", "adj_tol", "max_iter", "adj_max_iter")}
     net.solve(eta, warm="cold")
     net.grad(eta, warm="cold")
@@ -143,6 +153,8 @@ def tune_schedule(net: gx.Network, eta, iters=200, space=None, log=None):
     best = min(trials, key=lambda t: t["us_per_iteration"])
     best = {k: best[k] for k in SCHEDULE}
     net.set_schedule(**best)
+    if auto:
+        net.auto_path()
     net.set_opts(**keep)
     return dict(best=best, trials=trials, iterations=n)
 
@@ -168,15 +180,18 @@ def tune_schedule_step(net: gx.Network, eta, step=None, steps=2, reps=2, margin=
     a candidate is faster by more than `margin`: a single step's timing cannot tell apart
     schedules closer than that.  `flush()`, if given, runs before each step outside its
     timing (the caller's cache flush, so the steps are timed as the caller times them).
-    State and plan are restored at the end.  Unlike
-    `tune_schedule`, this times the steps' real mix of launches, including the ones where
-    most scenarios have converged.  Returns dict(best=..., default=..., trials=[...])."""
+    State and plan are restored at the end.  If the library chooses the path when the tuner is
+    called, its choice is timed as well, with the schedule picked, and kept unless the per-iteration
+    kernels alone are faster by more than `margin`.  Unlike `tune_schedule`, this times the steps'
+    real mix of launches, including the ones where most scenarios have converged.  Returns dict(best=..., default=..., trials=[...]), and
+    auto=dict(ms_per_step=..., kept=...) where the library chose."""
     space = space or SCHEDULE
     if step is None:
         def step(e):
             net.solve(e, warm="prev")
             net.grad(e, warm="prev")
     default = net.schedule()
+    auto = _path_is_auto(net)
     sx, sa, se = net.state(False).clone(), net.state(True).clone(), eta.clone()
 
     def restore():
@@ -184,10 +199,7 @@ def tune_schedule_step(net: gx.Network, eta, step=None, steps=2, reps=2, margin=
         net.state(True).copy_(sa)
         eta.copy_(se)
 
-    cands = [dict(bus_staged=b, bat_warps=w) for b in space["bus_staged"] for w in space["bat_warps"]]
-    trials = []
-    for cand in cands:
-        net.set_schedule(**cand)
+    def timed():
         best_ms = None
         for _ in range(reps):
             restore()
@@ -205,18 +217,34 @@ def tune_schedule_step(net: gx.Network, eta, step=None, steps=2, reps=2, margin=
             torch.cuda.synchronize()
             ms = sum(a.elapsed_time(b) for a, b in evs) / steps
             best_ms = ms if best_ms is None else min(best_ms, ms)
-        trials.append(dict(cand, ms_per_step=round(best_ms, 4)))
+        return best_ms
+
+    cands = [dict(bus_staged=b, bat_warps=w) for b in space["bus_staged"] for w in space["bat_warps"]]
+    trials = []
+    for cand in cands:
+        net.set_schedule(**cand)
+        trials.append(dict(cand, ms_per_step=round(timed(), 4)))
         if log:
             log(trials[-1])
     best = pick_schedule(trials, default, margin)
     net.set_schedule(**best)
+    out = dict(best=best, default=default, trials=trials)
+    if auto:
+        net.auto_path()
+        ms = timed()
+        kernels = next(t["ms_per_step"] for t in trials if {k: t[k] for k in SCHEDULE} == best)
+        out["auto"] = dict(ms_per_step=round(ms, 4), kept=kernels >= (1.0 - margin) * ms)
+        if not out["auto"]["kept"]:
+            net.set_schedule(**best)
+        if log:
+            log(out["auto"])
     # one more run captures the chosen schedule's graphs, so the caller's next step is not
     # charged for it; then state and plan go back to the previous plan's
     restore()
     step(eta)
     restore()
     torch.cuda.synchronize()
-    return dict(best=best, default=default, trials=trials)
+    return out
 
 
 def tune(net: gx.Network, nets, steps=3, h_tol=2e-3, g_slack=1.25, cache=None, log=None, alpha_frac=1e-2):
@@ -228,7 +256,7 @@ def tune(net: gx.Network, nets, steps=3, h_tol=2e-3, g_slack=1.25, cache=None, l
     eta_max = torch.tensor(np.concatenate([n["eta_max"] for n in nets]), dtype=torch.float32, device=dev)
     gamma = torch.tensor(np.concatenate([n["gamma"] for n in nets]), dtype=torch.float32, device=dev)
     base = {k: getattr(net.opts, k) for k in SPACE if k != "persistent" and k not in SCHEDULE}
-    base["persistent"] = False
+    base["persistent"] = None if _path_is_auto(net) else False
     base.update(net.schedule())
     g0 = torch.zeros_like(eta_min)
     net.solve(eta_min, warm="cold")

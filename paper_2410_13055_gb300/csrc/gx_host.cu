@@ -2167,6 +2167,13 @@ gx_status gx_network_use_persistent(gx_network* net, int on) {
     return GX_OK;
 }
 
+gx_status gx_network_auto_path(gx_network* net) {
+    if (!net) return fail(GX_ERR_INVALID_ARG, "net is NULL");
+    net->use_crs = -1;
+    net->sched_set = false;
+    return GX_OK;
+}
+
 gx_status gx_network_persistent_info(const gx_network* net, int scen, int* cluster_ctas) {
     if (!net || !cluster_ctas) return fail(GX_ERR_INVALID_ARG, "NULL argument");
     if (scen < 0 || scen >= net->S) return fail(GX_ERR_INVALID_ARG, "scenario out of range");

@@ -93,6 +93,7 @@ _SIGS = {
     "gx_profile_enable": (C.c_int, [_vp, C.c_int]),
     "gx_network_use_graphs": (C.c_int, [_vp, C.c_int]),
     "gx_network_use_persistent": (C.c_int, [_vp, C.c_int]),
+    "gx_network_auto_path": (C.c_int, [_vp]),
     "gx_network_set_schedule": (C.c_int, [_vp, C.POINTER(Schedule)]),
     "gx_network_get_schedule": (C.c_int, [_vp, C.POINTER(Schedule)]),
     "gx_network_persistent_info": (C.c_int, [_vp, C.c_int, C.POINTER(C.c_int)]),
@@ -229,6 +230,7 @@ class Network:
             self.eta_offsets.append(off)
             off += int(n["gen_bus"].size + n["line_from"].size + n["bat_bus"].size)
         self.last_stats = None
+        self._auto_path = True
 
     def __del__(self):
         h = getattr(self, "_h", None)
@@ -337,6 +339,7 @@ class Network:
         if bat_warps is not None:
             sc.bat_warps = int(bat_warps)
         _check(_lib.gx_network_set_schedule(self._h, C.byref(sc)), "gx_network_set_schedule", False)
+        self._auto_path = False
 
     def schedule(self):
         sc = Schedule()
@@ -348,6 +351,18 @@ class Network:
         per-iteration kernels for all of them; until this is called the library decides by
         estimated time (gx_network_use_persistent)."""
         _check(_lib.gx_network_use_persistent(self._h, int(bool(on))), "gx_network_use_persistent", False)
+        self._auto_path = False
+
+    def auto_path(self):
+        """Give the choice of path back to the library after use_persistent or set_schedule, whose
+        schedule stays in force for the per-iteration kernels (gx_network_auto_path)."""
+        _check(_lib.gx_network_auto_path(self._h), "gx_network_auto_path", False)
+        self._auto_path = True
+
+    def path_is_auto(self):
+        """Whether the library chooses the path: neither use_persistent nor set_schedule was called
+        since the network was made or auto_path."""
+        return self._auto_path
 
     def persistent_info(self):
         """Per scenario: CTAs of its resident cluster, 0 if it runs on the per-iteration kernels."""
