@@ -299,10 +299,11 @@ gx_status gx_network_get_schedule(const gx_network* net, gx_schedule* sched);
  * again as scenarios stop, by estimated time: scenarios go to clusters while all that are still
  * iterating fit the device side by side; never after a call of gx_network_set_schedule (until
  * gx_network_auto_path) or in another launch mode than 2, nor while gx_profile_enable is on.  The two
- * paths take bitwise the same iterates for horizons up to 192 hours (longer ones always run on the
- * per-iteration kernels where they have batteries); only the residual partials are summed in another
- * order, so that a scenario may stop at another residual check on the other path.  Equal calls take equal steps: which
- * path and cluster runs an iteration follows from the inputs and the device alone, not from timing. */
+ * paths take bitwise the same iterates (with battery horizons over 96 hours: at bat_warps 2; at 1 up
+ * to rounding); battery horizons over 192 hours, where they agree up to rounding only, take clusters
+ * on request alone.  The residual's partials are summed in another order, so that a scenario may stop
+ * at another residual check on the other path.  Equal calls take equal steps: which path and cluster
+ * runs an iteration follows from the inputs and the device alone, not from timing. */
 gx_status gx_network_use_persistent(gx_network* net, int on);
 /* Give the choice of path back to the library after gx_network_use_persistent or
  * gx_network_set_schedule.  The schedule stays as it was set, for what runs on the per-iteration

@@ -1155,7 +1155,8 @@ CrsFn crs_pick_impl(int kw, int hpl, int reg) {
     }
     if (hpl <= 1) return reg ? k_crs<ADJ, 1, 2, kV, 1> : k_crs<ADJ, 1, 2, kV, 0>;
     if (hpl <= 2) return reg ? k_crs<ADJ, 2, 2, kV, 1> : k_crs<ADJ, 2, 2, kV, 0>;
-    return reg ? k_crs<ADJ, 3, 2, kV, 1> : k_crs<ADJ, 3, 2, kV, 0>;
+    if (hpl <= 3) return reg ? k_crs<ADJ, 3, 2, kV, 1> : k_crs<ADJ, 3, 2, kV, 0>;
+    return k_crs<ADJ, 4, 2, kV, 0>;  // over 192 hours, on request only
 }
 
 }  // namespace

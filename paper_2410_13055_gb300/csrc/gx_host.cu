@@ -578,7 +578,8 @@ static double crs_cost(const ScenDev& sd, const CrsShape& p) {
 // SM's shared memory, the item width and block size of the least estimated time; cluster sizes
 // ascending, those that gain nothing over a smaller one left out.  Empty: the scenario runs on
 // the per-iteration kernels only.  Battery lanes are split as in the battery kernel (two warps
-// where the batch's longest horizon exceeds 96 hours).
+// where the batch's longest horizon exceeds 96 hours); four hours a lane, beyond 192 hours, round
+// otherwise than there and are taken on request only (crs_active).
 static const std::vector<CrsChoice>& crs_choices(gx_network* net, int s) {
     const ScenDev& sd = net->sdev[s];
     const auto key = std::make_pair(sd.net, sd.T);
@@ -599,9 +600,9 @@ static const std::vector<CrsChoice>& crs_choices(gx_network* net, int s) {
                     p.kw = net->ctx.max_bat_T > 96 && sd.T > 32 ? 2 : 1;
                     p.hpl = (sd.T + 32 * p.kw - 1) / (32 * p.kw);
                 }
-                if (p.hpl > 3) continue;
+                if (p.hpl > 4) continue;
                 const int HS = crs_hours(sd.T, C, V), nbo = (sd.B + C - 1) / C;
-                p.reg = p.kw == 2 && nbo * 64 <= threads;
+                p.reg = p.kw == 2 && p.hpl <= 3 && nbo * 64 <= threads;
                 for (int adj = 0; adj < 2; ++adj)
                     for (int sm = p.reg ? 0 : 1; sm >= 0; --sm) {
                         p.bat_smem[adj] = sm;

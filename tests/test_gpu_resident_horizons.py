@@ -1,5 +1,5 @@
 """Which horizons the cluster-resident loops take: any without batteries, up to 192 hours with them
-by the library's choice."""
+by the library's choice and all on request."""
 import numpy as np
 import pytest
 
@@ -32,3 +32,22 @@ def test_long_horizons_without_batteries_take_clusters_bitwise(T, S):
         assert min(h.persistent_info()) > 0
         for k, (x, y) in enumerate(zip(a, b)):
             assert torch.equal(x, y), (persistent, k)
+
+
+@pytest.mark.parametrize("T,B", [(193, 5), (224, 40), (256, 5)])
+def test_battery_horizons_over_192_hours_take_clusters_on_request(T, B):
+    """Up to the rounding of four hours a lane, where the two paths fuse differently: 100 iterations of
+    a few hundred roundings of 2^-24 each, on state of the loads' size."""
+    net, sc = synth.custom(12, 18, 36, B, T, S=1, seed=T)
+    out = []
+    for persistent in (False, True):
+        h = gpu_net([net], sc, kappa=50.0, tol=1e-12, adj_tol=1e-12, max_iter=100, adj_max_iter=100, check_every=20)
+        assert h.persistent_info() == [0]  # not by the library's choice
+        h.use_persistent(persistent)
+        assert (h.persistent_info()[0] > 0) == persistent
+        e = eta_tensor(net["eta_min"] * 1.05)
+        h.solve(e)
+        g = h.grad(e).double().cpu().numpy()
+        out.append([h.state(False).double().cpu().numpy(), g])
+    for x, y in zip(*out):
+        assert np.abs(x - y).max() <= 100 * 300 * 2.0 ** -24 * np.abs(x).max()
