@@ -309,8 +309,11 @@ gx_status gx_network_use_persistent(gx_network* net, int on);
  * gx_network_set_schedule.  The schedule stays as it was set, for what runs on the per-iteration
  * kernels. */
 gx_status gx_network_auto_path(gx_network* net);
-/* *cluster_ctas: CTAs of the cluster scenario `scen` runs on, 0 if it runs on the
- * per-iteration kernels (not resident, not launchable on this device, or switched off). */
+/* *cluster_ctas: CTAs of scenario `scen`'s cluster when every scenario that fits one has its own at
+ * the same time; 0 if it fits none (its state, or this device), or if clusters are switched off or not
+ * the library's choice as above.  Where the library decides, loops over scenarios that do not all fit
+ * side by side start on the per-iteration kernels, and clusters grow as scenarios stop.  Worked out by
+ * gx_network_bind: a call only reads it. */
 gx_status gx_network_persistent_info(const gx_network* net, int scen, int* cluster_ctas);
 
 /* Sampled kernel timing (the network must be bound).  While enabled, the last iteration of

@@ -105,6 +105,7 @@ struct gx_network {
     std::map<std::tuple<int, int, int, int>, bool> crs_ready;  // kernel instances asked for at bind: launchable
     std::vector<const std::vector<CrsChoice>*> crs_of;  // per scenario: its choices
     std::vector<double> crs_dh;                         // per scenario: its device-hours
+    std::vector<int> crs_ctas;                          // per scenario: its cluster beside all others that have one
     std::vector<int> crs_by_room, crs_by_us;  // scenarios that have choices, by their smallest cluster's room / time, descending
     int crs_clusters[kCrsMaxC + 1] = {};  // clusters of C whole-SM CTAs the device holds (set at bind)
     std::vector<int4> crs_bus, crs_line;
@@ -1383,6 +1384,16 @@ gx_status gx_network_bind(gx_network* net, void* dev_mem, size_t bytes, void* st
     build_crs_choices(net);
     std::vector<int> none(net->S);  // marks of the scenarios without a cluster
     for (int s = 0; s < net->S; ++s) none[s] = net->crs_of[s]->empty();
+    {
+        std::vector<const CrsChoice*> pick;
+        bool fits;
+        std::vector<int> fit;
+        for (int s = 0; s < net->S; ++s)
+            if (!none[s]) fit.push_back(s);
+        crs_pick(net, fit, &pick, &fits);
+        net->crs_ctas.assign(net->S, 0);
+        for (size_t i = 0; i < fit.size(); ++i) net->crs_ctas[fit[i]] = pick[i]->shape.C;
+    }
     GX_CUDA(cudaMemcpyAsync(net->dev + net->o_nact + 2 * sizeof(int), none.data(), 4 * (size_t)net->S, cudaMemcpyHostToDevice, st));
     GX_CUDA(cudaStreamSynchronize(st));  // (`none` is local)
     net->solved = false;
@@ -2179,15 +2190,7 @@ gx_status gx_network_persistent_info(const gx_network* net, int scen, int* clust
     if (!net || !cluster_ctas) return fail(GX_ERR_INVALID_ARG, "NULL argument");
     if (scen < 0 || scen >= net->S) return fail(GX_ERR_INVALID_ARG, "scenario out of range");
     *cluster_ctas = 0;
-    if (!net->dev || !crs_active(net)) return GX_OK;
-    std::vector<int> fit;
-    for (int s = 0; s < net->S; ++s)
-        if (!net->crs_of[s]->empty()) fit.push_back(s);
-    std::vector<const CrsChoice*> pick;
-    bool fits;
-    crs_pick(net, fit, &pick, &fits);
-    for (size_t i = 0; i < fit.size(); ++i)
-        if (fit[i] == scen) *cluster_ctas = pick[i]->shape.C;
+    if (net->dev && crs_active(net)) *cluster_ctas = net->crs_ctas[scen];
     return GX_OK;
 }
 

@@ -365,7 +365,8 @@ class Network:
         return self._auto_path
 
     def persistent_info(self):
-        """Per scenario: CTAs of its resident cluster, 0 if it runs on the per-iteration kernels."""
+        """Per scenario: CTAs of its cluster with all that fit one resident at the same time, 0 if it
+        fits none or clusters are off (gx_network_persistent_info)."""
         out = []
         for s in range(self.S):
             v = C.c_int(0)

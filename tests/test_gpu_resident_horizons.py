@@ -51,3 +51,22 @@ def test_battery_horizons_over_192_hours_take_clusters_on_request(T, B):
         out.append([h.state(False).double().cpu().numpy(), g])
     for x, y in zip(*out):
         assert np.abs(x - y).max() <= 100 * 300 * 2.0 ** -24 * np.abs(x).max()
+
+
+def test_cluster_query_only_reads():
+    """From several threads beside a solve: the answer is worked out when the network is bound."""
+    import threading
+
+    import torch
+    net, sc = synth.custom(5, 7, 6, 2, 24, S=512, seed=2)
+    h = gpu_net([net], sc, kappa=50.0, tol=1e-3, adj_tol=1e-3, max_iter=200, adj_max_iter=200)
+    got = []
+    threads = [threading.Thread(target=lambda: got.append(h.persistent_info())) for _ in range(4)]
+    for th in threads:
+        th.start()
+    h.solve(eta_tensor(net["eta_min"]))
+    for th in threads:
+        th.join()
+    torch.cuda.synchronize()
+    want = h.persistent_info()
+    assert min(want) > 0 and got == [want] * 4
