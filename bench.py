@@ -235,6 +235,23 @@ def roofline(config, prof, active, per_scen, n_scen, iters_per_step, ms_per_step
                       "ms_per_step": round(ms_per_step, 3)}}
 
 
+def path_roofline(roof, resident, n_scen, us_per_iteration):
+    """The roofline record where the library chooses the path.  The timing stamps are in the
+    per-iteration kernels, whose pass is not the timed steps' path: with every scenario in a cluster the
+    steps run none of those kernels, so their fraction of the HBM rate is not the steps' and stands
+    under a key of its own."""
+    of = {"us_per_iteration": us_per_iteration, "of": "the timed steps"}
+    if resident < n_scen:
+        return dict(roof, resident=of, timing=(
+            "device-timer stamps inside the per-iteration kernels in a pass of the same steps on those alone; the "
+            f"timed steps' loops start on them and go on in clusters ({resident} of {n_scen} scenarios fit one)"))
+    return {"bound": "latency and shared memory", "kernel": "k_crs", "achieved": None, "peak": roof["peak"],
+            "unit": roof["unit"], "frac": None, "traffic": None, "resident": of,
+            "timing": "the timed steps' loops run in clusters, with no HBM traffic per iteration",
+            "per_iteration_kernels": dict(roof, timing="device-timer stamps in a pass of the same steps on these "
+                                                       "kernels, which the timed steps do not run")}
+
+
 def measure(config, args, steps, warmup, dist=None, learned=False, cold=True, scenarios=None, accuracy=False):
     """Time `steps` previous-plan implicit-gradient steps of one workload (after `warmup`
     steps from a cold start), then a profiled pass of the same steps (kernel times and the
@@ -406,11 +423,8 @@ def measure(config, args, steps, warmup, dist=None, learned=False, cold=True, sc
                             "us_per_iteration": round(1e3 * resident_prof["ms"] / max(iters, 1.0), 3)}
     by_rule = resident > 0 and not args.persistent and args.bus_staged is None
     if by_rule and roof is not None:
-        # (timing stamps take the per-iteration kernels; the headline's loops run in clusters)
-        roof["timing"] = ("device-timer stamps inside the per-iteration kernels in a pass of the same steps; the "
-                          "headline's loops run cluster-resident, without per-iteration HBM traffic")
         its = float(sum(it_prev) + sum(ait_prev))
-        roof["resident"] = {"us_per_iteration": round(1e3 * ms_prev / max(its, 1.0), 3), "of": "the headline's steps"}
+        roof = path_roofline(roof, resident, len(scens), round(1e3 * ms_prev / max(its, 1.0), 3))
     path = ((f"cluster-resident persistent launches for {resident} of {len(scens)} scenarios, "
              "per-iteration kernels (CUDA graphs) for the rest") if args.persistent
             else (f"the library's rule: cluster-resident launches ({resident} of {len(scens)} scenarios fit a "
