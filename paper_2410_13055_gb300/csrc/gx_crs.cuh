@@ -115,6 +115,24 @@ struct FastDiv {
     __device__ __forceinline__ int div(int q) const { return d == 1 ? q : (int)__umulhi((unsigned)q, m); }
 };
 
+// Items 0 to n - 1 over the block's threads, kU of a thread's at a time: ld(q) reads from global
+// memory, st(q, v) stores.  The compiler keeps a load behind a store that might alias it, so a plain
+// copy loop waits for one round trip to L2 per value; here a thread's kU items are in flight together.
+template <int kU, class V, class Ld, class St>
+__device__ __forceinline__ void batched(int n, int tid, int nt, Ld ld, St st) {
+    for (int q0 = tid; q0 < n; q0 += kU * nt) {
+        V v[kU];
+#pragma unroll
+        for (int k = 0; k < kU; ++k) v[k] = ld(min(q0 + k * nt, n - 1));
+#pragma unroll
+        for (int k = 0; k < kU; ++k)
+            if (q0 + k * nt < n) st(q0 + k * nt, v[k]);
+    }
+}
+struct BusIn { float pbar, u, thb, xl, ld; };
+struct LineIn { float dl, vf, vt; int from, to; };
+struct BatIn { float xb; int slot; };
+
 // Operand order of the fused multiply-adds.  The iterates of this path equal those of the
 // per-iteration kernels bit for bit, so every sum of products that the compiler could fuse either
 // way is written out: fma_first fuses a x and rounds b y, fma_second the reverse.
@@ -818,8 +836,14 @@ __global__ void __launch_bounds__(kCrsMaxThreads, 1)
         m.busr[n] = make_int4(r.x * HS, r.y, r.z, (r1.x - r.x) | ((r1.y - r.y) << 12) | (int)((unsigned)(r1.z - r.z) << 24));
         const int nb = sd.bus0 + r.w;
         m.busf[n] = make_float4(c.bus_inv_cnt[nb], c.bus_inv_wsum[nb], c.bus_dres_w[nb], 0.f);
-        for (int g = r.x; g < r1.x; ++g)
-            m.genr[g] = make_int2(n * HS, __float_as_int(c.g_cost[sd.gen0 + R.gen[sd.gen0 + g]]));
+        for (int g = r.x; g < r1.x; g += 4) {
+            float cost[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) cost[k] = c.g_cost[sd.gen0 + R.gen[sd.gen0 + min(g + k, r1.x - 1)]];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (g + k < r1.x) m.genr[g + k] = make_int2(n * HS, __float_as_int(cost[k]));
+        }
     }
     // the entry past the last list is zero, and so are the rows that it leads to
     if (tid == 0) m.endr[2 * L] = make_int4(0, 0, 0, 0);
@@ -860,65 +884,107 @@ __global__ void __launch_bounds__(kCrsMaxThreads, 1)
         m.batg[j] = make_float2(__fmul_rn(fma_first(K.Ah, a, -c.rho, k), K.idet), __fmul_rn(fma_first(c.rho, a, -K.Ah, k), K.idet));
     }
     const int rows = dd_cls ? sd.n_dd : nbo;
-    for (int q = tid; q < rows * T; q += nt) {
-        const int j = q / T, t = q - j * T;
-        const int b = dd_cls ? R.cls_rep[sd.bat0 + j] : rank + j * C;
-        m.idd[q] = b < B ? 1.f / c.bat_dd[sd.e_bat + (long long)b * sd.Tp + t] : 0.f;
-    }
+    batched<4, float>(
+        rows * T, tid, nt,
+        [&](int q) {
+            const int j = q / T, t = q - j * T;
+            const int b = dd_cls ? R.cls_rep[sd.bat0 + j] : rank + j * C;
+            const float dd = c.bat_dd[sd.e_bat + (long long)min(b, B - 1) * sd.Tp + t];
+            return b < B ? 1.f / dd : 0.f;
+        },
+        [&](int q, float v) { m.idd[q] = v; });
 
     // ---- state in
-    for (int q = tid; q < N * HP; q += nt) {
-        const int n = q / HP, hl = q - n * HP;
-        const long long gi = sd.e_bus + (long long)R.bus[sd.bus0 + n].w * sd.Tp + h0 + hl;
-        const int li = n * HS + hl;
-        const bool in = hl < nh;
-        m.pbar[li] = in ? X.pbar[gi] : 0.f; m.u[li] = in ? X.u[gi] : 0.f;
-        m.thb[li] = in ? X.thb[gi] : 0.f; m.xl[li] = in ? X.xl[gi] : 0.f;
-        // adjoint coefficient: NaN where the bound is active, so the hour stays 0
-        m.ld[li] = ADJ ? (in ? c.al[gi] : __int_as_float(0x7fc00000)) : (in ? c.load[gi] : 0.f);
-    }
-    for (int q = tid; q < G * HP; q += nt) {
-        const int k = q / HP, hl = q - k * HP;
-        const int g = R.gen[sd.gen0 + k];
-        const long long gi = sd.e_gen + (long long)g * sd.Tp + h0 + hl;
-        const int li = k * HS + hl;
-        const bool in = hl < nh;
-        m.xg[li] = in ? X.xg[gi] : 0.f;
-        if (ADJ) {
-            m.cap[li] = in ? c.ag[gi] : __int_as_float(0x7fc00000);
-        } else {
-            const float etag = fmaxf(c.eta[sd.eta0 + g], 0.f);
-            m.cap[li] = in ? (c.g_firm[sd.gen0 + g] ? etag : c.cf[gi] * etag) : 0.f;
-        }
-    }
-    for (int q = tid; q < L * HP; q += nt) {
-        const int l = q / HP, hl = q - l * HP;
-        const long long gi = sd.e_line + (long long)l * sd.Tp + h0 + hl;
-        const int4 r = R.line[sd.line0 + l];
-        const bool in = hl < nh;
-        m.dl[l * HS + hl] = in ? X.dl[gi] : 0.f;
-        m.q[r.z * HS + hl] = in ? X.vf[gi] : 0.f;
-        m.q[r.w * HS + hl] = in ? X.vt[gi] : 0.f;
-    }
+    const FastDiv dp(HP > 0 ? HP : 1);
+    batched<2, BusIn>(
+        N * HP, tid, nt,
+        [&](int q) {
+            const int n = dp.div(q), hl = q - n * HP;
+            const bool in = hl < nh;
+            const long long gi = sd.e_bus + (long long)R.bus[sd.bus0 + n].w * sd.Tp + h0 + (in ? hl : 0);
+            BusIn v{X.pbar[gi], X.u[gi], X.thb[gi], X.xl[gi], ADJ ? c.al[gi] : c.load[gi]};
+            // adjoint coefficient: NaN where the bound is active, so the hour stays 0
+            if (!in) v = BusIn{0.f, 0.f, 0.f, 0.f, ADJ ? __int_as_float(0x7fc00000) : 0.f};
+            return v;
+        },
+        [&](int q, const BusIn& v) {
+            const int n = dp.div(q), li = n * HS + q - n * HP;
+            m.pbar[li] = v.pbar; m.u[li] = v.u; m.thb[li] = v.thb; m.xl[li] = v.xl; m.ld[li] = v.ld;
+        });
+    batched<4, float2>(
+        G * HP, tid, nt,
+        [&](int q) {
+            const int k = dp.div(q), hl = q - k * HP;
+            const bool in = hl < nh;
+            const int g = R.gen[sd.gen0 + k];
+            const long long gi = sd.e_gen + (long long)g * sd.Tp + h0 + (in ? hl : 0);
+            float2 v = make_float2(X.xg[gi], ADJ ? c.ag[gi] : c.cf[gi]);
+            if (!ADJ) {
+                const float etag = fmaxf(c.eta[sd.eta0 + g], 0.f);
+                v.y = c.g_firm[sd.gen0 + g] ? etag : v.y * etag;
+            }
+            if (!in) v = make_float2(0.f, ADJ ? __int_as_float(0x7fc00000) : 0.f);
+            return v;
+        },
+        [&](int q, const float2& v) {
+            const int k = dp.div(q), li = k * HS + q - k * HP;
+            m.xg[li] = v.x;
+            m.cap[li] = v.y;
+        });
+    batched<4, LineIn>(
+        L * HP, tid, nt,
+        [&](int q) {
+            const int l = dp.div(q), hl = q - l * HP;
+            const bool in = hl < nh;
+            const long long gi = sd.e_line + (long long)l * sd.Tp + h0 + (in ? hl : 0);
+            const int4 r = R.line[sd.line0 + l];
+            LineIn v{X.dl[gi], X.vf[gi], X.vt[gi], r.z, r.w};
+            if (!in) v.dl = v.vf = v.vt = 0.f;
+            return v;
+        },
+        [&](int q, const LineIn& v) {
+            const int l = dp.div(q), hl = q - l * HP;
+            m.dl[l * HS + hl] = v.dl;
+            m.q[v.from * HS + hl] = v.vf;
+            m.q[v.to * HS + hl] = v.vt;
+        });
     if (ADJ)
-        for (int q = tid; q < L * HQ; q += nt) {
-            const int l = q / HQ, hq = q - l * HQ;
-            unsigned b = 0;
+        batched<4, unsigned>(
+            L * HQ, tid, nt,
+            [&](int q) {
+                const int l = dq.div(q), hq = q - l * HQ;
+                unsigned b = 0;
 #pragma unroll
-            for (int h = 0; h < kV; ++h)
-                if (hq * kV + h < nh) b |= (c.m_line[sd.e_line + (long long)l * sd.Tp + h0 + hq * kV + h] ? 1u : 0u) << h;
-            m.lmask[l * (HS / kV) + hq] = (uint8_t)b;
-        }
-    for (int q = tid; q < B * HP; q += nt) {
-        const int b = q / HP, hl = q - b * HP;
-        m.xb[R.bat[sd.bat0 + b].y * HS + hl] = hl < nh ? X.xb[sd.e_bat + (long long)b * sd.Tp + h0 + hl] : 0.f;
-    }
+                for (int h = 0; h < kV; ++h) {
+                    const int hl = hq * kV + h;
+                    const unsigned on = c.m_line[sd.e_line + (long long)l * sd.Tp + h0 + min(hl, nh - 1)] ? 1u : 0u;
+                    b |= (hl < nh ? on : 0u) << h;
+                }
+                return b;
+            },
+            [&](int q, unsigned b) {
+                const int l = dq.div(q);
+                m.lmask[l * (HS / kV) + q - l * HQ] = (uint8_t)b;
+            });
+    batched<4, BatIn>(
+        B * HP, tid, nt,
+        [&](int q) {
+            const int b = dp.div(q), hl = q - b * HP;
+            const bool in = hl < nh;
+            BatIn v{X.xb[sd.e_bat + (long long)b * sd.Tp + h0 + (in ? hl : 0)], R.bat[sd.bat0 + b].y};
+            if (!in) v.xb = 0.f;
+            return v;
+        },
+        [&](int q, const BatIn& v) { m.xb[v.slot * HS + q - dp.div(q) * HP] = v.xb; });
     if (!kReg && bat_smem)
         for (int q = tid; q < own * T; q += nt) {
             const int j = q / T, t = q - j * T;
             const long long r = sd.e_bat + (long long)(rank + j * C) * sd.Tp + t;
+            float z[6];
 #pragma unroll
-            for (int k = 0; k < 6; ++k) m.bst[(j * 6 + k) * T + t] = X.zc[k * X.zstride + r];
+            for (int k = 0; k < 6; ++k) z[k] = X.zc[k * X.zstride + r];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) m.bst[(j * 6 + k) * T + t] = z[k];
         }
     __syncthreads();
     constexpr int NL = 32 * kW;
@@ -1105,26 +1171,37 @@ __global__ void __launch_bounds__(kCrsMaxThreads, 1)
     if (wait_v) res_wait(c, m, 1, ph & 1);
 
     // ---- state out
-    for (int q = tid; q < N * nh; q += nt) {
-        const int n = q / nh, hl = q - n * nh;
-        const long long gi = sd.e_bus + (long long)R.bus[sd.bus0 + n].w * sd.Tp + h0 + hl;
-        const int li = n * HS + hl;
-        X.pbar[gi] = m.pbar[li]; X.u[gi] = m.u[li]; X.thb[gi] = m.thb[li]; X.xl[gi] = m.xl[li];
-    }
-    for (int q = tid; q < G * nh; q += nt) {
-        const int k = q / nh, hl = q - k * nh;
-        X.xg[sd.e_gen + (long long)R.gen[sd.gen0 + k] * sd.Tp + h0 + hl] = m.xg[k * HS + hl];
-    }
-    for (int q = tid; q < L * nh; q += nt) {
-        const int l = q / nh, hl = q - l * nh;
-        const long long gi = sd.e_line + (long long)l * sd.Tp + h0 + hl;
-        const int4 r = R.line[sd.line0 + l];
-        X.dl[gi] = m.dl[l * HS + hl]; X.vf[gi] = m.q[r.z * HS + hl]; X.vt[gi] = m.q[r.w * HS + hl];
-    }
-    for (int q = tid; q < B * nh; q += nt) {
-        const int b = q / nh, hl = q - b * nh;
-        X.xb[sd.e_bat + (long long)b * sd.Tp + h0 + hl] = m.xb[R.bat[sd.bat0 + b].y * HS + hl];
-    }
+    const FastDiv dn(nh > 0 ? nh : 1);
+    batched<4, int>(
+        N * nh, tid, nt, [&](int q) { return R.bus[sd.bus0 + dn.div(q)].w; },
+        [&](int q, int bus) {
+            const int n = dn.div(q), hl = q - n * nh, li = n * HS + hl;
+            const long long gi = sd.e_bus + (long long)bus * sd.Tp + h0 + hl;
+            X.pbar[gi] = m.pbar[li]; X.u[gi] = m.u[li]; X.thb[gi] = m.thb[li]; X.xl[gi] = m.xl[li];
+        });
+    batched<8, int>(
+        G * nh, tid, nt, [&](int q) { return R.gen[sd.gen0 + dn.div(q)]; },
+        [&](int q, int g) {
+            const int k = dn.div(q), hl = q - k * nh;
+            X.xg[sd.e_gen + (long long)g * sd.Tp + h0 + hl] = m.xg[k * HS + hl];
+        });
+    batched<4, int2>(
+        L * nh, tid, nt,
+        [&](int q) {
+            const int4 r = R.line[sd.line0 + dn.div(q)];
+            return make_int2(r.z, r.w);
+        },
+        [&](int q, const int2& r) {
+            const int l = dn.div(q), hl = q - l * nh;
+            const long long gi = sd.e_line + (long long)l * sd.Tp + h0 + hl;
+            X.dl[gi] = m.dl[l * HS + hl]; X.vf[gi] = m.q[r.x * HS + hl]; X.vt[gi] = m.q[r.y * HS + hl];
+        });
+    batched<4, int>(
+        B * nh, tid, nt, [&](int q) { return R.bat[sd.bat0 + dn.div(q)].y; },
+        [&](int q, int slot) {
+            const int b = dn.div(q), hl = q - b * nh;
+            X.xb[sd.e_bat + (long long)b * sd.Tp + h0 + hl] = m.xb[slot * HS + hl];
+        });
     if (kReg) {
 #pragma unroll
         for (int r = 0; r < 6; ++r)

@@ -19,15 +19,15 @@ namespace gx {
 // device-hours (100 buses, 168 h: 10.9 us for 2 scenarios, 15.4 for 16).
 inline double stream_us(double dh) { return 10.0 + 3.5e-6 * dh; }
 
-// The time between two pauses of resident loops.  A pause costs 25 to 55 us (a launch, the state out
+// The time between two pauses of resident loops.  A pause costs about 43 us (a launch, the state out
 // and in, a look at the done flags), so it comes after at least
 constexpr double kCrsPause = 800.0;
 // microseconds, and a share of the time spent so far, as what is left to gain shrinks against it.
 constexpr double kCrsPauseShare = 0.125;
-// 16 x 168 h of 100 buses, five sets of inputs, plan steps and dispatches from nothing: 72.0 and 77.9 ms;
-// 300 us 73.3 and 81.1, 500 us 72.4 and 79.3, 1,200 us 73.0 and 79.0, a share of 0.2 71.9 and 78.6, no
-// pauses 99.0 and 86.4.  (A pause as soon as few enough were left, which depended on how far each
-// cluster had got: 70.5 and 75.4.)
+// 16 x 168 h of 100 buses, plan steps and dispatches from nothing, eight sets of inputs: 121.8 and
+// 127.5 ms; 600 us 122.1 and 129.6, 500 us with a share of a quarter 121.3 and 130.2; on five of the
+// sets 71.8 and 77.4, without pauses 99.0 and 86.4.  (A pause as soon as few enough were left, which
+// depended on how far each cluster had got: 118.5 and 123.1.)
 
 // Clusters of mixed sizes leave gaps in the processing clusters that hold them.
 inline double crs_room_limit(bool one_list) { return one_list ? 1.0 + 1e-9 : 0.9; }
