@@ -1947,7 +1947,7 @@ static gx_status collect_stats(gx_network* net, int adj, gx_stats* stats, int la
     int err = 0;
     GX_CUDA(cudaMemcpyAsync(&err, net->dev + net->o_err, sizeof(int), cudaMemcpyDeviceToHost, st));
     GX_CUDA(cudaStreamSynchronize(st));
-    if (err) return fail(err, "a bounded device-side wait gave up (bulk copies of the bus kernel)");
+    if (err) return fail(err, "a bounded device-side wait gave up (bulk copies of the bus kernel, or a cluster's exchanges)");
     gx_stats sx{};
     sx.launches = launches;
     gx_status worst = GX_OK;

@@ -60,3 +60,27 @@ def test_empty_lists_take_the_iterates_of_the_iteration_kernels(case):
         for k, (x, y) in enumerate(zip(a, b)):
             assert torch.equal(x, y), (case, persistent, k)
         assert bool(torch.isfinite(b[0]).all())
+
+
+def test_more_equal_scenarios_than_fit_change_path_bitwise():
+    """More scenarios than the device holds side by side: the loop starts on the per-iteration kernels
+    and the stragglers finish in clusters, with the iterates of the kernels alone."""
+    import torch
+    from paper_2410_13055_gb300 import synth
+    nets, scens = synth.medium(S=320, T=24)
+    e = eta_tensor(nets[0]["eta_min"] * 1.05)
+    out, launches = [], []
+    for persistent in (False, None, True):
+        h = gpu_net(nets, scens, kappa=50.0, tol=1e-3, adj_tol=1e-3, max_iter=2000, adj_max_iter=2000, rho=0.2)
+        if persistent is not None:
+            h.use_persistent(persistent)
+        h.solve(e)
+        launches.append(h.last_stats["launches"])
+        r = [h.state(False).clone(), h.array("iters").clone()]
+        g = h.grad(e)
+        out.append(r + [h.state(True).clone(), h.array("adj_iters").clone(), g.clone()])
+        torch.cuda.synchronize()
+    assert launches[2] < launches[1] < launches[0], launches
+    for o in out[1:]:
+        for k, (x, y) in enumerate(zip(out[0], o)):
+            assert torch.equal(x, y), k
