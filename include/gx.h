@@ -306,8 +306,8 @@ gx_status gx_network_get_schedule(const gx_network* net, gx_schedule* sched);
  * runs an iteration follows from the inputs and the device alone, not from timing. */
 gx_status gx_network_use_persistent(gx_network* net, int on);
 /* Give the choice of path back to the library after gx_network_use_persistent or
- * gx_network_set_schedule.  The schedule stays as it was set, for what runs on the per-iteration
- * kernels. */
+ * gx_network_set_schedule.  The schedule stays as it was set (until the next bind, which picks its
+ * own), for what runs on the per-iteration kernels. */
 gx_status gx_network_auto_path(gx_network* net);
 /* *cluster_ctas: CTAs of scenario `scen`'s cluster when every scenario that fits one has its own at
  * the same time; 0 if it fits none (its state, or this device), or if clusters are switched off or not
